@@ -198,8 +198,8 @@ SPLAT_API int64_t splat_view_pixel_offset(const splat_ctx *ctx, int32_t v);
 /* Render every registered view of the primitives g (g->n <= max_gaussians) into the packed
  * buffers depth[P], normal[3][P], alpha[P] (device, caller-owned).  The per-tile lists,
  * transmittances and contributor counts are kept in the context for the next backward call.
- * Stages: per-primitive projection and spherical bounding box (one pass over all views),
- * range sort, tile binning and sort, per-tile front-to-back compositing (one persistent launch
+ * Stages: per-primitive projection and spherical bounding box (one pass over all views), tile
+ * binning, sort of every tile's list by range, per-tile front-to-back compositing (one persistent launch
  * over the tiles of all views).  Errors: INVALID_ARG, STATE (no views), CUDA. */
 SPLAT_API int splat_render_views(splat_ctx *ctx, const splat_gaussians *g, float *depth,
                                  float *normal, float *alpha, void *stream);
@@ -411,9 +411,9 @@ SPLAT_API int splat_get_stats(splat_ctx *ctx, splat_stats *out);
 SPLAT_API int splat_set_profiling(splat_ctx *ctx, int enable);
 SPLAT_API int splat_kernel_times(splat_ctx *ctx, float *fwd_ms, float *bwd_ms);
 /* With profiling enabled: the durations (ms, waiting for the events) of the stages of the last
- * profiled render and refinement step, ms[7] = projection, range sort, emission (count, scan,
- * emit), tile sort, tile ranges and work order, loss, fused Adam; -1 for a stage not recorded
- * since profiling was enabled (the last two come from splat_refine_step only).
+ * profiled render and refinement step, ms[7] = projection, (no stage), emission (count, layout,
+ * emit), list sort, (no stage), loss, fused Adam; -1 for a stage not recorded since profiling was
+ * enabled (the last two come from splat_refine_step only) and for the two places without a stage.
  * Errors: INVALID_ARG, CUDA. */
 SPLAT_API int splat_stage_times(splat_ctx *ctx, float *ms);
 

@@ -52,13 +52,6 @@ bool supported_tile(int th, int tw)
            (th == 4 && tw == 64);
 }
 
-int bits_for(int64_t n)   // bits to hold values 0 .. n-1, rounded up to whole bytes
-{
-    int b = 0;
-    while ((int64_t{1} << b) < n) ++b;
-    return ((b + 7) / 8) * 8;
-}
-
 void split(double x, float &hi, float &lo)
 {
     hi = static_cast<float>(x);
@@ -66,6 +59,8 @@ void split(double x, float &hi, float &lo)
 }
 
 }  // namespace
+
+constexpr int kCountersBin = 8, kCounters = kCountersBin + splat::kBinWords;
 
 struct splat_ctx {
     splat_render_config cfg{};
@@ -80,6 +75,7 @@ struct splat_ctx {
     int n_views = 0;
     std::vector<ViewDesc> views;
     int64_t n_pixels = 0, n_tiles = 0;
+    int max_view_tiles = 0;
     ViewDesc *d_views = nullptr;
     SinCos2 *d_frames = nullptr;
     int32_t *d_tile_view = nullptr;
@@ -89,12 +85,15 @@ struct splat_ctx {
     uint32_t *d_tile_order = nullptr;
 
     // workspace
-    PairRec *d_recs = nullptr;
-    uint32_t *d_dkeys = nullptr, *d_dvals = nullptr, *d_dkeys2 = nullptr, *d_dvals2 = nullptr;
-    uint64_t *d_trect = nullptr, *d_srect = nullptr;   // pair tile rectangles, and in range order
     uint64_t *d_prect = nullptr;   // pair pixel rectangles with the normal-flip bit
-    uint32_t *d_tkeys = nullptr, *d_tvals = nullptr, *d_tkeys2 = nullptr, *d_tvals2 = nullptr;
-    uint32_t *d_block_sums = nullptr, *d_hist = nullptr;
+    // touching pairs by view and block of primitives: tile rectangles, range keys, counts
+    uint64_t *d_touch = nullptr;
+    float *d_kappa = nullptr;
+    uint32_t *d_touch_count = nullptr;
+    uint32_t *d_tile_count = nullptr, *d_cta_count = nullptr;
+    uint64_t *d_entries = nullptr, *d_entries2 = nullptr;   // tile lists (BinArgs)
+    uint8_t *d_blocks = nullptr;
+    splat::ListSegment *d_segments = nullptr;
     uint2 *d_ranges = nullptr;
     float *d_tfinal = nullptr;
     int32_t *d_nlast = nullptr;
@@ -109,14 +108,14 @@ struct splat_ctx {
     uint32_t *d_counters = nullptr;   // [0] pairs M, [1] status, [2] queue f, [3] queue b,
                                       // [4] (view, primitive) pairs that touch a tile,
                                       // [5] record chunks taken, [6] map-growth draws,
-                                      // [7] sampling step
+                                      // [7] sampling step, [8..] binning (splat::kBin...)
     unsigned long long *d_grow_sums = nullptr;  // map growth: block sums, Q, offset
     unsigned long long *d_evals = nullptr;      // [0] forward, [1] backward
 
     // profiling events: [0,1] forward compositing, [2,3] backward compositing, then one event
-    // after each stage of the last profiled render / refinement step (stage_ev[k] ends stage k,
-    // stage_ev[0] is recorded before the projection): projection, range sort, emission, tile
-    // sort, ranges and work order, loss, fused Adam
+    // after the stages of the last profiled render / refinement step: [0] before the
+    // projection, [1] after it, [3] after layout and emission, [4] after the list sort, [6] after
+    // the loss, [7] after the fused Adam
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
     static constexpr int kStageEvents = 8;
     cudaEvent_t stage_ev[kStageEvents] = {};
@@ -134,9 +133,7 @@ struct splat_ctx {
     uint8_t *d_active = nullptr;      // per view: sampled for the current step
     bool want_pose = false;         // backward calls also accumulate the pose gradient
     int64_t last_n = 0;
-    uint32_t *sorted_keys = nullptr, *sorted_vals = nullptr;
-    uint32_t *entry_rect = nullptr;   // per list entry: rectangle inside its tile (K4)
-    uint8_t *entry_blocks = nullptr;  // per list entry: 4 x 8 blocks it meets (K4)
+    bool last_sampled = false;      // the last render drew its views
 };
 
 namespace {
@@ -161,16 +158,14 @@ int check_gaussians(const splat_ctx *ctx, const splat_gaussians *g)
 splat::RenderArgs render_args(splat_ctx *ctx, const splat_gaussians *g)
 {
     splat::RenderArgs a{};
-    a.pos_logit = reinterpret_cast<const float4 *>(g->pos_logit);
     a.prim = ctx->d_prim;
     a.n = g->n;
     a.tiles = ctx->d_tileinfo;
     a.pixframes = ctx->d_pixframes;
     a.ranges = ctx->d_ranges;
     a.tile_order = ctx->d_tile_order;
-    a.sorted_vals = ctx->sorted_vals;
-    a.entry_rect = ctx->entry_rect;
-    a.entry_blocks = ctx->entry_blocks;
+    a.entries = reinterpret_cast<const uint2 *>(ctx->d_entries);
+    a.entry_blocks = ctx->d_blocks;
     a.rec = ctx->d_rec;
     a.rec_prev = ctx->d_rec_prev;
     a.rec_alloc = ctx->d_counters + 5;
@@ -191,18 +186,19 @@ splat::RenderArgs render_args(splat_ctx *ctx, const splat_gaussians *g)
     return a;
 }
 
-// forward pipeline: projection -> range sort -> emission -> tile sort -> ranges -> composite
+// forward pipeline: projection -> list layout -> emission -> list sort -> composite
 int render_core(splat_ctx *ctx, const splat_gaussians *g, float *depth, float *normal,
                 float *alpha, cudaStream_t st)
 {
     const int64_t n = g->n;
-    const int64_t npv = n * ctx->n_views;
     const int th = ctx->cfg.tile_h, tw = ctx->cfg.tile_w;
     uint32_t *cnt = ctx->d_counters;
     CK(cudaMemsetAsync(cnt, 0, sizeof(uint32_t), st));           // pair count
     CK(cudaMemsetAsync(cnt + 4, 0, 2 * sizeof(uint32_t), st));   // touching pairs, chunks
     CK(cudaMemsetAsync(cnt + 2, 0, sizeof(uint32_t), st));       // forward queue
     CK(cudaMemsetAsync(ctx->d_evals, 0, sizeof(unsigned long long), st));
+    CK(cudaMemsetAsync(ctx->d_tile_count, 0,
+                       sizeof(uint32_t) * static_cast<size_t>(ctx->n_tiles), st));
     const uint8_t *active = nullptr;
     if (ctx->samp_draws > 0) {
         CK(splat::launch_sample_views(ctx->n_views, ctx->samp_draws, ctx->d_samp_thr,
@@ -220,43 +216,61 @@ int render_core(splat_ctx *ctx, const splat_gaussians *g, float *depth, float *n
     if (prof)
         for (int k = 0; k < splat_ctx::kStageEvents; ++k) ctx->stage_rec[k] = false;
     CK(stage_mark(0));
-    CK(splat::launch_project(reinterpret_cast<const float4 *>(g->pos_logit),
-                             reinterpret_cast<const float4 *>(g->quat_wxyz),
-                             reinterpret_cast<const float2 *>(g->log_scale), n, ctx->d_views,
-                             ctx->n_views, ctx->cfg.sigma_cut, ctx->cfg.alpha_min, th, tw,
-                             ctx->cfg.flip_normals,
-                             ctx->d_recs, ctx->d_dkeys, ctx->d_dvals, ctx->d_trect,
-                             ctx->d_prect, ctx->d_prim, cnt + 1,
-                             cnt + 4, st,
-                             active));
+    splat::ProjectArgs pa{};
+    pa.pos_logit = reinterpret_cast<const float4 *>(g->pos_logit);
+    pa.quat = reinterpret_cast<const float4 *>(g->quat_wxyz);
+    pa.log_scale = reinterpret_cast<const float2 *>(g->log_scale);
+    pa.n = n;
+    pa.views = ctx->d_views;
+    pa.n_views = ctx->n_views;
+    pa.sigma = ctx->cfg.sigma_cut;
+    pa.alpha_min = ctx->cfg.alpha_min;
+    pa.tile_h = th;
+    pa.tile_w = tw;
+    pa.flip_normals = ctx->cfg.flip_normals;
+    pa.prect = ctx->d_prect;
+    pa.touch = ctx->d_touch;
+    pa.kappa = ctx->d_kappa;
+    pa.touch_count = ctx->d_touch_count;
+    pa.prim = ctx->d_prim;
+    pa.status = cnt + 1;
+    pa.n_valid = cnt + 4;
+    pa.active = active;
+    CK(splat::launch_project(pa, st));
     CK(stage_mark(1));
-    uint32_t *dk, *dv;
-    // the range sort drops the pairs that touch no tile (key 0xFFFFFFFF) in its first pass
-    // (its last pass also lays the pairs' tile rectangles out in range order for the emission)
-    CK(splat::radix_sort_pairs(ctx->d_dkeys, ctx->d_dvals, ctx->d_dkeys2, ctx->d_dvals2, nullptr,
-                               npv, 32, ctx->d_hist, &dk, &dv, st, cnt + 4, ctx->d_trect,
-                               ctx->d_srect));
-    CK(stage_mark(2));
-    CK(splat::launch_emit(dv, ctx->d_srect, npv, cnt + 4, ctx->d_views, n, ctx->d_block_sums,
-                          ctx->d_tkeys, ctx->d_tvals, ctx->cap.max_pairs, cnt, cnt + 1, st));
+    splat::BinArgs ba{};
+    ba.views = ctx->d_views;
+    ba.n_views = ctx->n_views;
+    ba.active = active;
+    ba.max_active = active ? std::min(ctx->samp_draws, ctx->n_views) : ctx->n_views;
+    ba.n = n;
+    ba.tile_h = th;
+    ba.tile_w = tw;
+    ba.n_tiles = ctx->n_tiles;
+    ba.tiles = ctx->d_tileinfo;
+    ba.prect = ctx->d_prect;
+    ba.touch = ctx->d_touch;
+    ba.kappa = ctx->d_kappa;
+    ba.touch_count = ctx->d_touch_count;
+    ba.max_pairs = ctx->cap.max_pairs;
+    ba.max_view_tiles = ctx->max_view_tiles;
+    ba.tile_count = ctx->d_tile_count;
+    ba.cta_count = ctx->d_cta_count;
+    ba.ranges = ctx->d_ranges;
+    ba.order = ctx->d_tile_order;
+    ba.entries = ctx->d_entries;
+    ba.entries2 = ctx->d_entries2;
+    ba.entry_blocks = ctx->d_blocks;
+    ba.segments = ctx->d_segments;
+    ba.d_count = cnt;
+    ba.status = cnt + 1;
+    ba.bin = cnt + kCountersBin;
+    ba.sms = ctx->sms;
+    CK(splat::launch_bin_counts(ba, st));
+    CK(splat::launch_emit(ba, st));
     CK(stage_mark(3));
-    uint32_t *tk, *tv;
-    CK(splat::radix_sort_pairs(ctx->d_tkeys, ctx->d_tvals, ctx->d_tkeys2, ctx->d_tvals2, cnt,
-                               ctx->cap.max_pairs, bits_for(ctx->n_tiles), ctx->d_hist, &tk, &tv,
-                               st));
+    CK(splat::launch_lists(ba, st));
     CK(stage_mark(4));
-    // the tile sort's other buffers are free: they take the entries' tile rectangles and the
-    // blocks each meets
-    uint32_t *rects = tv == ctx->d_tvals ? ctx->d_tvals2 : ctx->d_tvals;
-    uint8_t *blocks = reinterpret_cast<uint8_t *>(tk == ctx->d_tkeys ? ctx->d_tkeys2 : ctx->d_tkeys);
-    CK(splat::launch_ranges(tk, tv, ctx->d_prect, ctx->d_tileinfo, th, tw, cnt,
-                            ctx->cap.max_pairs, ctx->d_ranges, ctx->n_tiles, rects, blocks, st));
-    CK(splat::launch_order_tiles(ctx->d_ranges, ctx->n_tiles, ctx->d_tile_order, st));
-    CK(stage_mark(5));
-    ctx->sorted_keys = tk;
-    ctx->sorted_vals = tv;
-    ctx->entry_rect = rects;
-    ctx->entry_blocks = blocks;
     splat::RenderArgs a = render_args(ctx, g);
     a.depth = depth;
     a.normal = normal;
@@ -269,9 +283,8 @@ int render_core(splat_ctx *ctx, const splat_gaussians *g, float *depth, float *n
         CK(cudaEventRecord(ctx->ev[1], st));
         ctx->rec_fwd = true;
     }
-    // project 1, range sort 4 x 3, emission 3, tile sort 3 per byte, ranges 1, order 1,
-    // composite 1
-    ctx->launches += 1 + 12 + 3 + 3 * (bits_for(ctx->n_tiles) / 8) + 1 + 1 + 1;
+    ctx->launches += 1 + splat::bin_launches(n) + 1;   // projection, binning, compositing
+    ctx->last_sampled = active != nullptr;
     ctx->rendered = true;
     ctx->last_n = n;
     return SPLAT_OK;
@@ -309,9 +322,10 @@ int backward_core(splat_ctx *ctx, const splat_gaussians *g, const float *gD, con
 
 void free_ctx(splat_ctx *c)
 {
-    void *ptrs[] = {c->d_views, c->d_frames, c->d_tile_view, c->d_recs, c->d_dkeys, c->d_dvals,
-                    c->d_dkeys2, c->d_dvals2, c->d_trect, c->d_srect, c->d_prect, c->d_tkeys, c->d_tvals, c->d_tkeys2, c->d_tvals2,
-                    c->d_block_sums, c->d_hist, c->d_ranges, c->d_tfinal, c->d_nlast, c->d_wgrad, c->d_prim,
+    void *ptrs[] = {c->d_views, c->d_frames, c->d_tile_view, c->d_prect, c->d_touch, c->d_kappa,
+                    c->d_touch_count,
+                    c->d_tile_count, c->d_cta_count, c->d_entries, c->d_entries2, c->d_blocks, c->d_segments,
+                    c->d_ranges, c->d_tfinal, c->d_nlast, c->d_wgrad, c->d_prim,
                     c->d_pose, c->d_rec, c->d_rec_prev, c->d_rec_head, c->d_rec_fill,
                     c->d_samp_thr, c->d_active, c->d_grow_sums,
                     c->d_img, c->d_gimg, c->d_counters, c->d_evals, c->d_pixframes,
@@ -395,27 +409,29 @@ SPLAT_API int splat_ctx_create(const splat_render_config *cfg, const splat_capac
     if (e == cudaSuccess) e = dalloc(&c->d_tile_view, TT);
     if (e == cudaSuccess) e = dalloc(&c->d_tileinfo, TT);
     if (e == cudaSuccess) e = dalloc(&c->d_tile_order, TT);
-    if (e == cudaSuccess) e = dalloc(&c->d_recs, mpv);
-    if (e == cudaSuccess) e = dalloc(&c->d_dkeys, mpv);
-    if (e == cudaSuccess) e = dalloc(&c->d_dvals, mpv);
-    if (e == cudaSuccess) e = dalloc(&c->d_dkeys2, mpv);
-    if (e == cudaSuccess) e = dalloc(&c->d_dvals2, mpv);
-    if (e == cudaSuccess) e = dalloc(&c->d_trect, mpv);
-    if (e == cudaSuccess) e = dalloc(&c->d_srect, mpv);
     if (e == cudaSuccess) e = dalloc(&c->d_prect, mpv);
-    // the tile-sort buffers also hold the sorted lists the forward reads four entries at a
-    // time from a 4-aligned index: 128 spare entries keep the last vector in bounds
-    if (e == cudaSuccess) e = dalloc(&c->d_tkeys, M + 128);
-    if (e == cudaSuccess) e = dalloc(&c->d_tvals, M + 128);
-    if (e == cudaSuccess) e = dalloc(&c->d_tkeys2, M + 128);
-    if (e == cudaSuccess) e = dalloc(&c->d_tvals2, M + 128);
-    if (e == cudaSuccess) e = dalloc(&c->d_block_sums, splat::kScanGrid);
-    if (e == cudaSuccess) e = dalloc(&c->d_hist, static_cast<size_t>(splat::kHistWords));
+    if (e == cudaSuccess) e = dalloc(&c->d_touch, mpv);
+    if (e == cudaSuccess) e = dalloc(&c->d_kappa, mpv);
+    if (e == cudaSuccess)
+        e = dalloc(&c->d_touch_count,
+                   static_cast<size_t>(splat::max_project_blocks(cap->max_gaussians)) * cap->max_views);
+    if (e == cudaSuccess) e = dalloc(&c->d_tile_count, TT);
+    if (e == cudaSuccess)
+        e = dalloc(&c->d_cta_count, splat::cta_count_words(c->sms, cap->max_views, TT));
+    // the forward reads the lists four entries at a time from a 4-aligned index: 128 spare
+    // entries keep the last vector in bounds
+    if (e == cudaSuccess) e = dalloc(&c->d_entries, M + 128);
+    if (e == cudaSuccess) e = dalloc(&c->d_blocks, M + 128);
+    // a list holds each primitive once: only larger maps can have lists to cut into segments
+    if (cap->max_gaussians >= splat::kListCap) {
+        if (e == cudaSuccess) e = dalloc(&c->d_entries2, M);
+        if (e == cudaSuccess) e = dalloc(&c->d_segments, splat::max_segments(M));
+    }
     if (e == cudaSuccess) e = dalloc(&c->d_ranges, TT);
     if (e == cudaSuccess) e = dalloc(&c->d_tfinal, P);
     if (e == cudaSuccess) e = dalloc(&c->d_nlast, P);
     if (e == cudaSuccess) e = dalloc(&c->d_wgrad, static_cast<size_t>(cap->max_gaussians) * 4);
-    if (e == cudaSuccess) e = dalloc(&c->d_prim, static_cast<size_t>(cap->max_gaussians) * 3);
+    if (e == cudaSuccess) e = dalloc(&c->d_prim, static_cast<size_t>(cap->max_gaussians) * splat::kPrimRow);
     if (e == cudaSuccess) e = dalloc(&c->d_pose, static_cast<size_t>(cap->max_views) * 6);
     if (e == cudaSuccess) e = dalloc(&c->d_samp_thr, static_cast<size_t>(splat::kMaxViews));
     if (e == cudaSuccess) e = dalloc(&c->d_active, static_cast<size_t>(cap->max_views));
@@ -431,13 +447,14 @@ SPLAT_API int splat_ctx_create(const splat_render_config *cfg, const splat_capac
     if (e == cudaSuccess) e = dalloc(&c->d_rec_fill, static_cast<size_t>(items));
     if (e == cudaSuccess) e = dalloc(&c->d_img, static_cast<size_t>(P) * 5);
     if (e == cudaSuccess) e = dalloc(&c->d_gimg, static_cast<size_t>(P) * 5);
-    if (e == cudaSuccess) e = dalloc(&c->d_counters, 8);
+    if (e == cudaSuccess) e = dalloc(&c->d_counters, kCounters);
     if (e == cudaSuccess) e = dalloc(&c->d_evals, 2);
     for (int k = 0; k < 4 && e == cudaSuccess; ++k) e = cudaEventCreate(&c->ev[k]);
     for (int k = 0; k < splat_ctx::kStageEvents && e == cudaSuccess; ++k)
         e = cudaEventCreate(&c->stage_ev[k]);
-    if (e == cudaSuccess) e = cudaMemset(c->d_counters, 0, 8 * sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMemset(c->d_counters, 0, kCounters * sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMemset(c->d_evals, 0, 2 * sizeof(unsigned long long));
+    if (e == cudaSuccess) e = splat::prepare_lists();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         int r = cuda_fail(e, "splat_ctx_create");
@@ -624,6 +641,9 @@ SPLAT_API int splat_set_views(splat_ctx *ctx, int32_t n_views, const double *T_w
     ctx->n_views = n_views;
     ctx->n_pixels = pix;
     ctx->n_tiles = tiles;
+    ctx->max_view_tiles = 0;
+    for (const ViewDesc &v : views)
+        ctx->max_view_tiles = std::max(ctx->max_view_tiles, v.tiles_r * v.tiles_c);
     ctx->rendered = false;
     ctx->have_pose = false;
     ctx->samp_draws = 0;   // the sampling law depends on the views: set it again
@@ -1030,18 +1050,20 @@ SPLAT_API int splat_kernel_times(splat_ctx *ctx, float *fwd_ms, float *bwd_ms)
 SPLAT_API int splat_stage_times(splat_ctx *ctx, float *ms)
 {
     if (!ctx || !ms) return SPLAT_ERR_INVALID_ARG;
-    // stage k of the render runs between stage events k and k + 1; the loss between the end of
-    // the forward compositing and event 6, the fused Adam between the end of the backward and 7
+    // the loss runs between the end of the forward compositing and event 6, the fused Adam
+    // between the end of the backward and event 7; binning has no global range sort and no
+    // separate ranges pass
     struct Span {
         cudaEvent_t a, b;
         bool ok;
     };
+    const Span none{nullptr, nullptr, false};
     const Span spans[7] = {
         {ctx->stage_ev[0], ctx->stage_ev[1], ctx->stage_rec[0] && ctx->stage_rec[1]},
-        {ctx->stage_ev[1], ctx->stage_ev[2], ctx->stage_rec[1] && ctx->stage_rec[2]},
-        {ctx->stage_ev[2], ctx->stage_ev[3], ctx->stage_rec[2] && ctx->stage_rec[3]},
+        none,
+        {ctx->stage_ev[1], ctx->stage_ev[3], ctx->stage_rec[1] && ctx->stage_rec[3]},
         {ctx->stage_ev[3], ctx->stage_ev[4], ctx->stage_rec[3] && ctx->stage_rec[4]},
-        {ctx->stage_ev[4], ctx->stage_ev[5], ctx->stage_rec[4] && ctx->stage_rec[5]},
+        none,
         {ctx->ev[1], ctx->stage_ev[6], ctx->rec_fwd && ctx->stage_rec[6]},
         {ctx->ev[3], ctx->stage_ev[7], ctx->rec_bwd && ctx->stage_rec[7]},
     };
@@ -1056,26 +1078,62 @@ SPLAT_API int splat_stage_times(splat_ctx *ctx, float *ms)
 
 SPLAT_API int64_t splat_debug_copy(splat_ctx *ctx, int32_t which, void *dst, int64_t bytes)
 {
-    if (!ctx || !dst || bytes < 0) return -1;
+    if (!ctx || !dst || bytes < 0 || which < 0 || which > 5) return -1;
     if (cudaDeviceSynchronize() != cudaSuccess) return -1;
+    if (!ctx->rendered) return -1;
     uint32_t m = 0;
     if (cudaMemcpy(&m, ctx->d_counters, sizeof m, cudaMemcpyDeviceToHost) != cudaSuccess) return -1;
-    const void *src = nullptr;
-    int64_t need = 0;
-    switch (which) {
-    case 0: src = ctx->sorted_keys; need = int64_t{4} * m; break;
-    case 1: src = ctx->sorted_vals; need = int64_t{4} * m; break;
-    case 2: src = ctx->d_ranges; need = int64_t{8} * ctx->n_tiles; break;
-    case 3: src = ctx->d_recs; need = int64_t{16} * ctx->last_n * ctx->n_views; break;
-    case 4: src = ctx->d_tfinal; need = int64_t{4} * ctx->n_pixels; break;
-    case 5: src = ctx->d_nlast; need = int64_t{4} * ctx->n_pixels; break;
-    default: return -1;
-    }
-    if (!ctx->rendered || !src) return -1;
-    if (need > bytes) return -1;
-    if (need > 0 && cudaMemcpy(dst, src, static_cast<size_t>(need), cudaMemcpyDeviceToHost) != cudaSuccess)
+    auto get = [&](const void *src, int64_t need) -> int64_t {
+        if (need > bytes) return -1;
+        if (need > 0 && cudaMemcpy(dst, src, static_cast<size_t>(need), cudaMemcpyDeviceToHost) !=
+                            cudaSuccess)
+            return -1;
+        return need;
+    };
+    const int64_t npv = ctx->last_n * ctx->n_views;
+    try {
+        switch (which) {
+        case 0: {   // the tile of every entry, from the ranges
+            if (int64_t{4} * m > bytes) return -1;
+            std::vector<uint2> rg(static_cast<size_t>(ctx->n_tiles));
+            if (cudaMemcpy(rg.data(), ctx->d_ranges, sizeof(uint2) * rg.size(),
+                           cudaMemcpyDeviceToHost) != cudaSuccess)
+                return -1;
+            uint32_t *out = static_cast<uint32_t *>(dst);
+            for (size_t t = 0; t < rg.size(); ++t)
+                for (uint32_t j = rg[t].x; j < rg[t].y; ++j) out[j] = static_cast<uint32_t>(t);
+            return int64_t{4} * m;
+        }
+        case 1: {   // the pair ids of the (pair id, rectangle) entries
+            if (int64_t{4} * m > bytes) return -1;
+            if (m == 0) return 0;
+            if (cudaMemcpy2D(dst, 4, ctx->d_entries, 8, 4, m, cudaMemcpyDeviceToHost) !=
+                cudaSuccess)
+                return -1;
+            return int64_t{4} * m;
+        }
+        case 2: return get(ctx->d_ranges, int64_t{8} * ctx->n_tiles);
+        case 3: {
+            const int64_t need = static_cast<int64_t>(sizeof(PairRec)) * npv;
+            if (need > bytes) return -1;
+            if (need == 0) return 0;
+            PairRec *recs = nullptr;   // not a compute call: a temporary buffer is fine here
+            if (dalloc(&recs, static_cast<size_t>(npv)) != cudaSuccess) return -1;
+            cudaError_t e = splat::launch_records(
+                ctx->last_n, ctx->n_views, ctx->d_views, ctx->cfg.flip_normals, ctx->cfg.tile_h,
+                ctx->cfg.tile_w, ctx->d_prim, ctx->d_prect,
+                ctx->last_sampled ? ctx->d_active : nullptr, recs, nullptr);
+            if (e == cudaSuccess)
+                e = cudaMemcpy(dst, recs, static_cast<size_t>(need), cudaMemcpyDeviceToHost);
+            cudaFree(recs);
+            return e == cudaSuccess ? need : -1;
+        }
+        case 4: return get(ctx->d_tfinal, int64_t{4} * ctx->n_pixels);
+        default: return get(ctx->d_nlast, int64_t{4} * ctx->n_pixels);
+        }
+    } catch (...) {
         return -1;
-    return need;
+    }
 }
 
 }  // extern "C"

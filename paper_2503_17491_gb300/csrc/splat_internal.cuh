@@ -171,7 +171,7 @@ enum : uint32_t { kCountMask = 0x3FFFFFFFu, kPairFlip = 1u << 30, kPairInvalid =
 // ---------------------------------------------------------------------------------------------
 
 // A pair's pixel rectangle and normal-flip bit in one word: r0 | flip << 15, r1, c0, nc, 16 bits
-// each (rows and columns are below 2^15)
+// each (rows and columns are below 2^15); 0 for a pair that touches no tile (nc >= 1 otherwise)
 __host__ __device__ inline uint64_t pack_pixel_rect(const PairRec &rec)
 {
     const uint32_t r0 = static_cast<uint16_t>(rec.r0) | ((rec.cf & kPairFlip) ? 0x8000u : 0u);
@@ -192,15 +192,69 @@ __host__ __device__ inline PairRec unpack_pixel_rect(uint64_t w)
     return rec;
 }
 
-// A pair's tile rectangle in one word: first tile row, tile rows, first tile column, tile columns
-// (cyclic modulo the view's tile columns), 16 bits each; every field is below 2^13 for images
-// of at most 32,767 rows and columns and tiles of at least 4 pixels a side.
-__host__ __device__ inline uint64_t pack_tile_rect(int tr0, int ntr, int tc0, int ntc)
+// A pair's tile rectangle: first tile row and column, rows and columns, the columns cyclic modulo
+// the view's tile columns.
+struct TileRect {
+    int r0, nr, c0, nc;
+};
+
+// Blocks of primitives: the projection's CTAs, and the segments of its touching pairs.  Larger
+// maps take blocks of 1,024, so that the pairs a CTA has to box exactly fill more warps; smaller
+// ones of 256, so that there are CTAs for every SM.
+constexpr int kSmallBlock = 256, kLargeBlock = 1024;
+inline int block_prims(int64_t n) { return n < int64_t{1} << 18 ? kSmallBlock : kLargeBlock; }
+inline int64_t project_blocks(int64_t n)
 {
-    return static_cast<uint64_t>(static_cast<uint16_t>(tr0)) |
-           static_cast<uint64_t>(static_cast<uint16_t>(ntr)) << 16 |
-           static_cast<uint64_t>(static_cast<uint16_t>(tc0)) << 32 |
-           static_cast<uint64_t>(static_cast<uint16_t>(ntc)) << 48;
+    return (n + block_prims(n) - 1) / block_prims(n);
+}
+// the most blocks of any map of up to n primitives
+inline int64_t max_project_blocks(int64_t n)
+{
+    const int64_t small = n < int64_t{1} << 18 ? n : int64_t{1} << 18;
+    const int64_t a = small / kSmallBlock + 1, b = n / kLargeBlock + 1;
+    return a > b ? a : b;
+}
+
+// A touching pair in its block's segment: its tile rectangle and its primitive's place in the
+// block, 64 bits.  Images have at most 32,767 rows and columns and tiles at least 4 rows and 8
+// columns: at most 8,192 tile rows and 4,096 tile columns.
+__device__ __forceinline__ uint64_t pack_touch(const TileRect &t, uint32_t local)
+{
+    return static_cast<uint64_t>(t.r0) | static_cast<uint64_t>(t.nr) << 13 |
+           static_cast<uint64_t>(t.c0) << 27 | static_cast<uint64_t>(t.nc) << 39 |
+           static_cast<uint64_t>(local) << 52;
+}
+
+__device__ __forceinline__ TileRect unpack_touch(uint64_t w, uint32_t &local)
+{
+    local = static_cast<uint32_t>(w >> 52);
+    return TileRect{static_cast<int>(w & 0x1FFFu), static_cast<int>(w >> 13 & 0x3FFFu),
+                    static_cast<int>(w >> 27 & 0xFFFu), static_cast<int>(w >> 39 & 0x1FFFu)};
+}
+
+// the tiles a record's pixel rectangle meets: columns c0 .. c0 + nc - 1 (mod W), wrapping past
+// the last tile; tile sides are powers of two and every index here is non-negative, so shifts
+// divide
+__device__ __forceinline__ TileRect tile_rect(const PairRec &rec, int W, int tiles_c, int th_shift,
+                                              int tw_shift)
+{
+    TileRect t;
+    t.r0 = rec.r0 >> th_shift;
+    t.nr = (rec.r1 >> th_shift) - t.r0 + 1;
+    if (rec.nc >= W) {
+        t.c0 = 0;
+        t.nc = tiles_c;
+    } else {
+        const int cl = rec.c0 + rec.nc - 1;
+        const int b = cl < W ? cl >> tw_shift : tiles_c + ((cl - W) >> tw_shift);
+        t.c0 = rec.c0 >> tw_shift;
+        t.nc = b - t.c0 + 1;
+        if (t.nc >= tiles_c) {
+            t.c0 = 0;
+            t.nc = tiles_c;
+        }
+    }
+    return t;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -317,92 +371,118 @@ __device__ __forceinline__ void chain_params(const float4 pl, const float4 q, co
 // ---------------------------------------------------------------------------------------------
 struct Workspace;   // host-side bookkeeping, defined in splat_abi.cu
 
-// trect[p]: the pair's tile rectangle as one word (see pack_tile_rect), 0 when it touches none;
-// prect[p]: its pixel rectangle and normal-flip bit (pack_pixel_rect)
 // Record the text of a failed CUDA call for splat_last_cuda_error (thread-local) and return
 // SPLAT_ERR_CUDA.
 int cuda_fail(cudaError_t e, const char *what);
 
-cudaError_t launch_project(const float4 *pos_logit, const float4 *quat, const float2 *log_scale,
-                           int64_t n, const ViewDesc *views, int n_views, float sigma,
-                           float alpha_min, int tile_h, int tile_w, int flip_normals,
-                           PairRec *recs, uint32_t *dkeys, uint32_t *dvals, uint64_t *trect,
-                           uint64_t *prect, float4 *prim, uint32_t *status, uint32_t *n_valid,
-                           cudaStream_t st, const uint8_t *active = nullptr);
+// What the compositing kernels stage of a primitive, kPrimRow float4 written by the projection:
+// (s_a t_a, o), (s_b t_b, 1 or 0 for an invalid primitive), (t_n, 0), (mu, 0), in the world frame
+constexpr int kPrimRow = 4;
 
-// stable LSD radix sort of (uint32 key, uint32 value) pairs on key bits [0, bits);
-// the count is read on the device from *d_count (clamped to max_n); result lands in
-// (keys_out, vals_out).  tmp_hist holds kHistWords uint32.
-constexpr int kSortGrid = 608;    // 4 CTAs per SM (152 SMs)
-constexpr int kSortTile = 2048;   // keys per CTA tile (256 threads x 8)
-constexpr int kHistWords = kSortGrid * 256 + 256;   // per-CTA digit counts + digit totals
-// With d_count_kept non-null the first pass also drops every item whose key is 0xFFFFFFFF (which
-// would sort last) and the later passes sort the d_count_kept items left, which the caller has
-// counted beforehand.
-// With aux_out non-null the last pass also writes aux_out[i] = aux_in[value of sorted item i]:
-// a copy of per-value data in sorted order, so that the stages after the sort read it in order.
-cudaError_t radix_sort_pairs(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint32_t *vals_alt,
-                             const uint32_t *d_count, int64_t max_n, int bits, uint32_t *tmp_hist,
-                             uint32_t **keys_out, uint32_t **vals_out, cudaStream_t st,
-                             const uint32_t *d_count_kept = nullptr,
-                             const uint64_t *aux_in = nullptr, uint64_t *aux_out = nullptr);
+struct ProjectArgs {
+    const float4 *pos_logit, *quat;
+    const float2 *log_scale;
+    int64_t n;
+    const ViewDesc *views;
+    int n_views;
+    float sigma, alpha_min;
+    int tile_h, tile_w, flip_normals;
+    uint64_t *prect;        // per pair: pack_pixel_rect, 0 when it touches no tile
+    int block_prims;        // set by the launcher
+    // per (view, block): its touching pairs from place view * n + block's first primitive on,
+    // their range keys, and how many there are (view * project_blocks(n) + block)
+    uint64_t *touch;
+    float *kappa;
+    uint32_t *touch_count;
+    float4 *prim;
+    uint32_t *status;
+    uint32_t *n_valid;      // zeroed before: pairs that touch a tile
+    const uint8_t *active;  // per view (nullable): drawn for this step
+};
+cudaError_t launch_project(const ProjectArgs &a, cudaStream_t st);
+cudaError_t launch_records(int64_t n, int n_views, const ViewDesc *views, int flip_normals,
+                           int tile_h, int tile_w, const float4 *prim, const uint64_t *prect,
+                           const uint8_t *active, PairRec *recs, cudaStream_t st);
 
-// offsets of every sorted pair, emission of (global tile, pair id) entries, total pair count
-// emission grid: CTAs over the sorted pairs (measured on GB300: 1024 -> 4096 CTAs took the
-// three emission kernels from 0.142 to 0.131 ms on 4 M pairs); the CTA-sum scan runs in one CTA
-// of 1024 threads, kScanGrid / 1024 sums per thread
-constexpr int kScanGrid = 4096;
-// tile-ranges grid (grid-stride over the list entries): 6 CTAs per SM measured fastest
-// (0.089 ms on 6.1 M entries, against 0.113 ms with 16 per SM)
-constexpr int kRangesGrid = 912;
-// n_valid: device count of the leading sorted pairs that touch a tile (the rest touch none)
-// sorted_trect[j]: the tile rectangle of sorted pair j (the range sort's copy of trect)
-cudaError_t launch_emit(const uint32_t *sorted_pair_ids, const uint64_t *sorted_trect,
-                        int64_t n_pairs_total, const uint32_t *n_valid, const ViewDesc *views,
-                        int64_t n_per_view, uint32_t *block_sums, uint32_t *tile_keys,
-                        uint32_t *tile_vals, int64_t max_pairs, uint32_t *d_count,
-                        uint32_t *status, cudaStream_t st);
+// Binning (splat_sort.cu): from the projection's pixel rectangles to the per-tile lists in (range, id)
+// order, [start, end) per tile and the work order.  A list of more than kListCap entries is cut
+// into segments of at most kListCap before it is sorted.
+constexpr int kListCap = 4096;
+constexpr int kSegTarget = kListCap / 2;
+struct ListSegment {
+    uint32_t start, len, tile;
+};
+inline int64_t max_segments(int64_t max_pairs)   // ceil(len / target) of lists above the cap
+{
+    return max_pairs / kSegTarget + max_pairs / kListCap + 2;
+}
+struct BinArgs {
+    const ViewDesc *views;
+    int n_views;
+    const uint8_t *active;      // nullable: views drawn for this step, at most max_active
+    int max_active;
+    int64_t n;                  // primitives per view
+    int tile_h, tile_w;
+    int64_t n_tiles;
+    const TileInfo *tiles;
+    const uint64_t *prect, *touch;
+    const float *kappa;
+    const uint32_t *touch_count;
+    int64_t max_pairs;
+    int max_view_tiles;         // most tiles of one view
+    uint32_t *tile_count;       // zeroed before; counted, then counted down by the emission
+    uint32_t *cta_count;        // cta_count_words(...): the counts of every counting CTA
+    uint2 *ranges;
+    uint32_t *order;            // tiles by decreasing log2 of their list length
+    uint64_t *entries;          // emitted (range key << 32 | pair id), then the sorted entries
+    uint64_t *entries2;         // scratch of the same size (needed when n > kListCap)
+    uint8_t *entry_blocks;
+    ListSegment *segments;      // max_segments(max_pairs)
+    uint32_t *d_count;          // out: list entries
+    uint32_t *status;
+    uint32_t *bin;              // kBinWords counters (written by the layout kernel)
+    int sms;
+    int block_prims, blocks;    // the projection's blocks; these and chunk (blocks a counting CTA
+    int chunk;                  // takes) are set by the launchers
+};
+// kBinLong, kBinMid: tiles (in work order) with at least kListCap and at least 256 entries
+constexpr int kBinCtas = 4;              // counting and emitting CTAs per SM
+constexpr int kMinChunk = kLargeBlock;   // primitives each takes at least
+constexpr int kMaxSharedTiles = 12288;   // views up to this are counted in shared memory (48 KB)
+inline int64_t cta_count_words(int sms, int max_views, int64_t max_tiles)
+{
+    return (int64_t{kBinCtas} * sms + max_views) *
+           (max_tiles < kMaxSharedTiles ? max_tiles : kMaxSharedTiles);
+}
+enum { kBinLong = 0, kBinMid, kBinSegments, kBinQueueSeg, kBinWords };
+cudaError_t prepare_lists();    // before the first launch_lists on a device
+int bin_launches(int64_t n);    // kernels these three run for n primitives
+cudaError_t launch_bin_counts(const BinArgs &a, cudaStream_t st);   // count and layout
+cudaError_t launch_emit(const BinArgs &a, cudaStream_t st);
+cudaError_t launch_lists(const BinArgs &a, cudaStream_t st);
 
-// Pixel rectangle of a (view, primitive) record inside tile (tr, tc) of a tile_h x tile_w
-// tiling, packed as 4 bytes (r_lo, r_hi, c_lo, c_hi) with the record's normal-flip bit in bit 31;
-// the record's columns are cyclic modulo the image width cols.  0xFF (r_lo > r_hi) when empty.
+// Pixel rectangle of a (view, primitive) record inside the tile_h x tile_w tile with first row rb
+// and column cb, packed as 4 bytes (r_lo, r_hi, c_lo, c_hi) with the record's normal-flip bit in
+// bit 31; the record's columns are cyclic modulo the image width W.  0xFF (r_lo > r_hi) when empty.
 constexpr uint32_t kRectFlip = 0x80000000u;
 
-__device__ __forceinline__ uint32_t tile_local_rect(const PairRec &rec, int tr, int tc, int cols,
+__device__ __forceinline__ uint32_t tile_local_rect(const PairRec &rec, int rb, int cb, int W,
                                                     int tile_h, int tile_w)
 {
-    const int rb = tr * tile_h, cb = tc * tile_w;
-    int r_lo = rec.r0 - rb, r_hi = rec.r1 - rb;
-    r_lo = r_lo < 0 ? 0 : r_lo;
-    r_hi = r_hi > tile_h - 1 ? tile_h - 1 : r_hi;
-    if (r_lo > r_hi) return 0xFFu;
-    const int W = cols, nc = rec.nc;
+    const int r_lo = max(rec.r0 - rb, 0), r_hi = min(rec.r1 - rb, tile_h - 1);
+    const int nc = rec.nc;
     int c_lo, c_hi;
-    if (nc >= W) {
-        c_lo = 0;
-        c_hi = tile_w - 1;
+    if (rec.c0 + nc <= W) {   // the columns do not wrap
+        c_lo = max(rec.c0 - cb, 0);
+        c_hi = min(rec.c0 + nc - 1 - cb, tile_w - 1);
     } else {
-        int d = cb - rec.c0;     // tile start relative to the range start, in [0, W)
-        d += d < 0 ? W : 0;
-        int e = rec.c0 - cb;     // range start relative to the tile start, in [0, W)
-        e += e < 0 ? W : 0;
-        const bool start_in = d < nc;
-        const bool begins_here = e < tile_w;
-        if (start_in && begins_here && d != 0) {   // both ends of a wrapping range meet here
-            c_lo = 0;
-            c_hi = tile_w - 1;
-        } else if (start_in) {
-            c_lo = 0;
-            c_hi = nc - 1 - d;
-            c_hi = c_hi > tile_w - 1 ? tile_w - 1 : c_hi;
-        } else if (begins_here) {
-            c_lo = e;
-            c_hi = e + nc - 1;
-            c_hi = c_hi > tile_w - 1 ? tile_w - 1 : c_hi;
-        } else {
-            return 0xFFu;
-        }
+        // c0 .. W - 1 and 0 .. last; a tile that both ends meet is taken whole
+        const int last = rec.c0 + nc - 1 - W;
+        const bool head = rec.c0 < cb + tile_w, tail = cb <= last;
+        c_lo = tail ? 0 : max(rec.c0 - cb, 0);
+        c_hi = head ? tile_w - 1 : (tail ? min(last - cb, tile_w - 1) : -1);
     }
+    if (r_lo > r_hi || c_lo > c_hi) return 0xFFu;
     return static_cast<uint32_t>(r_lo) | (static_cast<uint32_t>(r_hi) << 8) |
            (static_cast<uint32_t>(c_lo) << 16) | (static_cast<uint32_t>(c_hi) << 24) |
            ((rec.cf & kPairFlip) ? kRectFlip : 0u);
@@ -415,38 +495,26 @@ __device__ __forceinline__ uint32_t rect_blocks(uint32_t rect, int tile_h, int t
     const int r_lo = rect & 0xFF, r_hi = (rect >> 8) & 0xFF;
     const int c_lo = (rect >> 16) & 0x3F, c_hi = (rect >> 24) & 0x3F;
     if (r_lo > r_hi || r_hi >= tile_h) return 0u;
-    const int wc = tile_w / 8;
     const uint32_t cols = ((2u << (c_hi >> 3)) - 1u) & ~((1u << (c_lo >> 3)) - 1u);
-    uint32_t m = 0u;
-    for (int rb = r_lo >> 2; rb <= r_hi >> 2; ++rb) m |= cols << (rb * wc);
-    return m;
+    const uint32_t rows = ((2u << (r_hi >> 2)) - 1u) & ~((1u << (r_lo >> 2)) - 1u);
+    // the row bits spread tile_w / 8 apart, each times the column bits
+    if (tile_w == 8) return rows;
+    if (tile_w == 16)
+        return cols * ((rows & 1u) | (rows & 2u) << 1 | (rows & 4u) << 2 | (rows & 8u) << 3);
+    if (tile_w == 32) return cols * ((rows & 1u) | (rows & 2u) << 3);
+    return cols;
 }
 
-// K4: [start, end) per tile from the sorted tile ids, and every list entry's pixel rectangle
-// inside its tile (tile_local_rect) in entry_rect and the 4 x 8 blocks it meets (rect_blocks) in
-// entry_blocks
-cudaError_t launch_ranges(const uint32_t *tile_keys, const uint32_t *tile_vals,
-                          const uint64_t *prect, const TileInfo *tiles, int tile_h, int tile_w,
-                          const uint32_t *d_count, int64_t max_pairs, uint2 *ranges,
-                          int64_t n_tiles, uint32_t *entry_rect, uint8_t *entry_blocks,
-                          cudaStream_t st);
-
-// tiles ordered by decreasing log2 of their list length (order inside a bucket unspecified)
-cudaError_t launch_order_tiles(const uint2 *ranges, int64_t n_tiles, uint32_t *order,
-                               cudaStream_t st);
-
 struct RenderArgs {
-    const float4 *pos_logit;      // per primitive: centre (the opacity logit is not read)
-    // per primitive, written by the projection: (s_a t_a, o), (s_b t_b, 0), (t_n, 0) -- the
-    // scaled tangent axes, the normal and the opacity in the world frame
-    const float4 *prim;
+    const float4 *prim;           // per primitive, kPrimRow float4 written by the projection
     int64_t n;                    // primitives per view (pair id = view * n + i)
     const TileInfo *tiles;        // global tile -> frame and addressing
     const PixFrame *pixframes;
     const uint2 *ranges;          // global tile -> [start, end)
     const uint32_t *tile_order;   // tiles in decreasing order of list length (work order)
-    const uint32_t *sorted_vals;  // pair ids in (tile, range, id) order
-    const uint32_t *entry_rect;   // per list entry: pixel rectangle inside its tile, flip bit
+    // per list entry, in (tile, range, id) order: pair id, pixel rectangle inside its tile with
+    // the flip bit
+    const uint2 *entries;
     const uint8_t *entry_blocks;  // per list entry: the 4 x 8 blocks of its tile it meets
     int64_t n_tiles;
     int64_t n_items;              // n_tiles x blocks per tile

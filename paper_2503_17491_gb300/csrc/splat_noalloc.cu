@@ -24,7 +24,6 @@
 
 #include "splat_internal.cuh"
 
-using splat::PairRec;
 using splat::PixFrame;
 using splat::TileInfo;
 using splat::ViewDesc;
@@ -42,22 +41,26 @@ constexpr int kMaxDevices = 64;
 constexpr size_t align256(size_t x) { return (x + 255) & ~size_t{255}; }
 
 // byte offsets inside the scratch array
-constexpr size_t kOffRecs = 0;
-constexpr size_t kOffDkeys = align256(kOffRecs + sizeof(PairRec) * kMaxGaussians);
-constexpr size_t kOffDvals = align256(kOffDkeys + 4 * kMaxGaussians);
-constexpr size_t kOffDkeys2 = align256(kOffDvals + 4 * kMaxGaussians);
-constexpr size_t kOffDvals2 = align256(kOffDkeys2 + 4 * kMaxGaussians);
-constexpr size_t kOffTrect = align256(kOffDvals2 + 4 * kMaxGaussians);
-constexpr size_t kOffSrect = align256(kOffTrect + 8 * kMaxGaussians);
-constexpr size_t kOffPrect = align256(kOffSrect + 8 * kMaxGaussians);
-constexpr size_t kOffPrim = align256(kOffPrect + 8 * kMaxGaussians);
-constexpr size_t kOffTkeys = align256(kOffPrim + 3 * sizeof(float4) * kMaxGaussians);
-constexpr size_t kOffTvals = align256(kOffTkeys + 4 * kMaxPairs);
-constexpr size_t kOffTkeys2 = align256(kOffTvals + 4 * kMaxPairs);
-constexpr size_t kOffTvals2 = align256(kOffTkeys2 + 4 * kMaxPairs);
-constexpr size_t kOffBlockSums = align256(kOffTvals2 + 4 * kMaxPairs);
-constexpr size_t kOffHist = align256(kOffBlockSums + 4 * splat::kScanGrid);
-constexpr size_t kOffRanges = align256(kOffHist + 4 * size_t{splat::kHistWords});
+constexpr size_t kOffPrect = 0;
+constexpr size_t kOffTouch = align256(kOffPrect + 8 * kMaxGaussians);
+constexpr size_t kOffKappa = align256(kOffTouch + 8 * kMaxGaussians);
+constexpr size_t kOffTouchCount = align256(kOffKappa + 4 * kMaxGaussians);
+constexpr size_t kOffPrim =
+    align256(kOffTouchCount + 4 * (kMaxGaussians / splat::kSmallBlock + 1));
+constexpr size_t kOffTileCount =
+    align256(kOffPrim + splat::kPrimRow * sizeof(float4) * kMaxGaussians);
+constexpr size_t kOffCtaCount = align256(kOffTileCount + 4 * size_t{kMaxTiles});
+// one view: a counting CTA takes at least kMinChunk primitives
+constexpr size_t kCountCtas = kMaxGaussians / splat::kMinChunk + 1;
+static_assert(kMaxGaussians < 1 << 18, "blocks of kSmallBlock primitives");
+static_assert(kMaxTiles <= splat::kMaxSharedTiles, "counted in shared memory");
+constexpr size_t kOffEntries = align256(kOffCtaCount + 4 * kCountCtas * kMaxTiles);
+constexpr size_t kOffEntries2 = align256(kOffEntries + 8 * (kMaxPairs + 128));
+constexpr size_t kOffBlocks = align256(kOffEntries2 + 8 * kMaxPairs);
+constexpr size_t kOffSegments = align256(kOffBlocks + kMaxPairs + 128);
+constexpr size_t kOffRanges =
+    align256(kOffSegments + sizeof(splat::ListSegment) *
+                                (kMaxPairs / splat::kSegTarget + kMaxPairs / splat::kListCap + 2));
 constexpr size_t kOffOrder = align256(kOffRanges + 8 * size_t{kMaxTiles});
 constexpr size_t kOffTiles = align256(kOffOrder + 4 * size_t{kMaxTiles});
 constexpr size_t kOffPix = align256(kOffTiles + sizeof(TileInfo) * kMaxTiles);
@@ -65,7 +68,8 @@ constexpr size_t kOffView = align256(kOffPix + sizeof(PixFrame) * size_t{kMaxTil
 constexpr size_t kOffTfinal = align256(kOffView + sizeof(ViewDesc));
 constexpr size_t kOffNlast = align256(kOffTfinal + 4 * kMaxPixels);
 constexpr size_t kOffCounters = align256(kOffNlast + 4 * kMaxPixels);
-constexpr size_t kOffEvals = align256(kOffCounters + 4 * 8);
+constexpr int kCountersBin = 8, kCounters = kCountersBin + splat::kBinWords;
+constexpr size_t kOffEvals = align256(kOffCounters + 4 * kCounters);
 constexpr size_t kScratchBytes = align256(kOffEvals + 8 * 2);
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -82,13 +86,6 @@ void split(double x, float &hi, float &lo)
 {
     hi = static_cast<float>(x);
     lo = static_cast<float>(x - static_cast<double>(hi));
-}
-
-int bits_for(int64_t n)
-{
-    int b = 0;
-    while ((int64_t{1} << b) < n) ++b;
-    return ((b + 7) / 8) * 8;
 }
 
 // view tables of one view in the host arrays (same definitions as view registration)
@@ -245,21 +242,10 @@ extern "C" SPLAT_API int splat_render_noalloc(const splat_gaussians *g,
     const int64_t n = g->n;
     const int64_t P = int64_t{intr->rows} * intr->cols;
 
-    PairRec *recs = reinterpret_cast<PairRec *>(base + kOffRecs);
-    uint32_t *dkeys = reinterpret_cast<uint32_t *>(base + kOffDkeys);
-    uint32_t *dvals = reinterpret_cast<uint32_t *>(base + kOffDvals);
-    uint32_t *dkeys2 = reinterpret_cast<uint32_t *>(base + kOffDkeys2);
-    uint32_t *dvals2 = reinterpret_cast<uint32_t *>(base + kOffDvals2);
-    uint64_t *trect = reinterpret_cast<uint64_t *>(base + kOffTrect);
-    uint64_t *srect = reinterpret_cast<uint64_t *>(base + kOffSrect);
-    uint64_t *prect = reinterpret_cast<uint64_t *>(base + kOffPrect);
-    uint32_t *tkeys = reinterpret_cast<uint32_t *>(base + kOffTkeys);
-    uint32_t *tvals = reinterpret_cast<uint32_t *>(base + kOffTvals);
-    uint32_t *tkeys2 = reinterpret_cast<uint32_t *>(base + kOffTkeys2);
-    uint32_t *tvals2 = reinterpret_cast<uint32_t *>(base + kOffTvals2);
     float4 *prim = reinterpret_cast<float4 *>(base + kOffPrim);
-    uint32_t *block_sums = reinterpret_cast<uint32_t *>(base + kOffBlockSums);
-    uint32_t *hist = reinterpret_cast<uint32_t *>(base + kOffHist);
+    uint32_t *tile_count = reinterpret_cast<uint32_t *>(base + kOffTileCount);
+    uint64_t *entries = reinterpret_cast<uint64_t *>(base + kOffEntries);
+    uint8_t *blocks = base + kOffBlocks;
     uint2 *ranges = reinterpret_cast<uint2 *>(base + kOffRanges);
     uint32_t *order = reinterpret_cast<uint32_t *>(base + kOffOrder);
     TileInfo *tiles = reinterpret_cast<TileInfo *>(base + kOffTiles);
@@ -276,38 +262,70 @@ extern "C" SPLAT_API int splat_render_noalloc(const splat_gaussians *g,
     NA_CK(cudaMemcpyAsync(tiles, g_tiles, sizeof(TileInfo) * n_tiles, cudaMemcpyHostToDevice, st));
     NA_CK(cudaMemcpyAsync(pix, g_pix, sizeof(PixFrame) * g_view.tiles_r * th * tw,
                           cudaMemcpyHostToDevice, st));
-    NA_CK(cudaMemsetAsync(cnt, 0, 4 * 8, st));
+    NA_CK(cudaMemsetAsync(cnt, 0, 4 * kCounters, st));
+    NA_CK(cudaMemsetAsync(tile_count, 0, 4 * n_tiles, st));
     NA_CK(cudaMemsetAsync(evals, 0, 8 * 2, st));
 
-    NA_CK(splat::launch_project(reinterpret_cast<const float4 *>(g->pos_logit),
-                                reinterpret_cast<const float4 *>(g->quat_wxyz),
-                                reinterpret_cast<const float2 *>(g->log_scale), n, view, 1,
-                                cfg.sigma_cut, cfg.alpha_min, th, tw, cfg.flip_normals, recs, dkeys,
-                                dvals, trect, prect, prim, cnt + 1, cnt + 4, st));
-    uint32_t *dk, *dv;
-    NA_CK(splat::radix_sort_pairs(dkeys, dvals, dkeys2, dvals2, nullptr, n, 32, hist, &dk, &dv, st,
-                                  nullptr, trect, srect));
-    NA_CK(splat::launch_emit(dv, srect, n, cnt + 4, view, n, block_sums, tkeys, tvals, kMaxPairs,
-                             cnt, cnt + 1, st));
-    uint32_t *tk, *tv;
-    NA_CK(splat::radix_sort_pairs(tkeys, tvals, tkeys2, tvals2, cnt, kMaxPairs, bits_for(n_tiles),
-                                  hist, &tk, &tv, st));
-    uint32_t *rects = tv == tvals ? tvals2 : tvals;   // the tile sort's free buffers
-    uint8_t *blocks = reinterpret_cast<uint8_t *>(tk == tkeys ? tkeys2 : tkeys);
-    NA_CK(splat::launch_ranges(tk, tv, prect, tiles, th, tw, cnt, kMaxPairs, ranges, n_tiles, rects,
-                               blocks, st));
-    NA_CK(splat::launch_order_tiles(ranges, n_tiles, order, st));
+    int sms = 0;
+    NA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    splat::ProjectArgs pa{};
+    pa.pos_logit = reinterpret_cast<const float4 *>(g->pos_logit);
+    pa.quat = reinterpret_cast<const float4 *>(g->quat_wxyz);
+    pa.log_scale = reinterpret_cast<const float2 *>(g->log_scale);
+    pa.n = n;
+    pa.views = view;
+    pa.n_views = 1;
+    pa.sigma = cfg.sigma_cut;
+    pa.alpha_min = cfg.alpha_min;
+    pa.tile_h = th;
+    pa.tile_w = tw;
+    pa.flip_normals = cfg.flip_normals;
+    pa.prect = reinterpret_cast<uint64_t *>(base + kOffPrect);
+    pa.touch = reinterpret_cast<uint64_t *>(base + kOffTouch);
+    pa.kappa = reinterpret_cast<float *>(base + kOffKappa);
+    pa.touch_count = reinterpret_cast<uint32_t *>(base + kOffTouchCount);
+    pa.prim = prim;
+    pa.status = cnt + 1;
+    pa.n_valid = cnt + 4;
+    NA_CK(splat::launch_project(pa, st));
+    splat::BinArgs ba{};
+    ba.views = view;
+    ba.n_views = ba.max_active = 1;
+    ba.n = n;
+    ba.tile_h = th;
+    ba.tile_w = tw;
+    ba.n_tiles = n_tiles;
+    ba.tiles = tiles;
+    ba.prect = pa.prect;
+    ba.touch = pa.touch;
+    ba.kappa = pa.kappa;
+    ba.touch_count = pa.touch_count;
+    ba.max_pairs = kMaxPairs;
+    ba.max_view_tiles = static_cast<int>(n_tiles);
+    ba.tile_count = tile_count;
+    ba.cta_count = reinterpret_cast<uint32_t *>(base + kOffCtaCount);
+    ba.ranges = ranges;
+    ba.order = order;
+    ba.entries = entries;
+    ba.entries2 = reinterpret_cast<uint64_t *>(base + kOffEntries2);
+    ba.entry_blocks = blocks;
+    ba.segments = reinterpret_cast<splat::ListSegment *>(base + kOffSegments);
+    ba.d_count = cnt;
+    ba.status = cnt + 1;
+    ba.bin = cnt + kCountersBin;
+    ba.sms = sms;
+    NA_CK(splat::launch_bin_counts(ba, st));
+    NA_CK(splat::launch_emit(ba, st));
+    NA_CK(splat::launch_lists(ba, st));
 
     splat::RenderArgs a{};
-    a.pos_logit = reinterpret_cast<const float4 *>(g->pos_logit);
     a.prim = prim;
     a.n = n;
     a.tiles = tiles;
     a.pixframes = pix;
     a.ranges = ranges;
     a.tile_order = order;
-    a.sorted_vals = tv;
-    a.entry_rect = rects;
+    a.entries = reinterpret_cast<const uint2 *>(entries);
     a.entry_blocks = blocks;
     a.status = cnt + 1;   // no contributor records (forward only)
     a.n_tiles = n_tiles;
@@ -324,8 +342,6 @@ extern "C" SPLAT_API int splat_render_noalloc(const splat_gaussians *g,
     a.n_last = nlast;
     a.queue = cnt + 2;
     a.evals = evals;
-    int sms = 0;
-    NA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int grid = sms * splat::render_occupancy(th, tw, false);
     NA_CK(splat::launch_render_fwd(a, th, tw, grid, st));
 

@@ -263,8 +263,8 @@ __device__ __forceinline__ uint32_t stage(const RenderArgs &A, const TileInfo &t
                                           bool flip, uint32_t rect, WarpBatch &w, int s)
 {
     const int64_t i = static_cast<int64_t>(p) - static_cast<int64_t>(ti.view) * A.n;
-    const float4 pl = A.pos_logit[i];
-    const float4 ea = A.prim[3 * i], eb = A.prim[3 * i + 1], en = A.prim[3 * i + 2];
+    const float4 *e = A.prim + kPrimRow * i;
+    const float4 ea = e[0], eb = e[1], en = e[2], pl = e[3];
     const float *M = ti.M_hi;
     w.a[s] = make_float4(M[0] * ea.x + M[1] * ea.y + M[2] * ea.z,
                          M[3] * ea.x + M[4] * ea.y + M[5] * ea.z,
@@ -591,9 +591,9 @@ __global__ void __launch_bounds__(kBlock, 3) k_render_fwd(const RenderArgs A)
         // Walk the tile's list 128 entries at a time from the 4-aligned entry at or below its
         // start: each lane reads the block masks of four consecutive entries as one word (the
         // next chunk's word is loaded ahead), the entries that meet the block are appended to
-        // the queue in list order (a warp prefix sum of the lanes' counts), with their pair ids
-        // and rectangles read as one 16-byte vector each, and every 32 queued entries are
-        // staged and composited.
+        // the queue in list order (a warp prefix sum of the lanes' counts), their pair ids and
+        // rectangles read as two 16-byte vectors, and every 32 queued entries are staged and
+        // composited.
         const uint32_t *mask_words = reinterpret_cast<const uint32_t *>(A.entry_blocks);
         const uint32_t base = rg.x & ~3u;
         uint32_t mw = 0u;
@@ -610,13 +610,14 @@ __global__ void __launch_bounds__(kBlock, 3) k_render_fwd(const RenderArgs A)
                 const uint32_t j = j0 + k;
                 if (j >= rg.x && j < rg.y && ((mw >> (8 * k + blk)) & 1u)) rel4 |= 1u << k;
             }
-            uint4 pv = make_uint4(0u, 0u, 0u, 0u), rv = pv;
+            uint4 e01 = make_uint4(0u, 0u, 0u, 0u), e23 = e01;
             if (rel4) {
-                pv = *reinterpret_cast<const uint4 *>(A.sorted_vals + j0);
-                rv = *reinterpret_cast<const uint4 *>(A.entry_rect + j0);
+                const uint4 *e = reinterpret_cast<const uint4 *>(A.entries + j0);
+                e01 = e[0];
+                e23 = e[1];
             }
-            const uint32_t pa[4] = {pv.x, pv.y, pv.z, pv.w};
-            const uint32_t ra[4] = {rv.x, rv.y, rv.z, rv.w};
+            const uint32_t pa[4] = {e01.x, e01.z, e23.x, e23.z};
+            const uint32_t ra[4] = {e01.y, e01.w, e23.y, e23.w};
             // once some pixels of the block are saturated, an entry whose rectangle covers only
             // saturated ones is passed over
             const uint32_t live = __ballot_sync(kFull, !done);

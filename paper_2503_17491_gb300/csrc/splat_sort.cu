@@ -1,512 +1,834 @@
-// K2-K4: tile binning.
+// K2-K4: tile binning, from the projection's pixel rectangles to the per-tile lists in
+// (range, primitive id) order (Sec. 3.2.1).
 //
-// The per-tile lists sorted by range (Sec. 3.2.1) are built in three steps:
-//   1. a stable radix sort of all (view, primitive) pairs by their binary32 range key
-//      (one key per pair, not per tile: far fewer keys than (tile, primitive) entries);
-//   2. emission, in that order, of one (global tile id, pair id) entry per touched tile, at
-//      offsets given by an exclusive scan of the tile counts (K2);
-//   3. a stable radix sort of the entries by tile id (K3).  Stability keeps step 1's order
-//      inside every tile, so each list ends up in (tile, range, id) order -- the same order as
-//      sorting 64-bit (tile << 32 | range bits) keys with the id as the final tie-break.
-// Tile ranges [start, end) follow from the sorted tile ids (K4).
+//   count    list lengths: a CTA counts the tiles of a chunk of one view's touching pairs in
+//            shared memory and adds its counts to the global ones;
+//   layout   one CTA: [start, end) of every tile's list by an exclusive scan of the counts, the
+//            work order (longest lists first) and the total;
+//   emission (range key << 32 | pair id) into each touched tile's slice: a CTA reserves as many
+//            places of each tile as it counted with one atomic and hands them out in shared
+//            memory;
+//   split    only lists above kListCap: one CTA cuts a list by its leading key bits into
+//            segments of at most kListCap entries;
+//   lists    every list or segment is sorted in shared memory by the 64-bit key, by one warp up
+//            to 255 entries, by one CTA above, and written back with each entry's pixel
+//            rectangle inside its tile and the 4 x 8 blocks it meets.
+// The keys are unique (the pair id is part of them), so the order in which places are handed out
+// does not matter: the sorted lists are the same bits in every run.
 //
-// The sort is a reduce-then-scan LSD radix sort with 8-bit digits on a fixed grid of CTAs, so
-// that the element count can live on the device (it is data dependent after emission) and the
-// whole pipeline can be captured in a CUDA graph.  Ranking inside a CTA tile is warp-level
-// (match.any) and stable in (warp, item, lane) = index order; the ranked tile is first sorted
-// by digit in shared memory and then written out run by run, so that global stores coalesce.
+// Why not a global radix sort: sorting all pairs by range and the entries by tile takes four plus
+// two passes of three launches each, whose per-tile ranking is one serial chain of shared memory
+// per warp; here an entry is written once and read by the list sort, in five launches.  From
+// pairs to lists, 12 views x 500 k primitives (5.3 M entries): 0.51 ms in 24 launches -> 0.22 ms
+// (count 0.031, layout 0.007, emission 0.066, split 0.025, lists 0.105); 64 tiles of 1,500
+// entries: 0.13 -> 0.022 ms.  The lists stage is bound by the shared-memory latency of its four
+// passes over the keys, the counting stages by instruction issue.
+// Everything runs on counts that stay on the device, with fixed launch shapes, so the pipeline
+// can be captured in a CUDA graph.
 
 #include "splat_internal.cuh"
 
 namespace splat {
 namespace {
 
-constexpr int kRadix = 256;
-constexpr int kThreads = 256;
-constexpr int kItems = kSortTile / kThreads;   // 8
-constexpr int kWarps = kThreads / 32;
-
-__device__ __forceinline__ int64_t chunk_of(int64_t n, int grid)
-{
-    int64_t c = (n + grid - 1) / grid;
-    return (c + kSortTile - 1) / kSortTile * kSortTile;
-}
-
-__device__ __forceinline__ int64_t clamp_count(const uint32_t *d_count, int64_t max_n)
-{
-    int64_t n = d_count ? static_cast<int64_t>(*d_count) : max_n;
-    return n < max_n ? n : max_n;
-}
-
-// per-CTA digit histogram: hist[digit * grid + cta]
-__global__ void __launch_bounds__(kThreads) k_upsweep(const uint32_t *__restrict__ keys,
-                                                      const uint32_t *d_count, int64_t max_n,
-                                                      int shift, int drop_max,
-                                                      uint32_t *__restrict__ hist)
-{
-    __shared__ uint32_t s_cnt[kWarps][kRadix];
-    const int tid = threadIdx.x, warp = tid >> 5;
-    for (int k = tid; k < kWarps * kRadix; k += kThreads) (&s_cnt[0][0])[k] = 0;
-    __syncthreads();
-    const int64_t n = clamp_count(d_count, max_n);
-    const int64_t chunk = chunk_of(n, gridDim.x);
-    const int64_t begin = chunk * blockIdx.x;
-    const int64_t end = begin + chunk < n ? begin + chunk : n;
-    for (int64_t j = begin + tid; j < end; j += kThreads) {
-        const uint32_t k = keys[j];
-        if (!(drop_max && k == 0xFFFFFFFFu)) atomicAdd(&s_cnt[warp][(k >> shift) & 0xFF], 1u);
-    }
-    __syncthreads();
-    uint32_t t = 0;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) t += s_cnt[w][tid];
-    hist[static_cast<int64_t>(tid) * gridDim.x + blockIdx.x] = t;
-}
-
-// per digit (one warp each): exclusive scan of its kSortGrid per-CTA counts hist[d * grid + b]
-// in place, and the digit's total into dtot[d].  Each lane takes a run of kPer consecutive
-// counts, so all loads are issued before the one warp scan of the run sums.
-__global__ void __launch_bounds__(256) k_scan_digits(uint32_t *__restrict__ hist, int grid,
-                                                     uint32_t *__restrict__ dtot)
-{
-    constexpr int kPer = (kSortGrid + 31) / 32;
-    const int lane = threadIdx.x & 31;
-    const int d = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (d >= kRadix) return;
-    uint32_t *h = hist + static_cast<int64_t>(d) * grid;
-    uint32_t v[kPer];
-    uint32_t sum = 0;
-#pragma unroll
-    for (int i = 0; i < kPer; ++i) {
-        const int b = lane * kPer + i;
-        v[i] = b < grid ? h[b] : 0u;
-        sum += v[i];
-    }
-    uint32_t x = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-        if (lane >= o) x += y;
-    }
-    uint32_t run = x - sum;
-#pragma unroll
-    for (int i = 0; i < kPer; ++i) {
-        const int b = lane * kPer + i;
-        if (b < grid) h[b] = run;
-        run += v[i];
-    }
-    const uint32_t total = __shfl_sync(0xFFFFFFFFu, x, 31);
-    if (lane == 0) dtot[d] = total;
-}
-
-__global__ void __launch_bounds__(kThreads) k_downsweep(
-    const uint32_t *__restrict__ keys_in, const uint32_t *__restrict__ vals_in,
-    uint32_t *__restrict__ keys_out, uint32_t *__restrict__ vals_out, const uint32_t *d_count,
-    int64_t max_n, int shift, int drop_max, const uint32_t *__restrict__ hist,
-    const uint32_t *__restrict__ dtot, const uint64_t *__restrict__ aux_in,
-    uint64_t *__restrict__ aux_out)
-{
-    __shared__ uint32_t s_base[kRadix];          // running global offset per digit
-    __shared__ uint32_t s_wcnt[kWarps][kRadix];  // per-warp digit counts -> warp prefixes
-    __shared__ uint32_t s_tile[kRadix];          // digit totals of the current tile
-    __shared__ uint32_t s_toff[kRadix];          // digit offsets inside the current tile
-    __shared__ uint32_t s_wsum[kWarps];
-    __shared__ uint32_t s_kept;                  // items of the current tile that are written
-    __shared__ uint32_t s_key[kSortTile], s_val[kSortTile];   // the tile, sorted by digit
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t n = clamp_count(d_count, max_n);
-    const int64_t chunk = chunk_of(n, gridDim.x);
-    const int64_t begin = chunk * blockIdx.x;
-    const int64_t end = begin + chunk < n ? begin + chunk : n;
-    if (begin >= end) return;
-    {   // digit base: exclusive scan of the digit totals, plus this CTA's offset in its digit
-        const uint32_t t = dtot[tid];
-        uint32_t x = t;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) s_tile[warp] = x;
-        __syncthreads();
-        uint32_t wbase = 0;
-        for (int w = 0; w < warp; ++w) wbase += s_tile[w];
-        s_base[tid] = wbase + x - t + hist[static_cast<int64_t>(tid) * gridDim.x + blockIdx.x];
-        __syncthreads();
-    }
-    const uint32_t lt_mask = (1u << lane) - 1u;
-
-    for (int64_t tb = begin; tb < end; tb += kSortTile) {
-        for (int k = tid; k < kWarps * kRadix; k += kThreads) (&s_wcnt[0][0])[k] = 0;
-        __syncthreads();
-        uint32_t key[kItems], val[kItems], rank[kItems];
-        int dig[kItems];
-#pragma unroll
-        for (int it = 0; it < kItems; ++it) {
-            const int64_t j = tb + warp * (32 * kItems) + it * 32 + lane;
-            key[it] = j < end ? keys_in[j] : 0u;
-            const bool valid = j < end && !(drop_max && key[it] == 0xFFFFFFFFu);
-            val[it] = valid ? vals_in[j] : 0u;
-            dig[it] = valid ? static_cast<int>((key[it] >> shift) & 0xFF) : kRadix + lane;
-            const uint32_t peers = __match_any_sync(0xFFFFFFFFu, dig[it]);
-            uint32_t before = 0;
-            if (valid) before = s_wcnt[warp][dig[it]];
-            __syncwarp();
-            rank[it] = before + __popc(peers & lt_mask);
-            const int last = 31 - __clz(peers);
-            if (valid && lane == last) s_wcnt[warp][dig[it]] = before + __popc(peers);
-            __syncwarp();
-        }
-        __syncthreads();
-        {   // digit tid: exclusive prefix over warps, tile total
-            uint32_t run = 0;
-#pragma unroll
-            for (int w = 0; w < kWarps; ++w) {
-                const uint32_t c = s_wcnt[w][tid];
-                s_wcnt[w][tid] = run;
-                run += c;
-            }
-            s_tile[tid] = run;
-            // the digit's offset inside the tile: exclusive scan of the tile totals over digits
-            uint32_t x = run;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-                if (lane >= o) x += y;
-            }
-            if (lane == 31) s_wsum[warp] = x;
-            __syncthreads();
-            uint32_t wbase = 0;
-            for (int w = 0; w < warp; ++w) wbase += s_wsum[w];
-            s_toff[tid] = wbase + x - run;
-            if (tid == kRadix - 1) s_kept = wbase + x;
-        }
-        __syncthreads();
-        // sort the tile by digit in shared memory (stable: warp, item, lane order) ...
-#pragma unroll
-        for (int it = 0; it < kItems; ++it) {
-            if (dig[it] < kRadix) {
-                const uint32_t lpos = s_toff[dig[it]] + s_wcnt[warp][dig[it]] + rank[it];
-                s_key[lpos] = key[it];
-                s_val[lpos] = val[it];
-            }
-        }
-        __syncthreads();
-        // ... and write each digit's run to its global place: consecutive threads, consecutive
-        // addresses
-        const int cnt = static_cast<int>(s_kept);
-        for (int i = tid; i < cnt; i += kThreads) {
-            const uint32_t k = s_key[i];
-            const int d = static_cast<int>((k >> shift) & 0xFF);
-            const uint32_t pos = s_base[d] + (static_cast<uint32_t>(i) - s_toff[d]);
-            keys_out[pos] = k;
-            vals_out[pos] = s_val[i];
-            if (aux_out) aux_out[pos] = aux_in[s_val[i]];
-        }
-        __syncthreads();
-        s_base[tid] += s_tile[tid];
-        __syncthreads();
-    }
-}
+constexpr uint32_t kFull = 0xFFFFFFFFu;
+constexpr int kListThreads = 256, kListCtas = 3;   // CTAs per SM
+constexpr int kListWarps = kListThreads / 32;
+constexpr int kWarpCap = 256;             // lists below this are sorted by one warp
+constexpr int kMaxItems = kListCap / kListThreads;   // 16 keys a thread
+constexpr int kMidBucket = 9;             // 32 - clz(kWarpCap): lists of 256 and more
+constexpr int kLongBucket = 13;           // lists of kListCap and more
+static_assert(kWarpCap == 1 << (kMidBucket - 1) && kListCap == 1 << (kLongBucket - 1), "buckets");
 
 // ---------------------------------------------------------------------------------------------
-// emission (K2)
+// layout (one CTA)
 // ---------------------------------------------------------------------------------------------
+constexpr int kLayoutThreads = 1024;
 
-__device__ __forceinline__ uint32_t rect_count(uint64_t w)
-{
-    return static_cast<uint32_t>((w >> 16) & 0xFFFFu) * static_cast<uint32_t>(w >> 48);
-}
+__device__ __forceinline__ int len_bucket(uint32_t len) { return len ? 32 - __clz(len) : 0; }
 
-// per-CTA sums of the tile counts of its chunk of sorted pairs
-__global__ void __launch_bounds__(kThreads) k_count_sums(const uint64_t *__restrict__ srect,
-                                                         int64_t n_total, const uint32_t *n_valid,
-                                                         uint32_t *__restrict__ block_sums)
+// exclusive sum over the CTA's threads; *total gets the sum of all
+template <int kThreads, typename T>
+__device__ __forceinline__ T block_excl_scan(T v, T *s_warp, T *total)
 {
-    __shared__ unsigned long long s_sum[kWarps];
-    const int64_t n = clamp_count(n_valid, n_total);
-    const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
-    const int64_t b = chunk * blockIdx.x;
-    const int64_t e = b + chunk < n ? b + chunk : n;
-    unsigned long long sum = 0;
-    for (int64_t j = b + threadIdx.x; j < e; j += kThreads) sum += rect_count(srect[j]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-    if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = sum;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long t = 0;
-        for (int w = 0; w < kWarps; ++w) t += s_sum[w];
-        block_sums[blockIdx.x] = t > 0xFFFFFFFFull ? 0xFFFFFFFFu : static_cast<uint32_t>(t);
-    }
-}
-
-// exclusive scan of the CTA sums (grid <= kScanGrid entries, kScanPer consecutive ones per
-// thread); total -> *d_count (saturated)
-constexpr int kScanPer = kScanGrid / 1024;
-static_assert(kScanGrid % 1024 == 0, "the CTA-sum scan takes whole runs of 1024");
-__global__ void __launch_bounds__(1024) k_scan_sums(uint32_t *__restrict__ block_sums, int grid,
-                                                    int64_t max_pairs, uint32_t *d_count,
-                                                    uint32_t *status)
-{
-    __shared__ unsigned long long s_w[32];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint32_t e[kScanPer];
-    unsigned long long v = 0;
-#pragma unroll
-    for (int i = 0; i < kScanPer; ++i) {
-        const int b = tid * kScanPer + i;
-        e[i] = b < grid ? block_sums[b] : 0u;
-        v += e[i];
-    }
-    unsigned long long x = v;   // warp inclusive scan, then the warps' totals scanned by warp 0
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    T x = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        const T y = __shfl_up_sync(kFull, x, o);
         if (lane >= o) x += y;
     }
-    if (lane == 31) s_w[warp] = x;
+    if (lane == 31) s_warp[warp] = x;
     __syncthreads();
     if (warp == 0) {
-        const unsigned long long w = s_w[lane];
-        unsigned long long z = w;
+        const T w = lane < kThreads / 32 ? s_warp[lane] : T(0);
+        T z = w;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, z, o);
+            const T y = __shfl_up_sync(kFull, z, o);
             if (lane >= o) z += y;
         }
-        s_w[lane] = z - w;
+        if (lane < kThreads / 32) s_warp[lane] = z - w;
+        if (lane == 31) s_warp[32] = z;
     }
     __syncthreads();
-    const unsigned long long incl = x + s_w[warp];
-    unsigned long long run = incl - v;
-#pragma unroll
-    for (int i = 0; i < kScanPer; ++i) {
-        const int b = tid * kScanPer + i;
-        if (b < grid) block_sums[b] = run > 0xFFFFFFFFull ? 0xFFFFFFFFu : static_cast<uint32_t>(run);
-        run += e[i];
-    }
-    if (tid == 1023) {
-        const unsigned long long total = incl;
-        if (total > static_cast<unsigned long long>(max_pairs)) {
-            atomicOr(status, SPLAT_STATUS_CAPACITY);
-            *d_count = static_cast<uint32_t>(max_pairs);
-        } else {
-            *d_count = static_cast<uint32_t>(total);
-        }
-    }
+    if (total) *total = s_warp[32];
+    return x - v + s_warp[warp];
 }
 
-// Emission: each CTA takes its chunk of sorted pairs 256 at a time, reading the pair ids and
-// their tile rectangles in sorted order; a CTA scan of the tile counts gives every pair its run
-// of output entries, and then each thread writes one entry at a time -- consecutive threads,
-// consecutive entries -- finding its pair by binary search over the run ends.  Entry k of a
-// pair with tile columns tc0 .. tc0 + ntc - 1 (mod tiles_c) and first tile row tr0 is tile row
-// tr0 + k / ntc, column tc0 + k % ntc: row-major over the pair's tile rectangle.
-__global__ void __launch_bounds__(kThreads) k_emit(
-    const uint32_t *__restrict__ sorted, const uint64_t *__restrict__ srect, int64_t n_total,
-    const uint32_t *n_valid, const ViewDesc *__restrict__ views, int64_t n_per_view,
-    const uint32_t *__restrict__ block_base, uint32_t *__restrict__ tile_keys,
-    uint32_t *__restrict__ tile_vals, int64_t max_pairs)
+__global__ void __launch_bounds__(kLayoutThreads) k_layout(
+    const uint32_t *__restrict__ tile_count, int64_t n_tiles, int64_t max_pairs,
+    uint2 *__restrict__ ranges, uint32_t *__restrict__ order, uint32_t *__restrict__ d_count,
+    uint32_t *status, uint32_t *__restrict__ bin)
 {
-    __shared__ uint32_t s_warp[kWarps];
-    __shared__ uint32_t s_carry;
-    __shared__ uint32_t s_end[kThreads];    // end of each pair's run inside the batch
-    __shared__ uint32_t s_p[kThreads];      // pair id
-    __shared__ uint32_t s_row0[kThreads];   // global id of the tile (first tile row, column 0)
-    __shared__ int s_tc0[kThreads], s_ntc[kThreads], s_tilesc[kThreads];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t n = clamp_count(n_valid, n_total);
-    const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
-    const int64_t b = chunk * blockIdx.x;
-    const int64_t e = b + chunk < n ? b + chunk : n;
-    const uint32_t npv = static_cast<uint32_t>(n_per_view);
-    if (tid == 0) s_carry = block_base[blockIdx.x];
-    __syncthreads();
-    for (int64_t base = b; base < e; base += kThreads) {
-        const int64_t j = base + tid;
-        uint32_t p = 0, cnt = 0;
-        uint64_t w = 0;
-        if (j < e) {
-            p = sorted[j];
-            w = srect[j];
-            cnt = rect_count(w);
-        }
-        // block inclusive scan of cnt
-        uint32_t x = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) s_warp[warp] = x;
-        if (cnt) {
-            const ViewDesc &vd = views[p / npv];
-            s_row0[tid] = static_cast<uint32_t>(vd.tile_offset +
-                                                static_cast<int64_t>(w & 0xFFFFu) * vd.tiles_c);
-            s_tc0[tid] = static_cast<int>((w >> 32) & 0xFFFFu);
-            s_ntc[tid] = static_cast<int>(w >> 48);
-            s_tilesc[tid] = vd.tiles_c;
-        }
-        s_p[tid] = p;
-        __syncthreads();
-        uint32_t wbase = 0, total = 0;
-#pragma unroll
-        for (int k = 0; k < kWarps; ++k) {
-            const uint32_t sw = s_warp[k];
-            wbase += k < warp ? sw : 0u;
-            total += sw;
-        }
-        s_end[tid] = wbase + x;
-        __syncthreads();
-        const uint64_t carry = s_carry;
-        for (uint32_t q = tid; q < total; q += kThreads) {
-            int lo = 0, hi = kThreads - 1;   // first pair whose run ends after q
-#pragma unroll
-            for (int step = 0; step < 8; ++step) {
-                const int mid = (lo + hi) >> 1;
-                if (s_end[mid] > q) hi = mid; else lo = mid + 1;
-            }
-            const uint32_t k = q - (lo ? s_end[lo - 1] : 0u);
-            const uint32_t ntc = static_cast<uint32_t>(s_ntc[lo]);
-            const uint32_t row = k / ntc;
-            int tc = s_tc0[lo] + static_cast<int>(k - row * ntc);
-            const int tiles_c = s_tilesc[lo];
-            tc = tc >= tiles_c ? tc - tiles_c : tc;
-            const uint64_t o = carry + q;
-            if (o < static_cast<uint64_t>(max_pairs)) {
-                tile_keys[o] = s_row0[lo] + row * static_cast<uint32_t>(tiles_c) +
-                               static_cast<uint32_t>(tc);
-                tile_vals[o] = s_p[lo];
-            }
-        }
-        __syncthreads();
-        if (tid == 0) s_carry += total;
-        __syncthreads();
-    }
-}
-
-// K4: [start, end) per tile from sorted tile ids (ranges zeroed before), and each entry's pixel
-// rectangle inside its tile, so that the renderer's warps (eight per tile) need not each gather
-// the record and clip it
-__global__ void k_ranges(const uint32_t *__restrict__ keys, const uint32_t *__restrict__ vals,
-                         const uint64_t *__restrict__ prect, const TileInfo *__restrict__ tiles,
-                         int tile_h, int tile_w, const uint32_t *d_count, int64_t max_pairs,
-                         uint2 *__restrict__ ranges, uint32_t *__restrict__ entry_rect,
-                         uint8_t *__restrict__ entry_blocks)
-{
-    const int64_t m = clamp_count(d_count, max_pairs);
-    for (int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; j < m;
-         j += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const uint32_t t = keys[j];
-        if (j == 0 || keys[j - 1] != t) ranges[t].x = static_cast<uint32_t>(j);
-        if (j == m - 1 || keys[j + 1] != t) ranges[t].y = static_cast<uint32_t>(j + 1);
-        const TileInfo &ti = tiles[t];
-        const uint32_t r = tile_local_rect(unpack_pixel_rect(prect[vals[j]]), ti.tr, ti.tc,
-                                           ti.cols, tile_h, tile_w);
-        entry_rect[j] = r;
-        entry_blocks[j] = static_cast<uint8_t>(rect_blocks(r & ~kRectFlip, tile_h, tile_w));
-    }
-}
-
-// work order of the compositing kernels: longest lists first, by log2 of the length, so that
-// the persistent queue ends on short items (one CTA; a few microseconds)
-__global__ void __launch_bounds__(1024) k_order_tiles(const uint2 *__restrict__ ranges,
-                                                      int64_t n_tiles, uint32_t *__restrict__ order)
-{
+    __shared__ unsigned long long s_warp[33];
     __shared__ uint32_t s_cnt[33], s_off[33];
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31;
     if (tid < 33) s_cnt[tid] = 0;
     __syncthreads();
-    for (int64_t t = tid; t < n_tiles; t += blockDim.x) {
-        const uint2 r = ranges[t];
-        const uint32_t len = r.y - r.x;
-        atomicAdd(&s_cnt[len ? 32 - __clz(len) : 0], 1u);
+    // each thread takes a run of consecutive tiles; the loop bounds are uniform so that the
+    // whole warp takes part in the matches
+    const int64_t per = (n_tiles + kLayoutThreads - 1) / kLayoutThreads;
+    const int64_t t0 = per * tid;
+    unsigned long long sum = 0;
+    for (int64_t k = 0; k < per; ++k) {
+        const bool in = t0 + k < n_tiles;
+        const uint32_t len = in ? tile_count[t0 + k] : 0u;
+        sum += len;
+        const int b = in ? len_bucket(len) : 33;
+        const uint32_t peers = __match_any_sync(kFull, b);
+        if (in && lane == __ffs(peers) - 1) atomicAdd(&s_cnt[b], __popc(peers));
+    }
+    unsigned long long total;
+    unsigned long long run = block_excl_scan<kLayoutThreads>(sum, s_warp, &total);
+    if (tid == 0) {
+        uint32_t at = 0;
+        for (int b = 32; b >= 0; --b) {
+            s_off[b] = at;
+            at += s_cnt[b];
+        }
+        bin[kBinLong] = s_off[kLongBucket - 1];
+        bin[kBinSegments] = 0u;
+        bin[kBinQueueSeg] = 0u;
+        bin[kBinMid] = s_off[kMidBucket - 1];
+        const bool over = total > static_cast<unsigned long long>(max_pairs);
+        if (over) atomicOr(status, SPLAT_STATUS_CAPACITY);
+        *d_count = static_cast<uint32_t>(over ? max_pairs : static_cast<int64_t>(total));
     }
     __syncthreads();
-    if (tid == 0) {
-        uint32_t run = 0;
-        for (int b = 32; b >= 0; --b) {
-            s_off[b] = run;
-            run += s_cnt[b];
+    // past the capacity a list keeps the places below it (the status bit marks the result)
+    const unsigned long long cap = static_cast<unsigned long long>(max_pairs);
+    for (int64_t k = 0; k < per; ++k) {
+        const bool in = t0 + k < n_tiles;
+        const uint32_t len = in ? tile_count[t0 + k] : 0u;
+        const int b = in ? len_bucket(len) : 33;
+        const uint32_t peers = __match_any_sync(kFull, b);
+        const int lead = __ffs(peers) - 1;
+        uint32_t at = 0;
+        if (in && lane == lead) at = atomicAdd(&s_off[b], __popc(peers));
+        at = __shfl_sync(kFull, at, lead) + __popc(peers & ((1u << lane) - 1u));
+        if (in) {
+            order[at] = static_cast<uint32_t>(t0 + k);
+            const unsigned long long e = run + len;
+            ranges[t0 + k] = len == 0 ? make_uint2(0u, 0u)
+                                      : make_uint2(static_cast<uint32_t>(run < cap ? run : cap),
+                                                   static_cast<uint32_t>(e < cap ? e : cap));
+            run = e;
         }
     }
-    __syncthreads();
-    for (int64_t t = tid; t < n_tiles; t += blockDim.x) {
-        const uint2 r = ranges[t];
-        const uint32_t len = r.y - r.x;
-        order[atomicAdd(&s_off[len ? 32 - __clz(len) : 0], 1u)] = static_cast<uint32_t>(t);
+}
+
+// ---------------------------------------------------------------------------------------------
+// count and emission: a CTA takes a chunk of one view's touching pairs
+// ---------------------------------------------------------------------------------------------
+constexpr int kChunkThreads = 512;
+
+struct Chunk {
+    const uint64_t *touch;
+    const float *kappa;
+    const uint32_t *touch_count;
+    int begin, end;        // units of 32 places: unit u is places 32 u .. of the view
+    int unit_shift;        // log2 of the units a block
+    int tiles_c, n_tiles;
+    uint32_t *tile_count;
+    uint32_t *cta_count;   // this CTA's count of every tile of the view
+    const uint2 *ranges;
+};
+
+__device__ __forceinline__ Chunk chunk_of(const BinArgs &A, int v)
+{
+    const ViewDesc &vd = A.views[v];
+    const int64_t p0 = static_cast<int64_t>(v) * A.n;
+    int row = v;   // the view's rank among the drawn ones
+    if (A.active) {
+        row = 0;
+        for (int k = 0; k < v; ++k) row += A.active[k] ? 1 : 0;
     }
+    const int first = A.chunk * static_cast<int>(blockIdx.x);
+    Chunk c;
+    c.touch = A.touch + p0;
+    c.kappa = A.kappa + p0;
+    c.touch_count = A.touch_count + static_cast<int64_t>(v) * A.blocks;
+    c.unit_shift = __ffs(A.block_prims) - 1 - 5;   // block_prims is a power of two
+    c.begin = first << c.unit_shift;
+    c.end = min(first + A.chunk, A.blocks) << c.unit_shift;
+    c.tiles_c = vd.tiles_c;
+    c.n_tiles = vd.tiles_r * vd.tiles_c;
+    c.tile_count = A.tile_count + vd.tile_offset;
+    c.cta_count = A.cta_count +
+                  (static_cast<int64_t>(row) * gridDim.x + blockIdx.x) * A.max_view_tiles;
+    c.ranges = A.ranges + vd.tile_offset;
+    return c;
+}
+
+// f(tile of the view, place of the pair, its primitive in the view) for every tile of every
+// touching pair of the chunk, 32 pairs a warp at a time, kUnitLoads of them read ahead.  While no
+// pair of a warp touches more than kLaneTiles tiles, every lane walks its own; otherwise the warp
+// numbers the tiles of its 32 pairs by a prefix sum and gives one to every lane, so that one wide
+// pair costs its warp no more than as many narrow ones.
+constexpr int kLaneTiles = 8, kUnitLoads = 4;
+
+template <typename F>
+__device__ __forceinline__ void for_each_entry(const Chunk &c, F f)
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t tiles_c = static_cast<uint32_t>(c.tiles_c);
+    constexpr int kWarps = kChunkThreads / 32;
+    for (int u0 = c.begin + static_cast<int>(threadIdx.x >> 5); u0 < c.end;
+         u0 += kWarps * kUnitLoads) {
+        uint32_t live[kUnitLoads];   // the unit's pairs
+        uint64_t word[kUnitLoads];
+#pragma unroll
+        for (int i = 0; i < kUnitLoads; ++i) {
+            const int u = u0 + i * kWarps;
+            const uint32_t n = u < c.end ? c.touch_count[u >> c.unit_shift] : 0u;
+            const uint32_t b = static_cast<uint32_t>(u - (u >> c.unit_shift << c.unit_shift)) * 32u;
+            live[i] = n > b ? n - b : 0u;
+        }
+#pragma unroll
+        for (int i = 0; i < kUnitLoads; ++i)
+            word[i] = static_cast<uint32_t>(lane) < live[i]
+                          ? c.touch[32 * static_cast<int64_t>(u0 + i * kWarps) + lane]
+                          : 0ull;
+#pragma unroll 1
+        for (int i = 0; i < kUnitLoads; ++i) {
+            if (live[i] == 0u) continue;
+            const int u = u0 + i * kWarps;
+            const uint32_t at0 = 32u * static_cast<uint32_t>(u);
+            const uint32_t first = 32u * static_cast<uint32_t>(u >> c.unit_shift << c.unit_shift);
+            TileRect t{};
+            uint32_t local = 0, cnt = 0;
+            if (static_cast<uint32_t>(lane) < live[i]) {
+                t = unpack_touch(word[i], local);
+                cnt = static_cast<uint32_t>(t.nr) * static_cast<uint32_t>(t.nc);
+            }
+            if (!__any_sync(kFull, cnt > kLaneTiles)) {
+                uint32_t row = static_cast<uint32_t>(t.r0) * tiles_c;
+                uint32_t col = static_cast<uint32_t>(t.c0);
+                int left = t.nc;
+                for (uint32_t k = 0; k < cnt; ++k) {
+                    f(row + col, at0 + lane, first + local);
+                    col = col + 1 == tiles_c ? 0u : col + 1;
+                    if (--left == 0) {   // the next tile row
+                        left = t.nc;
+                        col = static_cast<uint32_t>(t.c0);
+                        row += tiles_c;
+                    }
+                }
+                continue;
+            }
+            uint32_t incl = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const uint32_t total = __shfl_sync(kFull, incl, 31);
+            const uint32_t rc = static_cast<uint32_t>(t.r0) | static_cast<uint32_t>(t.c0) << 16;
+            const uint32_t cl = static_cast<uint32_t>(t.nc) | local << 16;
+            for (uint32_t q0 = 0; q0 < total; q0 += 32) {
+                const uint32_t q = q0 + lane;
+                int src = 0;   // the first lane whose run ends after q
+#pragma unroll
+                for (int s = 16; s > 0; s >>= 1)
+                    if (__shfl_sync(kFull, incl, src + s - 1) <= q) src += s;
+                const uint32_t k = q - __shfl_sync(kFull, incl - cnt, src);
+                const uint32_t r = __shfl_sync(kFull, rc, src), m = __shfl_sync(kFull, cl, src);
+                if (q < total) {
+                    const uint32_t nc = m & 0xFFFFu, row = k / nc;
+                    uint32_t col = (r >> 16) + (k - row * nc);
+                    col = col >= tiles_c ? col - tiles_c : col;
+                    f(((r & 0xFFFFu) + row) * tiles_c + col, at0 + src, first + (m >> 16));
+                }
+            }
+        }
+    }
+}
+
+// With shared counters a tile's count sees one global atomic per CTA instead of one per entry:
+// neighbouring threads' pairs fall on a few hundred tiles of one view, and same-address atomics
+// in L2 serialise (emission of 5.3 M entries: 0.95 ms with an atomic per entry).
+template <bool kShared>
+__global__ void __launch_bounds__(kChunkThreads) k_count(const BinArgs A)
+{
+    extern __shared__ uint32_t s_cnt[];
+    const int v = blockIdx.y;
+    if (A.active && !A.active[v]) return;
+    const Chunk c = chunk_of(A, v);
+    if (kShared) {
+        for (int t = threadIdx.x; t < c.n_tiles; t += kChunkThreads) s_cnt[t] = 0u;
+        __syncthreads();
+    }
+    uint32_t *cnt = kShared ? s_cnt : c.tile_count;
+    for_each_entry(c, [&](uint32_t t, uint32_t, uint32_t) { atomicAdd(cnt + t, 1u); });
+    if (kShared) {
+        __syncthreads();
+        for (int t = threadIdx.x; t < c.n_tiles; t += kChunkThreads) {
+            const uint32_t n = s_cnt[t];
+            if (n) atomicAdd(c.tile_count + t, n);
+            c.cta_count[t] = n;
+        }
+    }
+}
+
+template <bool kShared>
+__global__ void __launch_bounds__(kChunkThreads) k_emit(const BinArgs A)
+{
+    extern __shared__ uint32_t s_cnt[];
+    const int v = blockIdx.y;
+    if (A.active && !A.active[v]) return;
+    const Chunk c = chunk_of(A, v);
+    if (kShared) {
+        for (int t = threadIdx.x; t < c.n_tiles; t += kChunkThreads) {
+            const uint32_t n = c.cta_count[t];   // the tile's count counts down: this CTA takes
+            if (n) s_cnt[t] = atomicSub(c.tile_count + t, n) - n;   // the places [s_cnt, s_cnt + n)
+        }
+        __syncthreads();
+    }
+    const uint32_t p0 = static_cast<uint32_t>(static_cast<int64_t>(v) * A.n);
+    for_each_entry(c, [&](uint32_t t, uint32_t at, uint32_t i) {
+        const uint32_t k =
+            kShared ? atomicAdd(s_cnt + t, 1u) : atomicSub(c.tile_count + t, 1u) - 1u;
+        const uint2 rg = c.ranges[t];
+        if (k < rg.y - rg.x)   // past the capacity the list ends early
+            A.entries[rg.x + k] =
+                static_cast<uint64_t>(__float_as_uint(c.kappa[at])) << 32 | (p0 + i);
+    });
+}
+
+// ---------------------------------------------------------------------------------------------
+// long lists: one most-significant-bits pass into segments
+// ---------------------------------------------------------------------------------------------
+constexpr int kSplitThreads = 512;
+constexpr int kSplitBins = 4096;
+constexpr int kBinsPer = kSplitBins / kSplitThreads;
+
+// 128 bins an octave of range from 2^-12 on (the ends take what lies beyond)
+__device__ __forceinline__ uint32_t split_bin(uint64_t key)
+{
+    constexpr int kFirst = (127 - 12) << 7;
+    const int b = static_cast<int>(key >> 48) - kFirst;
+    return static_cast<uint32_t>(b < 0 ? 0 : (b > kSplitBins - 1 ? kSplitBins - 1 : b));
+}
+
+// f(key) for the keys src[0 .. n), kSplitLoads loads in flight a thread
+constexpr int kSplitLoads = 8;
+template <typename F>
+__device__ __forceinline__ void for_each_key(const uint64_t *src, uint32_t n, F f)
+{
+    for (uint32_t b = 0; b < n; b += kSplitThreads * kSplitLoads) {
+        uint64_t k[kSplitLoads];
+#pragma unroll
+        for (int u = 0; u < kSplitLoads; ++u) {
+            const uint32_t j = b + u * kSplitThreads + threadIdx.x;
+            k[u] = j < n ? src[j] : ~0ull;
+        }
+#pragma unroll
+        for (int u = 0; u < kSplitLoads; ++u)
+            if (b + u * kSplitThreads + threadIdx.x < n) f(k[u]);
+    }
+}
+
+// One CTA per long list: a histogram over split_bin, bins gathered into segments by the
+// kSegTarget-entry stretch of the list their first entry falls into, and the entries scattered by
+// bin.  A segment holds fewer than kSegTarget entries plus its last bin, so it exceeds kListCap
+// only when one bin alone holds more than kSegTarget (the list sort then merges it in global
+// memory).
+__global__ void __launch_bounds__(kSplitThreads) k_split(const BinArgs A)
+{
+    __shared__ uint32_t s_bin[kSplitBins];
+    __shared__ uint32_t s_start[kSplitBins + 1];
+    __shared__ uint32_t s_warp[33];
+    __shared__ uint32_t s_base;
+    const int tid = threadIdx.x;
+    const uint32_t n_long = A.bin[kBinLong];
+    for (uint32_t l = blockIdx.x; l < n_long; l += gridDim.x) {
+        const uint32_t tile = A.order[l];
+        const uint2 rg = A.ranges[tile];
+        const uint32_t len = rg.y - rg.x;
+        const uint64_t *src = A.entries + rg.x;
+        __syncthreads();
+        for (int k = tid; k < kSplitBins; k += kSplitThreads) s_bin[k] = 0u;
+        __syncthreads();
+        for_each_key(src, len, [&](uint64_t e) { atomicAdd(&s_bin[split_bin(e)], 1u); });
+        __syncthreads();
+        uint32_t c[kBinsPer], sum = 0;
+#pragma unroll
+        for (int i = 0; i < kBinsPer; ++i) {
+            c[i] = s_bin[tid * kBinsPer + i];
+            sum += c[i];
+        }
+        uint32_t at = block_excl_scan<kSplitThreads>(sum, s_warp, static_cast<uint32_t *>(nullptr));
+        uint32_t pre[kBinsPer];
+#pragma unroll
+        for (int i = 0; i < kBinsPer; ++i) {
+            pre[i] = at;
+            s_bin[tid * kBinsPer + i] = at;   // the bin's first place, then its cursor
+            at += c[i];
+        }
+        __syncthreads();
+        // a segment starts at every bin whose first entry lies in another kSegTarget stretch than
+        // the previous bin's
+        uint32_t first[kBinsPer], ns = 0;
+#pragma unroll
+        for (int i = 0; i < kBinsPer; ++i) {
+            const int b = tid * kBinsPer + i;
+            const uint32_t before = b == 0 ? 0u : (i > 0 ? pre[i - 1] : s_bin[b - 1]);
+            first[i] = pre[i] < len &&
+                       (b == 0 || pre[i] / kSegTarget != before / kSegTarget) ? 1u : 0u;
+            ns += first[i];
+        }
+        __syncthreads();
+        uint32_t n_seg;
+        uint32_t q = block_excl_scan<kSplitThreads>(ns, s_warp, &n_seg);
+#pragma unroll
+        for (int i = 0; i < kBinsPer; ++i)
+            if (first[i]) s_start[q++] = pre[i];
+        if (tid == 0) {
+            s_start[n_seg] = len;
+            s_base = atomicAdd(A.bin + kBinSegments, n_seg);
+        }
+        __syncthreads();
+        for (uint32_t k = tid; k < n_seg; k += kSplitThreads)
+            A.segments[s_base + k] =
+                ListSegment{rg.x + s_start[k], s_start[k + 1] - s_start[k], tile};
+        for_each_key(src, len, [&](uint64_t e) {
+            const uint32_t o = atomicAdd(&s_bin[split_bin(e)], 1u);
+            A.entries2[rg.x + o] = e;
+        });
+    }
+}
+
+// ---------------------------------------------------------------------------------------------
+// list sort
+// ---------------------------------------------------------------------------------------------
+
+// one spare word per 16 keys: threads that walk runs a power of two apart spread over the banks
+__device__ __forceinline__ int pad(int i) { return i + (i >> 4); }
+
+template <int G>
+__device__ __forceinline__ void group_sync()
+{
+    if (G == 32) __syncwarp();
+    else __syncthreads();
+}
+
+__device__ __forceinline__ void order_pair(uint64_t &a, uint64_t &b)
+{
+    const uint64_t lo = a < b ? a : b, hi = a < b ? b : a;
+    a = lo;
+    b = hi;
+}
+
+// Batcher's odd-even merge sort of E keys in registers: phase p merges sorted runs of p keys, in
+// steps of comparison distance q = p, p / 2, ..., 1
+template <int E, int P, int Q>
+__device__ __forceinline__ void network(uint64_t (&k)[E])
+{
+    if constexpr (P < E) {
+#pragma unroll
+        for (int i = 0; i + Q < E; ++i)
+            if (i >= Q % P && (i - Q % P) / Q % 2 == 0 && i / (2 * P) == (i + Q) / (2 * P))
+                order_pair(k[i], k[i + Q]);
+        if constexpr (Q > 1) network<E, P, Q / 2>(k);
+        else network<E, 2 * P, 2 * P>(k);
+    }
+}
+
+// Sorts the n <= G * E keys src[0 .. n) into s (padded places), with G threads (a warp or the
+// CTA) of E keys each: every thread sorts its keys in registers (network), then
+// runs of E, 2E, ... keys are merged pairwise, each thread finding its E outputs by a binary
+// search along its diagonal (merge path).
+template <int E, int G>
+__device__ __forceinline__ void sort_keys(const uint64_t *src, int n, uint64_t *s, int g)
+{
+    uint64_t k[E];
+#pragma unroll
+    for (int i = 0; i < E; ++i) {   // coalesced read, then each thread's own run
+        const int j = g + i * G;
+        if (j < n) s[pad(j)] = src[j];
+    }
+    group_sync<G>();
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+        const int j = g * E + i;
+        k[i] = j < n ? s[pad(j)] : ~0ull;
+    }
+    network<E, 1, 1>(k);
+    group_sync<G>();
+#pragma unroll
+    for (int i = 0; i < E; ++i) s[pad(g * E + i)] = k[i];
+    group_sync<G>();
+    for (int w = E; w < n; w <<= 1) {
+        const int base = (g * E) & ~(2 * w - 1), diag = g * E - base;
+        if (base + w < n) {   // otherwise the run has no partner and stays
+            const int a0 = base, b0 = base + w;
+            int lo = diag > w ? diag - w : 0, hi = diag < w ? diag : w;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (s[pad(a0 + mid)] < s[pad(b0 + diag - 1 - mid)]) lo = mid + 1;
+                else hi = mid;
+            }
+            int i = lo, j = diag - lo;
+            uint64_t a = i < w ? s[pad(a0 + i)] : ~0ull, b = j < w ? s[pad(b0 + j)] : ~0ull;
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const bool left = a < b || j >= w;
+                k[e] = left ? a : b;
+                if (left) {
+                    ++i;
+                    a = i < w ? s[pad(a0 + i)] : ~0ull;
+                } else {
+                    ++j;
+                    b = j < w ? s[pad(b0 + j)] : ~0ull;
+                }
+            }
+        }
+        group_sync<G>();
+        if (base + w < n) {
+#pragma unroll
+            for (int e = 0; e < E; ++e) s[pad(g * E + e)] = k[e];
+        }
+        group_sync<G>();
+    }
+}
+
+// an entry of the list: pair id, pixel rectangle inside the tile, blocks met
+struct ListTile {
+    int rb, cb, cols;   // the tile's first row and column, the image's width
+};
+
+__device__ __forceinline__ void write_entry(const BinArgs &A, uint32_t at, uint64_t key,
+                                            const ListTile &t)
+{
+    const uint32_t p = static_cast<uint32_t>(key);
+    const uint32_t r = tile_local_rect(unpack_pixel_rect(A.prect[p]), t.rb, t.cb, t.cols, A.tile_h,
+                                       A.tile_w);
+    reinterpret_cast<uint2 *>(A.entries)[at] = make_uint2(p, r);
+    A.entry_blocks[at] =
+        static_cast<uint8_t>(rect_blocks(r & ~kRectFlip, A.tile_h, A.tile_w));
+}
+
+__device__ __forceinline__ ListTile list_tile(const BinArgs &A, uint32_t tile)
+{
+    const TileInfo &ti = A.tiles[tile];
+    return ListTile{ti.tr * A.tile_h, ti.tc * A.tile_w, ti.cols};
+}
+
+// bins of a list: two to four a key, 16-bit counters in pairs
+constexpr int kMaxBins = 2 * kListCap;
+// lists with a bin above this are merge sorted: an entry is compared with its whole bin
+constexpr int kMaxInBin = 32;
+
+struct ListShared {
+    uint64_t key[kListCap + kListCap / 16];
+    uint32_t bins[kMaxBins / 2 + kMaxBins / 64];
+    uint32_t item, lo, hi, worst;
+    uint32_t warp[33];
+};
+
+// place of a counter word: one spare per 32, so that threads scanning runs of words spread over
+// the banks
+__device__ __forceinline__ uint32_t bin_word(uint32_t w) { return w + (w >> 5); }
+
+// exclusive scan of the 16-bit counters packed two to a word, in place, by a group of G threads
+template <int G>
+__device__ __forceinline__ uint32_t scan_bins(uint32_t *bins, int words, uint32_t *s_warp, int g)
+{
+    // each thread takes a run of consecutive words; returns the largest counter it saw
+    const int per = (words + G - 1) / G;
+    uint32_t sum = 0, worst = 0;
+    for (int i = 0; i < per; ++i) {
+        const int w = g * per + i;
+        if (w < words) {
+            const uint32_t c = bins[bin_word(w)], a = c & 0xFFFFu, b = c >> 16;
+            sum += a + b;
+            worst = max(worst, max(a, b));
+        }
+    }
+    uint32_t at;
+    if (G == 32) {
+        uint32_t x = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(kFull, x, o);
+            if (g >= o) x += y;
+        }
+        at = x - sum;
+    } else {
+        at = block_excl_scan<G>(sum, s_warp, static_cast<uint32_t *>(nullptr));
+    }
+    for (int i = 0; i < per; ++i) {
+        const int w = g * per + i;
+        if (w < words) {
+            const uint32_t c = bins[bin_word(w)], a = c & 0xFFFFu, b = c >> 16;
+            bins[bin_word(w)] = at | (at + a) << 16;
+            at += a + b;
+        }
+    }
+    return worst;
+}
+
+__device__ __forceinline__ uint32_t add_bin(uint32_t *bins, uint32_t b)
+{
+    const int sh = (b & 1u) << 4;
+    return (atomicAdd(bins + bin_word(b >> 1), 1u << sh) >> sh) & 0xFFFFu;
+}
+
+__device__ __forceinline__ uint32_t get_bin(const uint32_t *bins, uint32_t b)
+{
+    return (bins[bin_word(b >> 1)] >> ((b & 1u) << 4)) & 0xFFFFu;
+}
+
+// Sorts one list of n keys and writes its entries, with a group of G threads (a warp or the CTA).
+// The keys go into two to four bins a key, linear in the range key's bits between the list's
+// smallest and largest (floats of one sign order as integers), are laid out by bin, and each is
+// then ranked against the other keys of its bin -- one or two on lists whose ranges spread.  A
+// list with a bin above kMaxInBin (a wall behind a near object) is merge sorted.  The keys are
+// read three times rather than held: they stay in L1, and short loops keep the code in the
+// instruction cache.
+template <int G>
+__device__ __forceinline__ void sort_list(const BinArgs &A, const uint64_t *src, uint32_t start,
+                                          int n, uint32_t tile, uint64_t *key, uint32_t *bins,
+                                          ListShared &sh, int g)
+{
+    src += start;
+    const int log_bins = min(32 - __clz(n) + 1, G == 32 ? 9 : 13);
+    const int words = 1 << (log_bins - 1);
+    for (int w = g; w < words; w += G) bins[bin_word(w)] = 0u;
+    const uint32_t *hi_word = reinterpret_cast<const uint32_t *>(src) + 1;   // the range keys
+    uint32_t lo = kFull, hi = 0u;
+#pragma unroll 4
+    for (int j = g; j < n; j += G) {
+        const uint32_t k = hi_word[2 * j];
+        lo = min(lo, k);
+        hi = max(hi, k);
+    }
+    lo = __reduce_min_sync(kFull, lo);
+    hi = __reduce_max_sync(kFull, hi);
+    if (G > 32) {
+        if (g == 0) {
+            sh.lo = kFull;
+            sh.hi = 0u;
+            sh.worst = 0u;
+        }
+        __syncthreads();
+        if ((g & 31) == 0) {
+            atomicMin(&sh.lo, lo);
+            atomicMax(&sh.hi, hi);
+        }
+        __syncthreads();
+        lo = sh.lo;
+        hi = sh.hi;
+    } else {
+        __syncwarp();
+    }
+    const int down = max(0, 32 - __clz(hi - lo) - log_bins);
+#pragma unroll 4
+    for (int j = g; j < n; j += G) add_bin(bins, (hi_word[2 * j] - lo) >> down);
+    group_sync<G>();
+    uint32_t worst = __reduce_max_sync(kFull, scan_bins<G>(bins, words, sh.warp, g));
+    if (G > 32) {
+        if ((g & 31) == 0) atomicMax(&sh.worst, worst);
+        __syncthreads();
+        worst = sh.worst;
+    } else {
+        __syncwarp();
+    }
+    const ListTile t = list_tile(A, tile);
+    if (worst <= kMaxInBin) {
+#pragma unroll 4
+        for (int j = g; j < n; j += G) {
+            const uint64_t k = src[j];
+            key[add_bin(bins, (static_cast<uint32_t>(k >> 32) - lo) >> down)] = k;
+        }
+        group_sync<G>();   // every counter now stands at its bin's end
+        for (int j = g; j < n; j += G) {
+            const uint64_t k = key[j];
+            const uint32_t b = (static_cast<uint32_t>(k >> 32) - lo) >> down;
+            const int b0 = b == 0 ? 0 : static_cast<int>(get_bin(bins, b - 1));
+            const int b1 = static_cast<int>(get_bin(bins, b));
+            int at = b0;
+            if (b1 - b0 > 1)
+                for (int q = b0; q < b1; ++q) at += key[q] < k ? 1 : 0;
+            write_entry(A, start + at, k, t);
+        }
+    } else {
+        constexpr int E = G == 32 ? kWarpCap / 32 : kMaxItems;
+        sort_keys<E, G>(src, n, key, g);
+        for (int j = g; j < n; j += G) write_entry(A, start + j, key[pad(j)], t);
+    }
+    group_sync<G>();
+}
+
+// A segment above kListCap (more than kSegTarget primitives of a tile within one bin of range):
+// chunks of kListCap sorted in place, then merged pairwise between the two buffers, 16 outputs a
+// thread by merge path straight from global memory.
+__device__ __noinline__ void sort_oversized(const BinArgs &A, const ListSegment &sg, uint64_t *s)
+{
+    const int tid = threadIdx.x;
+    uint64_t *in = A.entries2 + sg.start, *out = A.entries + sg.start;
+    for (uint32_t c = 0; c < sg.len; c += kListCap) {
+        const int n = static_cast<int>(sg.len - c < kListCap ? sg.len - c : kListCap);
+        sort_keys<kMaxItems, kListThreads>(in + c, n, s, tid);
+        for (int j = tid; j < n; j += kListThreads) in[c + j] = s[pad(j)];
+        __syncthreads();
+    }
+    const int64_t len = sg.len;
+    for (int64_t w = kListCap; w < len; w <<= 1) {
+        for (int64_t d = static_cast<int64_t>(tid) * kMaxItems; d < len;
+             d += kListThreads * kMaxItems) {
+            const int64_t base = d / (2 * w) * (2 * w), diag = d - base;
+            const int64_t la = len - base < w ? len - base : w;
+            const int64_t lb = len - base - la < w ? len - base - la : w;
+            const uint64_t *a = in + base, *b = in + base + la;
+            int64_t lo = diag > lb ? diag - lb : 0, hi = diag < la ? diag : la;
+            while (lo < hi) {
+                const int64_t mid = (lo + hi) >> 1;
+                if (a[mid] < b[diag - 1 - mid]) lo = mid + 1;
+                else hi = mid;
+            }
+            int64_t i = lo, j = diag - lo;
+            for (int e = 0; e < kMaxItems && i + j < la + lb; ++e) {
+                const bool left = j >= lb || (i < la && a[i] < b[j]);
+                out[d + e] = left ? a[i++] : b[j++];
+            }
+        }
+        __syncthreads();
+        uint64_t *t = in;
+        in = out;
+        out = t;
+    }
+    const ListTile t = list_tile(A, sg.tile);
+    for (uint32_t j = tid; j < sg.len; j += kListThreads)
+        write_entry(A, sg.start + j, in[j], t);
+    __syncthreads();
+}
+
+// Persistent: the CTAs take segments and lists of 256 entries and more, longest first; then their
+// warps take the shorter lists.
+__global__ void __launch_bounds__(kListThreads, kListCtas) k_lists(const BinArgs A)
+{
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    ListShared &sh = *reinterpret_cast<ListShared *>(s_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t n_long = A.bin[kBinLong], n_seg = A.bin[kBinSegments];
+    const uint32_t n_mid = A.bin[kBinMid];
+    const uint32_t n_cta = n_seg + (n_mid - n_long);
+    for (uint32_t item = blockIdx.x; item < n_cta;) {
+        ListSegment sg;
+        const uint64_t *src = A.entries;
+        if (item < n_seg) {
+            sg = A.segments[item];
+            src = A.entries2;
+        } else {
+            sg.tile = A.order[n_long + item - n_seg];
+            const uint2 rg = A.ranges[sg.tile];
+            sg.start = rg.x;
+            sg.len = rg.y - rg.x;
+        }
+        if (sg.len > kListCap)
+            sort_oversized(A, sg, sh.key);
+        else if (sg.len > 0)
+            sort_list<kListThreads>(A, src, sg.start, static_cast<int>(sg.len), sg.tile, sh.key,
+                                    sh.bins, sh, tid);
+        if (tid == 0) sh.item = atomicAdd(A.bin + kBinQueueSeg, 1u) + gridDim.x;
+        __syncthreads();
+        item = sh.item;
+        __syncthreads();
+    }
+    uint64_t *key = sh.key + warp * (kWarpCap + kWarpCap / 16);
+    uint32_t *bins = sh.bins + warp * (kWarpCap + kWarpCap / 32);
+    for (uint32_t item = n_mid + blockIdx.x * kListWarps + warp; item < A.n_tiles;
+         item += gridDim.x * kListWarps) {
+        const uint32_t tile = A.order[item];
+        const uint2 rg = A.ranges[tile];
+        if (rg.y > rg.x)
+            sort_list<32>(A, A.entries, rg.x, static_cast<int>(rg.y - rg.x), tile, key, bins, sh,
+                          lane);
+    }
+}
+
+// blocks a CTA counts or emits: at most kBinCtas CTAs per SM over the drawn views, at least
+// kMinChunk primitives (below that the CTA's counters cost more than its pairs)
+dim3 chunk_grid(BinArgs &a)
+{
+    a.block_prims = block_prims(a.n);
+    a.blocks = static_cast<int>(project_blocks(a.n));
+    const int64_t c = int64_t{a.blocks} * a.max_active / (int64_t{kBinCtas} * a.sms) + 1;
+    const int64_t least = kMinChunk / a.block_prims;
+    a.chunk = static_cast<int>(c < least ? least : c);
+    return dim3(static_cast<unsigned>((a.blocks + a.chunk - 1) / a.chunk),
+                static_cast<unsigned>(a.n_views));
 }
 
 }  // namespace
 
-cudaError_t launch_order_tiles(const uint2 *ranges, int64_t n_tiles, uint32_t *order,
-                               cudaStream_t st)
+// k_lists' shared memory is above the 48 KB static limit: allow it once
+cudaError_t prepare_lists()
 {
-    if (n_tiles <= 0) return cudaSuccess;
-    k_order_tiles<<<1, 1024, 0, st>>>(ranges, n_tiles, order);
-    return cudaGetLastError();
+    static const cudaError_t e = cudaFuncSetAttribute(
+        k_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(ListShared)));
+    return e;
 }
 
-cudaError_t radix_sort_pairs(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint32_t *vals_alt,
-                             const uint32_t *d_count, int64_t max_n, int bits, uint32_t *tmp_hist,
-                             uint32_t **keys_out, uint32_t **vals_out, cudaStream_t st,
-                             const uint32_t *d_count_kept, const uint64_t *aux_in,
-                             uint64_t *aux_out)
+int bin_launches(int64_t n) { return n >= kListCap ? 5 : 4; }
+
+cudaError_t launch_bin_counts(const BinArgs &args, cudaStream_t st)
 {
-    uint32_t *kin = keys, *vin = vals, *kout = keys_alt, *vout = vals_alt;
-    if (max_n > 0) {
-        for (int shift = 0; shift < bits; shift += 8) {
-            uint32_t *dtot = tmp_hist + kSortGrid * kRadix;
-            // with d_count_kept, the first pass drops the key 0xFFFFFFFF and the later passes
-            // sort the d_count_kept items left
-            const int drop = d_count_kept && shift == 0;
-            const uint32_t *cnt = d_count_kept && shift > 0 ? d_count_kept : d_count;
-            k_upsweep<<<kSortGrid, kThreads, 0, st>>>(kin, cnt, max_n, shift, drop, tmp_hist);
-            k_scan_digits<<<kRadix / 8, 256, 0, st>>>(tmp_hist, kSortGrid, dtot);
-            const bool last = shift + 8 >= bits;
-            k_downsweep<<<kSortGrid, kThreads, 0, st>>>(kin, vin, kout, vout, cnt, max_n, shift,
-                                                        drop, tmp_hist, dtot, aux_in,
-                                                        last ? aux_out : nullptr);
-            uint32_t *t = kin;
-            kin = kout;
-            kout = t;
-            t = vin;
-            vin = vout;
-            vout = t;
-        }
+    BinArgs a = args;
+    if (a.n > 0) {
+        const dim3 grid = chunk_grid(a);
+        if (a.max_view_tiles <= kMaxSharedTiles)
+            k_count<true><<<grid, kChunkThreads, 4 * a.max_view_tiles, st>>>(a);
+        else
+            k_count<false><<<grid, kChunkThreads, 0, st>>>(a);
     }
-    *keys_out = kin;
-    *vals_out = vin;
+    k_layout<<<1, kLayoutThreads, 0, st>>>(a.tile_count, a.n_tiles, a.max_pairs, a.ranges, a.order,
+                                           a.d_count, a.status, a.bin);
     return cudaGetLastError();
 }
 
-cudaError_t launch_emit(const uint32_t *sorted_pair_ids, const uint64_t *sorted_trect,
-                        int64_t n_pairs_total, const uint32_t *n_valid, const ViewDesc *views,
-                        int64_t n_per_view, uint32_t *block_sums, uint32_t *tile_keys,
-                        uint32_t *tile_vals, int64_t max_pairs, uint32_t *d_count,
-                        uint32_t *status, cudaStream_t st)
+cudaError_t launch_emit(const BinArgs &args, cudaStream_t st)
 {
-    k_count_sums<<<kScanGrid, kThreads, 0, st>>>(sorted_trect, n_pairs_total, n_valid, block_sums);
-    k_scan_sums<<<1, 1024, 0, st>>>(block_sums, kScanGrid, max_pairs, d_count, status);
-    k_emit<<<kScanGrid, kThreads, 0, st>>>(sorted_pair_ids, sorted_trect, n_pairs_total, n_valid,
-                                           views, n_per_view, block_sums, tile_keys, tile_vals,
-                                           max_pairs);
+    BinArgs a = args;
+    if (a.n <= 0) return cudaSuccess;
+    const dim3 grid = chunk_grid(a);
+    if (a.max_view_tiles <= kMaxSharedTiles)
+        k_emit<true><<<grid, kChunkThreads, 4 * a.max_view_tiles, st>>>(a);
+    else
+        k_emit<false><<<grid, kChunkThreads, 0, st>>>(a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_ranges(const uint32_t *tile_keys, const uint32_t *tile_vals,
-                          const uint64_t *prect, const TileInfo *tiles, int tile_h, int tile_w,
-                          const uint32_t *d_count, int64_t max_pairs, uint2 *ranges,
-                          int64_t n_tiles, uint32_t *entry_rect, uint8_t *entry_blocks,
-                          cudaStream_t st)
+cudaError_t launch_lists(const BinArgs &a, cudaStream_t st)
 {
-    cudaError_t e = cudaMemsetAsync(ranges, 0, sizeof(uint2) * static_cast<size_t>(n_tiles), st);
+    if (a.n <= 0) return cudaSuccess;
+    const cudaError_t e = prepare_lists();
     if (e != cudaSuccess) return e;
-    k_ranges<<<kRangesGrid, 256, 0, st>>>(tile_keys, tile_vals, prect, tiles, tile_h, tile_w,
-                                            d_count, max_pairs, ranges, entry_rect,
-                                            entry_blocks);
+    // a list holds each primitive once: below kListCap primitives none is long
+    if (a.n >= kListCap) k_split<<<2 * a.sms, kSplitThreads, 0, st>>>(a);
+    k_lists<<<kListCtas * a.sms, kListThreads, sizeof(ListShared), st>>>(a);
     return cudaGetLastError();
 }
 

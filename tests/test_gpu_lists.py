@@ -1,0 +1,77 @@
+"""The per-tile lists at the sizes where the list sort changes its path: one warp or one CTA per
+list, each number of keys a thread, lists cut into segments, segments that stay too large because
+their primitives share a range, and rectangles counted and emitted by a whole warp.  Lists and
+records bit-exact against the oracle.  Marked gpu."""
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2503_17491_gb300 import scenes
+from gpu_common import check_lists, make_ctx, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _build():
+    oracle.build()
+
+
+def _one_tile(n, ranges, seed):
+    """n primitives of about two columns' width in the directions of one tile's inner pixels, at
+    the given ranges: each meets that tile and no other."""
+    rng = np.random.default_rng(seed)
+    g = math.pi - 2 * math.pi * (24 + rng.uniform(-4, 4, n)) / 64
+    th = math.radians(10) * rng.uniform(-0.3, 0.3, n)
+    p = np.stack([np.cos(th) * np.cos(g), np.cos(th) * np.sin(g), np.sin(th)], 1) * ranges[:, None]
+    pl, q, ls = scenes.gaussians_on(p, -p, rng, jitter=0.0)
+    ls[:] = np.log(0.04 * ranges)[:, None]
+    view = scenes.View(np.eye(4), 16, 64, scenes.deg(-10), scenes.deg(10))
+    return scenes.Scene(f"one_tile{n}", pl, q, ls, [view])
+
+
+def _check(s, tile=(16, 16)):
+    ctx = make_ctx(s.n, s.views, tile)
+    ctx.render(*to_dev(s))
+    assert ctx.status() == 0
+    m = check_lists(ctx, s, s.views, tile)
+    r = ctx.sorted_lists()[2].astype(np.int64)
+    return m, int((r[:, 1] - r[:, 0]).max())
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 128, 129, 255, 256, 257, 1024, 1025, 2048, 2049,
+                               4095, 4096, 4097, 8192, 20_001])
+def test_list_lengths(n):
+    rng = np.random.default_rng(n)
+    assert _check(_one_tile(n, rng.uniform(2.0, 60.0, n), n))[1] == n
+
+
+@pytest.mark.parametrize("n,kind", [(300, "equal"), (4096, "equal"), (9000, "equal"),
+                                    (9000, "wall"), (20_000, "two")])
+def test_shared_ranges(n, kind):
+    """Ties are broken by the primitive id, and a bin of the segmentation that holds more than a
+    segment's worth is merged: every primitive at one place, a thin wall behind a near object, and
+    two places."""
+    rng = np.random.default_rng(n)
+    r = np.full(n, 7.0)
+    if kind == "wall":
+        r = 30.0 + 1e-4 * rng.uniform(0, 1, n)
+        r[:5] = rng.uniform(0.5, 2.0, 5)
+    s = _one_tile(n, r, 3)
+    if kind != "wall":
+        s.pos_logit[:, :3] = s.pos_logit[0, :3]
+    if kind == "two":
+        s.pos_logit[::2, :3] *= 1.5
+    assert _check(s)[1] == n
+
+
+@pytest.mark.parametrize("tile", [(16, 16), (8, 32), (32, 8), (4, 64)])
+def test_wide_rectangles(tile):
+    """Near, large primitives beside small ones: rectangles of one tile up to whole tile rows and
+    every tile, across the seam, on a ragged image."""
+    s = scenes.tiny_scene(700, 21, rows=45, cols=333, fov_deg=40, dist=(0.4, 6.0),
+                          log_scale=(-3.0, 0.7))
+    m, _ = _check(s, tile)
+    assert m > 10 * s.n
