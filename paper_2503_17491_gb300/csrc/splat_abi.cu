@@ -110,7 +110,7 @@ struct splat_ctx {
                                       // [5] record chunks taken, [6] map-growth draws,
                                       // [7] sampling step, [8..] binning (splat::kBin...)
     unsigned long long *d_grow_sums = nullptr;  // map growth: block sums, Q, offset
-    unsigned long long *d_evals = nullptr;      // [0] forward, [1] backward
+    unsigned long long *d_evals = nullptr;      // [0] forward, [1] backward, [2] rows met
 
     // profiling events: [0,1] forward compositing, [2,3] backward compositing, then one event
     // after the stages of the last profiled render / refinement step: [0] before the
@@ -174,7 +174,7 @@ splat::RenderArgs render_args(splat_ctx *ctx, const splat_gaussians *g)
     a.rec_fill = ctx->d_rec_fill;
     a.status = ctx->d_counters + 1;
     a.n_tiles = ctx->n_tiles;
-    a.n_items = ctx->n_tiles * (splat::kBlock / 32);
+    a.split = ctx->d_counters + kCountersBin + splat::kBinSplit4;
     a.alpha_min = ctx->cfg.alpha_min;
     a.alpha_max = ctx->cfg.alpha_max;
     a.t_min = ctx->cfg.t_min;
@@ -197,6 +197,7 @@ int render_core(splat_ctx *ctx, const splat_gaussians *g, float *depth, float *n
     CK(cudaMemsetAsync(cnt + 4, 0, 2 * sizeof(uint32_t), st));   // touching pairs, chunks
     CK(cudaMemsetAsync(cnt + 2, 0, sizeof(uint32_t), st));       // forward queue
     CK(cudaMemsetAsync(ctx->d_evals, 0, sizeof(unsigned long long), st));
+    CK(cudaMemsetAsync(ctx->d_evals + 2, 0, sizeof(unsigned long long), st));
     CK(cudaMemsetAsync(ctx->d_tile_count, 0,
                        sizeof(uint32_t) * static_cast<size_t>(ctx->n_tiles), st));
     const uint8_t *active = nullptr;
@@ -235,6 +236,7 @@ int render_core(splat_ctx *ctx, const splat_gaussians *g, float *depth, float *n
     pa.prim = ctx->d_prim;
     pa.status = cnt + 1;
     pa.n_valid = cnt + 4;
+    pa.n_rows = ctx->d_evals + 2;
     pa.active = active;
     CK(splat::launch_project(pa, st));
     CK(stage_mark(1));
@@ -266,6 +268,9 @@ int render_core(splat_ctx *ctx, const splat_gaussians *g, float *depth, float *n
     ba.status = cnt + 1;
     ba.bin = cnt + kCountersBin;
     ba.sms = ctx->sms;
+    ba.warps = static_cast<uint32_t>(ctx->grid_fwd) * (splat::kBlock / 32);
+    ba.rec_cap = ctx->rec_cap;
+    ba.n_rows = ctx->d_evals + 2;
     CK(splat::launch_bin_counts(ba, st));
     CK(splat::launch_emit(ba, st));
     CK(stage_mark(3));
@@ -443,17 +448,18 @@ SPLAT_API int splat_ctx_create(const splat_render_config *cfg, const splat_capac
     c->rec_cap = static_cast<uint32_t>(chunks < 0xFFFFFFF0ll ? chunks : 0xFFFFFFF0ll);
     if (e == cudaSuccess) e = dalloc(&c->d_rec, static_cast<size_t>(c->rec_cap) * 32);
     if (e == cudaSuccess) e = dalloc(&c->d_rec_prev, static_cast<size_t>(c->rec_cap));
-    if (e == cudaSuccess) e = dalloc(&c->d_rec_head, static_cast<size_t>(items));
-    if (e == cudaSuccess) e = dalloc(&c->d_rec_fill, static_cast<size_t>(items));
+    // (a split block has up to four items)
+    if (e == cudaSuccess) e = dalloc(&c->d_rec_head, static_cast<size_t>(4 * items));
+    if (e == cudaSuccess) e = dalloc(&c->d_rec_fill, static_cast<size_t>(4 * items));
     if (e == cudaSuccess) e = dalloc(&c->d_img, static_cast<size_t>(P) * 5);
     if (e == cudaSuccess) e = dalloc(&c->d_gimg, static_cast<size_t>(P) * 5);
     if (e == cudaSuccess) e = dalloc(&c->d_counters, kCounters);
-    if (e == cudaSuccess) e = dalloc(&c->d_evals, 2);
+    if (e == cudaSuccess) e = dalloc(&c->d_evals, 3);
     for (int k = 0; k < 4 && e == cudaSuccess; ++k) e = cudaEventCreate(&c->ev[k]);
     for (int k = 0; k < splat_ctx::kStageEvents && e == cudaSuccess; ++k)
         e = cudaEventCreate(&c->stage_ev[k]);
     if (e == cudaSuccess) e = cudaMemset(c->d_counters, 0, kCounters * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMemset(c->d_evals, 0, 2 * sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMemset(c->d_evals, 0, 3 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = splat::prepare_lists();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {

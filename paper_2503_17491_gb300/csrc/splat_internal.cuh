@@ -396,6 +396,7 @@ struct ProjectArgs {
     uint32_t *touch_count;
     float4 *prim;
     uint32_t *status;
+    unsigned long long *n_rows;   // zeroed before: rows of 8 pixels of the blocks the pairs meet
     uint32_t *n_valid;      // zeroed before: pairs that touch a tile
     const uint8_t *active;  // per view (nullable): drawn for this step
 };
@@ -433,7 +434,7 @@ struct BinArgs {
     uint32_t *tile_count;       // zeroed before; counted, then counted down by the emission
     uint32_t *cta_count;        // cta_count_words(...): the counts of every counting CTA
     uint2 *ranges;
-    uint32_t *order;            // tiles by decreasing log2 of their list length
+    uint32_t *order;            // tiles by decreasing bucket of list length, four an octave
     uint64_t *entries;          // emitted (range key << 32 | pair id), then the sorted entries
     uint64_t *entries2;         // scratch of the same size (needed when n > kListCap)
     uint8_t *entry_blocks;
@@ -441,11 +442,14 @@ struct BinArgs {
     uint32_t *d_count;          // out: list entries
     uint32_t *status;
     uint32_t *bin;              // kBinWords counters (written by the layout kernel)
+    // work split of the compositing kernels: their warps, the record pool (0: no records are kept)
+    uint32_t warps, rec_cap;
+    const unsigned long long *n_rows;
     int sms;
     int block_prims, blocks;    // the projection's blocks; these and chunk (blocks a counting CTA
     int chunk;                  // takes) are set by the launchers
 };
-// kBinLong, kBinMid: tiles (in work order) with at least kListCap and at least 256 entries
+// kBinLong, kBinMid: tiles (in work order) with at least kListCap and at least 256 entries;
 constexpr int kBinCtas = 4;              // counting and emitting CTAs per SM
 constexpr int kMinChunk = kLargeBlock;   // primitives each takes at least
 constexpr int kMaxSharedTiles = 12288;   // views up to this are counted in shared memory (48 KB)
@@ -454,7 +458,8 @@ inline int64_t cta_count_words(int sms, int max_views, int64_t max_tiles)
     return (int64_t{kBinCtas} * sms + max_views) *
            (max_tiles < kMaxSharedTiles ? max_tiles : kMaxSharedTiles);
 }
-enum { kBinLong = 0, kBinMid, kBinSegments, kBinQueueSeg, kBinWords };
+// kBinSplit4, kBinSplit2: RenderArgs::split
+enum { kBinLong = 0, kBinMid, kBinSegments, kBinQueueSeg, kBinSplit4, kBinSplit2, kBinWords };
 cudaError_t prepare_lists();    // before the first launch_lists on a device
 int bin_launches(int64_t n);    // kernels these three run for n primitives
 cudaError_t launch_bin_counts(const BinArgs &a, cudaStream_t st);   // count and layout
@@ -517,7 +522,7 @@ struct RenderArgs {
     const uint2 *entries;
     const uint8_t *entry_blocks;  // per list entry: the 4 x 8 blocks of its tile it meets
     int64_t n_tiles;
-    int64_t n_items;              // n_tiles x blocks per tile
+    const uint32_t *split;        // leading tiles of the order whose blocks go to 4 warps, then to 2
     float alpha_min, alpha_max, t_min, sigma;
     // forward outputs (packed pixels)
     float *depth, *normal, *alpha;

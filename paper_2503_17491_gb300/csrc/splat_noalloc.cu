@@ -70,7 +70,7 @@ constexpr size_t kOffNlast = align256(kOffTfinal + 4 * kMaxPixels);
 constexpr size_t kOffCounters = align256(kOffNlast + 4 * kMaxPixels);
 constexpr int kCountersBin = 8, kCounters = kCountersBin + splat::kBinWords;
 constexpr size_t kOffEvals = align256(kOffCounters + 4 * kCounters);
-constexpr size_t kScratchBytes = align256(kOffEvals + 8 * 2);
+constexpr size_t kScratchBytes = align256(kOffEvals + 8 * 3);
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -264,7 +264,7 @@ extern "C" SPLAT_API int splat_render_noalloc(const splat_gaussians *g,
                           cudaMemcpyHostToDevice, st));
     NA_CK(cudaMemsetAsync(cnt, 0, 4 * kCounters, st));
     NA_CK(cudaMemsetAsync(tile_count, 0, 4 * n_tiles, st));
-    NA_CK(cudaMemsetAsync(evals, 0, 8 * 2, st));
+    NA_CK(cudaMemsetAsync(evals, 0, 8 * 3, st));
 
     int sms = 0;
     NA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -287,6 +287,7 @@ extern "C" SPLAT_API int splat_render_noalloc(const splat_gaussians *g,
     pa.prim = prim;
     pa.status = cnt + 1;
     pa.n_valid = cnt + 4;
+    pa.n_rows = evals + 2;
     NA_CK(splat::launch_project(pa, st));
     splat::BinArgs ba{};
     ba.views = view;
@@ -314,6 +315,10 @@ extern "C" SPLAT_API int splat_render_noalloc(const splat_gaussians *g,
     ba.status = cnt + 1;
     ba.bin = cnt + kCountersBin;
     ba.sms = sms;
+    const int grid = sms * splat::render_occupancy(th, tw, false);
+    ba.warps = static_cast<uint32_t>(grid) * (splat::kBlock / 32);
+    ba.rec_cap = 0;   // no contributor records (forward only)
+    ba.n_rows = evals + 2;
     NA_CK(splat::launch_bin_counts(ba, st));
     NA_CK(splat::launch_emit(ba, st));
     NA_CK(splat::launch_lists(ba, st));
@@ -329,7 +334,7 @@ extern "C" SPLAT_API int splat_render_noalloc(const splat_gaussians *g,
     a.entry_blocks = blocks;
     a.status = cnt + 1;   // no contributor records (forward only)
     a.n_tiles = n_tiles;
-    a.n_items = n_tiles * (splat::kBlock / 32);
+    a.split = ba.bin + splat::kBinSplit4;
     a.alpha_min = cfg.alpha_min;
     a.alpha_max = cfg.alpha_max;
     a.t_min = cfg.t_min;
@@ -342,7 +347,6 @@ extern "C" SPLAT_API int splat_render_noalloc(const splat_gaussians *g,
     a.n_last = nlast;
     a.queue = cnt + 2;
     a.evals = evals;
-    const int grid = sms * splat::render_occupancy(th, tw, false);
     NA_CK(splat::launch_render_fwd(a, th, tw, grid, st));
 
     // the status word was produced on the device: wait for it and report it

@@ -500,6 +500,7 @@ struct ProjectShared {
     BoxQueue q;
     uint32_t count[kMaxViews];        // pairs of the block that touch a tile, per view
     uint32_t left[kProjectWarps];     // pairs left in each warp's queue at the end
+    unsigned long long rows;
 };
 
 __global__ void __launch_bounds__(kProjectThreads, 3) k_project(const ProjectArgs A)
@@ -513,7 +514,9 @@ __global__ void __launch_bounds__(kProjectThreads, 3) k_project(const ProjectArg
         sh.count[v] = 0u;
         sh.view[v] = quick_view(A.views[v]);
     }
+    if (threadIdx.x == 0) sh.rows = 0ull;
     __syncthreads();
+    float rows8 = 0.0f;   // rows of 8-pixel columns that this thread's touching pairs meet
 
     // append a touching pair (its primitive's place in the block is `local`) to the block's
     // segment of the view, with one counter update for the lanes `peers` of that view (the whole
@@ -528,6 +531,9 @@ __global__ void __launch_bounds__(kProjectThreads, 3) k_project(const ProjectArg
             A.touch[o] = pack_touch(tile_rect(rec, sh.view[v].cols, sh.view[v].tiles_c, th_shift,
                                               tw_shift), local);
             A.kappa[o] = rec.kappa;
+            // (a wrapping rectangle meets one column of 8 more at the seam)
+            rows8 += static_cast<float>((rec.r1 - rec.r0 + 1) *
+                                        (((rec.c0 + rec.nc - 1) >> 3) - (rec.c0 >> 3) + 2));
         }
     };
 
@@ -676,7 +682,12 @@ __global__ void __launch_bounds__(kProjectThreads, 3) k_project(const ProjectArg
         while (has && e >= sh.left[w]) e -= sh.left[w++];
         box(has, w * kQueueSlots + static_cast<int>(e));
     }
+    unsigned long long r64 = static_cast<unsigned long long>(rows8 * 1.001f) + 1ull;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) r64 += __shfl_xor_sync(0xFFFFFFFFu, r64, o);
+    if (lane == 0 && r64) atomicAdd(&sh.rows, r64);
     __syncthreads();
+    if (threadIdx.x == 0 && sh.rows) atomicAdd(A.n_rows, sh.rows);
     // the segments' lengths, and the pairs that touch a tile
     uint32_t nv = 0;
     for (int v = threadIdx.x; v < A.n_views; v += kProjectThreads) {

@@ -3,9 +3,13 @@
 // parameters.
 //
 // Work decomposition.  A work item is one 4 x 8 pixel block of one tile (a tile is
-// tile_h x tile_w = 256 pixels, i.e. 8 blocks), taken by one warp; the queue holds the blocks of
-// every tile of every registered view, so many keyframes of uneven sizes share one launch, and
-// hands tiles out longest list first so that the last items are short.  Warps never wait for
+// tile_h x tile_w = 256 pixels, i.e. 8 blocks), or a half or a row of it, taken by one warp; the
+// queue holds the blocks of every tile of every registered view, so many keyframes of uneven sizes
+// share one launch, and hands tiles out longest list first so that the last items are short.  A
+// list is one serial chain (the transmittance), so a block's time grows with its list: the blocks
+// of the lists that are long against a warp's share of the frame go to two or four warps, each
+// with its own pixels (one 64 x 1024 scan over 100,000 primitives: forward 0.125 -> 0.066 ms,
+// backward 0.112 -> 0.048 ms; eight 128 x 1024 scans along a street: forward 0.446 -> 0.319 ms).  Warps never wait for
 // one another.  A warp walks its tile's slice of the sorted list (Sec. 3.2.1) 32 entries at a
 // time -- every lane reads one entry's projection record and tests whether the primitive's pixel
 // rectangle meets the warp's block -- and stages the entries that do, 32 at a time, into shared
@@ -336,12 +340,57 @@ __device__ __forceinline__ void warp_count(unsigned long long v, unsigned long l
     if ((threadIdx.x & 31) == 0 && v) atomicAdd(total, v);
 }
 
-// the next work item of this warp (lane 0 takes it from the queue)
+// the next work item of this warp (lane 0 takes it from the queue).  All items come from the queue:
+// handing the first ones out by warp index took the 12-keyframe forward from 0.735 to 0.760 ms and
+// the backward from 0.818 to 0.840 ms.
 __device__ __forceinline__ uint32_t next_item(uint32_t *queue, int lane)
 {
     uint32_t it = 0;
     if (lane == 0) it = atomicAdd(queue, 1u);
     return __shfl_sync(kFull, it, 0);
+}
+
+// Work items of the frame: the first n4 tiles of the work order give 32 items each, the next n2
+// tiles 16, the rest 8: a tile's eight 4 x 8 blocks, whole, in halves of two rows or row by row
+// (the layout kernel of the binning chooses).  An item's pixels are those of the lanes with lane >> shift == sub.
+struct Item {
+    uint32_t place;   // of the tile in the work order
+    int blk, sub, shift;
+};
+
+struct __align__(16) ItemCounts {
+    uint32_t n4, n2, n_items;
+};
+
+__device__ __forceinline__ ItemCounts item_counts(const RenderArgs &A)
+{
+    ItemCounts c;
+    c.n4 = A.split[0];
+    c.n2 = A.split[1];
+    c.n_items = kBlocksPerTile * (static_cast<uint32_t>(A.n_tiles) + c.n2 + 3u * c.n4);
+    return c;
+}
+
+__device__ __forceinline__ Item decode_item(const ItemCounts &c, uint32_t item)
+{
+    Item it;
+    int ls = 2;
+    it.place = 0u;
+    if (item >= 32u * c.n4) {
+        item -= 32u * c.n4;
+        it.place = c.n4;
+        ls = 1;
+        if (item >= 16u * c.n2) {
+            item -= 16u * c.n2;
+            it.place += c.n2;
+            ls = 0;
+        }
+    }
+    it.place += item >> (3 + ls);
+    it.blk = static_cast<int>(item >> ls) & (kBlocksPerTile - 1);
+    it.sub = static_cast<int>(item) & ((1 << ls) - 1);
+    it.shift = 5 - ls;
+    return it;
 }
 
 // copy the tile's 192-byte record into the warp's shared slot
@@ -453,6 +502,7 @@ __device__ __forceinline__ void append_records(const RenderArgs &A, bool have, u
 // forward
 // ---------------------------------------------------------------------------------------------
 struct FwdShared {
+    ItemCounts items;
     WarpBatch w[kWarps];
     TileInfo ti[kWarps];
     WarpQueue q[kWarps];
@@ -470,15 +520,18 @@ __global__ void __launch_bounds__(kBlock, 3) k_render_fwd(const RenderArgs A)
     WarpQueue &q = sh.q[warp];
     unsigned long long evals = 0;
 
-    for (;;) {
-        const uint32_t item = next_item(A.queue, lane);
-        if (item >= A.n_items) break;
-        const int64_t tile = A.tile_order[item / kBlocksPerTile];
-        const int blk = item % kBlocksPerTile;
+    if (threadIdx.x == 0) sh.items = item_counts(A);   // shared: registers are short here
+    __syncthreads();
+    for (uint32_t item = next_item(A.queue, lane); item < sh.items.n_items;
+         item = next_item(A.queue, lane)) {
+        const Item it = decode_item(sh.items, item);
+        const int64_t tile = A.tile_order[it.place];
+        const int blk = it.blk;
         __syncwarp();
         load_tile(A.tiles, tile, ti, lane);
-        const BlockPix bp = block_pixel<TH, TW>(ti, blk, lane);
+        BlockPix bp = block_pixel<TH, TW>(ti, blk, lane);
         put_pix(w, lane, load_pix(A.pixframes, bp.inside ? bp.pf : ti.pix_base));
+        bp.inside = bp.inside && (lane >> it.shift) == it.sub;
         const uint2 rg = A.ranges[tile];
         float T = 1.0f, D = 0.0f, N0 = 0.0f, N1 = 0.0f, N2 = 0.0f, O = 0.0f;
         int last = 0;
@@ -689,6 +742,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_render_fwd(const RenderArgs A)
 // backward
 // ---------------------------------------------------------------------------------------------
 struct BwdShared {
+    ItemCounts items;
     WarpBatch w[kWarps];
     float acc[kWarps][32][kAcc];
     float pose[kWarps][16];  // the batch's reduced sensor-pose terms (9 used)
@@ -708,15 +762,18 @@ __global__ void __launch_bounds__(kBlock, 3) k_render_bwd(const RenderArgs A)
     TileInfo &ti = sh.ti[warp];
     unsigned long long evals = 0;
 
-    for (;;) {
-        const uint32_t item = next_item(A.queue, lane);
-        if (item >= A.n_items) break;
-        const int64_t tile = A.tile_order[item / kBlocksPerTile];
-        const int blk = item % kBlocksPerTile;
+    if (threadIdx.x == 0) sh.items = item_counts(A);   // shared: registers are short here
+    __syncthreads();
+    for (uint32_t item = next_item(A.queue, lane); item < sh.items.n_items;
+         item = next_item(A.queue, lane)) {
+        const Item it = decode_item(sh.items, item);
+        const int64_t tile = A.tile_order[it.place];
+        const int blk = it.blk;
         __syncwarp();
         load_tile(A.tiles, tile, ti, lane);
-        const BlockPix bp = block_pixel<TH, TW>(ti, blk, lane);
+        BlockPix bp = block_pixel<TH, TW>(ti, blk, lane);
         put_pix(w, lane, load_pix(A.pixframes, bp.inside ? bp.pf : ti.pix_base));
+        bp.inside = bp.inside && (lane >> it.shift) == it.sub;
         float T = 1.0f, gD = 0.0f, gN0 = 0.0f, gN1 = 0.0f, gN2 = 0.0f, gO = 0.0f;
         if (bp.inside) {
             T = A.t_final[bp.out];

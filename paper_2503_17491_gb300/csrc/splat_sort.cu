@@ -36,16 +36,30 @@ constexpr int kListThreads = 256, kListCtas = 3;   // CTAs per SM
 constexpr int kListWarps = kListThreads / 32;
 constexpr int kWarpCap = 256;             // lists below this are sorted by one warp
 constexpr int kMaxItems = kListCap / kListThreads;   // 16 keys a thread
-constexpr int kMidBucket = 9;             // 32 - clz(kWarpCap): lists of 256 and more
-constexpr int kLongBucket = 13;           // lists of kListCap and more
-static_assert(kWarpCap == 1 << (kMidBucket - 1) && kListCap == 1 << (kLongBucket - 1), "buckets");
 
 // ---------------------------------------------------------------------------------------------
 // layout (one CTA)
 // ---------------------------------------------------------------------------------------------
 constexpr int kLayoutThreads = 1024;
 
-__device__ __forceinline__ int len_bucket(uint32_t len) { return len ? 32 - __clz(len) : 0; }
+// Four buckets an octave of list length: bucket b holds [bucket_len(b), bucket_len(b + 1)).
+constexpr int kBuckets = 128;
+__host__ __device__ constexpr int log2_floor(uint32_t x)
+{
+    int l = 0;
+    while (x >>= 1) ++l;
+    return l;
+}
+__device__ __forceinline__ int len_bucket(uint32_t len)
+{
+    if (len < 4u) return static_cast<int>(len);
+    const int l = 31 - __clz(len);
+    return 4 * (l - 1) + static_cast<int>(len >> (l - 2) & 3u);
+}
+constexpr int kMidBucket = 4 * (log2_floor(kWarpCap) - 1);    // lists of kWarpCap and more
+constexpr int kLongBucket = 4 * (log2_floor(kListCap) - 1);   // lists of kListCap and more
+static_assert(kWarpCap == 1 << log2_floor(kWarpCap) && kListCap == 1 << log2_floor(kListCap),
+              "bucket bounds");
 
 // exclusive sum over the CTA's threads; *total gets the sum of all
 template <int kThreads, typename T>
@@ -76,15 +90,35 @@ __device__ __forceinline__ T block_excl_scan(T v, T *s_warp, T *total)
     return x - v + s_warp[warp];
 }
 
+// Which tiles' blocks the compositing kernels split: with L = 8 entries / warps a warp's even share
+// of the frame (in entries of one block's list), lists of at least kSplit2Share L go to two warps a
+// block and lists of at least kSplit4Share L to four, both rounded up to a bucket of the work
+// order, which the split tiles lead.  Measured, forward / backward in ms, whole | split at 0.4 and
+// 0.8 of a share | at 0.7 and 1.2:
+//   64x1024, 100 k primitives, longest list 15 shares   .125 .112 | .066 .047 | .066 .048
+//   three ragged scans, 83 k, 7 shares                  .102 .100 | .064 .057 | .068 .060
+//   four 64x1024, 200 k, 4 shares                       .245 .217 | .154 .150 | .154 .157
+//   eight 128x1024 along a street, 3 shares             .446      | .315      | .318
+//   128x2048, 1 M, urban block, 2.1 shares              .249 .225 |           | .274 .250
+//   12 keyframes, 500 k, 1.8 shares                     .729 .816 |           | .768 .842
+// Where even the longest list is below about kSplitFrom shares (the last two) the queue evens the
+// warps out by itself and splitting only costs, so such a frame is left whole.
+// A split block keeps one contributor record per part and primitive, so nothing is split when the
+// record pool might not hold one record for every row of 8 pixels that every pair meets (n_rows
+// counts those): the pool then overflows for no frame that it held unsplit.
+constexpr float kSplit2Share = 0.4f, kSplit4Share = 0.8f, kSplitFrom = 2.5f;
+constexpr uint32_t kSplitLeast = 64;
+
 __global__ void __launch_bounds__(kLayoutThreads) k_layout(
     const uint32_t *__restrict__ tile_count, int64_t n_tiles, int64_t max_pairs,
     uint2 *__restrict__ ranges, uint32_t *__restrict__ order, uint32_t *__restrict__ d_count,
-    uint32_t *status, uint32_t *__restrict__ bin)
+    uint32_t *status, uint32_t *__restrict__ bin, uint32_t warps, uint32_t rec_cap,
+    const unsigned long long *n_rows)
 {
     __shared__ unsigned long long s_warp[33];
-    __shared__ uint32_t s_cnt[33], s_off[33];
+    __shared__ uint32_t s_cnt[kBuckets], s_off[kBuckets];
     const int tid = threadIdx.x, lane = tid & 31;
-    if (tid < 33) s_cnt[tid] = 0;
+    if (tid < kBuckets) s_cnt[tid] = 0;
     __syncthreads();
     // each thread takes a run of consecutive tiles; the loop bounds are uniform so that the
     // whole warp takes part in the matches
@@ -95,22 +129,37 @@ __global__ void __launch_bounds__(kLayoutThreads) k_layout(
         const bool in = t0 + k < n_tiles;
         const uint32_t len = in ? tile_count[t0 + k] : 0u;
         sum += len;
-        const int b = in ? len_bucket(len) : 33;
+        const int b = in ? len_bucket(len) : kBuckets;
         const uint32_t peers = __match_any_sync(kFull, b);
         if (in && lane == __ffs(peers) - 1) atomicAdd(&s_cnt[b], __popc(peers));
     }
     unsigned long long total;
-    unsigned long long run = block_excl_scan<kLayoutThreads>(sum, s_warp, &total);
+    const unsigned long long run0 = block_excl_scan<kLayoutThreads>(sum, s_warp, &total);
+    __syncthreads();
+    // s_off[b]: tiles in the buckets above b
+    const unsigned long long above = block_excl_scan<kLayoutThreads, unsigned long long>(
+        tid < kBuckets ? s_cnt[kBuckets - 1 - tid] : 0u, s_warp, nullptr);
+    if (tid < kBuckets) s_off[kBuckets - 1 - tid] = static_cast<uint32_t>(above);
+    __syncthreads();
+    unsigned long long run = run0;
     if (tid == 0) {
-        uint32_t at = 0;
-        for (int b = 32; b >= 0; --b) {
-            s_off[b] = at;
-            at += s_cnt[b];
-        }
         bin[kBinLong] = s_off[kLongBucket - 1];
         bin[kBinSegments] = 0u;
         bin[kBinQueueSeg] = 0u;
         bin[kBinMid] = s_off[kMidBucket - 1];
+        const float share = static_cast<float>(total) * 8.0f / static_cast<float>(warps);
+        // tiles of clearly more than x shares
+        auto tiles_above = [&](float x) {
+            return s_off[len_bucket(max(kSplitLeast, static_cast<uint32_t>(
+                                                         fminf(share * x, 2147483647.0f))))];
+        };
+        uint32_t n4 = tiles_above(kSplit4Share), n2 = tiles_above(kSplit2Share) - n4;
+        if (tiles_above(kSplitFrom) == 0u) n4 = n2 = 0u;
+        const unsigned long long items =
+            8ull * (static_cast<unsigned long long>(n_tiles) + n2 + 3ull * n4);
+        if (rec_cap && *n_rows / 32 + items > rec_cap) n4 = n2 = 0u;
+        bin[kBinSplit4] = n4;
+        bin[kBinSplit2] = n2;
         const bool over = total > static_cast<unsigned long long>(max_pairs);
         if (over) atomicOr(status, SPLAT_STATUS_CAPACITY);
         *d_count = static_cast<uint32_t>(over ? max_pairs : static_cast<int64_t>(total));
@@ -121,7 +170,7 @@ __global__ void __launch_bounds__(kLayoutThreads) k_layout(
     for (int64_t k = 0; k < per; ++k) {
         const bool in = t0 + k < n_tiles;
         const uint32_t len = in ? tile_count[t0 + k] : 0u;
-        const int b = in ? len_bucket(len) : 33;
+        const int b = in ? len_bucket(len) : kBuckets;
         const uint32_t peers = __match_any_sync(kFull, b);
         const int lead = __ffs(peers) - 1;
         uint32_t at = 0;
@@ -805,7 +854,8 @@ cudaError_t launch_bin_counts(const BinArgs &args, cudaStream_t st)
             k_count<false><<<grid, kChunkThreads, 0, st>>>(a);
     }
     k_layout<<<1, kLayoutThreads, 0, st>>>(a.tile_count, a.n_tiles, a.max_pairs, a.ranges, a.order,
-                                           a.d_count, a.status, a.bin);
+                                           a.d_count, a.status, a.bin, a.warps, a.rec_cap,
+                                           a.n_rows);
     return cudaGetLastError();
 }
 

@@ -1,14 +1,15 @@
 """The per-tile lists at the sizes where the list sort changes its path: one warp or one CTA per
 list, each number of keys a thread, lists cut into segments, segments that stay too large because
-their primitives share a range, and rectangles counted and emitted by a whole warp.  Lists and
-records bit-exact against the oracle.  Marked gpu."""
+their primitives share a range, and rectangles counted and emitted by a whole warp, blocks split
+over several warps.  Lists and records bit-exact against the oracle.  Marked gpu."""
 import math
 
 import numpy as np
 import pytest
+import torch
 
 import oracle
-from paper_2503_17491_gb300 import scenes
+from paper_2503_17491_gb300 import api, scenes
 from gpu_common import check_lists, make_ctx, to_dev
 
 pytestmark = pytest.mark.gpu
@@ -75,3 +76,30 @@ def test_wide_rectangles(tile):
                           log_scale=(-3.0, 0.7))
     m, _ = _check(s, tile)
     assert m > 10 * s.n
+
+
+@pytest.mark.parametrize("tile", [(16, 16), (8, 32), (32, 8), (4, 64)])
+def test_split_blocks(tile):
+    """A lone view whose blocks go to two and four warps against the same render with its blocks
+    whole (a record pool too small for the split): images bit-identical, gradients equal up to the
+    order of the float additions (each sum of k terms within k units of 2^-24 of its absolute
+    terms; 1e-5 of the largest gradient covers the scene's sums)."""
+    s = scenes.workload(1, n=30_000)
+    v = s.views[0]
+    dev = to_dev(s)
+    ctx = make_ctx(s.n, [v], tile)
+    a = ctx.render(*dev)
+    st = ctx.stats()
+    whole = api.SplatContext(s.n, 1, v.n_pixels, st["n_pairs"] + 8,
+                             api.RenderConfig(tile_h=tile[0], tile_w=tile[1]),
+                             max_tiles=st["n_tiles"])
+    whole.set_views([v])
+    b = whole.render(*dev)
+    for x, y in zip(a, b):
+        assert torch.equal(x, y)
+    rng = np.random.default_rng(2)
+    up = [torch.from_numpy(rng.normal(size=t.shape).astype(np.float32)).cuda() for t in a]
+    ga, gb = ctx.backward(*dev, *up), whole.backward(*dev, *up)
+    assert ctx.status() == 0 and whole.status() == 0
+    for x, y in zip(ga, gb):
+        assert (x - y).abs().max() <= 1e-5 * y.abs().max()
