@@ -205,10 +205,9 @@ class SplatContext:
     def backward(self, pos_logit, quat, log_scale, gD, gN, gO, out=None, accumulate=False,
                  stream=None):
         n = pos_logit.shape[0]
-        if out is None:
-            out = (torch.zeros(n, 4, device=pos_logit.device),
-                   torch.zeros(n, 4, device=pos_logit.device),
-                   torch.zeros(n, 2, device=pos_logit.device))
+        if out is None:   # overwritten whole unless added to
+            new = torch.zeros if accumulate else torch.empty
+            out = tuple(new(n, w, device=pos_logit.device) for w in (4, 4, 2))
         g = self._g(pos_logit, quat, log_scale)
         _lib.check(self.lib.splat_render_views_backward(
             self.h, ctypes.byref(g), _ptr(gD), _ptr(gN), _ptr(gO), _ptr(out[0]), _ptr(out[1]),

@@ -61,6 +61,9 @@ void split(double x, float &hi, float &lo)
 }  // namespace
 
 constexpr int kCountersBin = 8, kCounters = kCountersBin + splat::kBinWords;
+// words of splat_ctx::d_zero: queue f, pairs that touch a tile, record chunks taken, forward
+// evaluations (64 bits), rows met (64 bits), then one word per tile
+enum { kZeroQueue = 0, kZeroTouching, kZeroChunks, kZeroEvals = 4, kZeroRows = 6, kZeroTiles = 8 };
 
 struct splat_ctx {
     splat_render_config cfg{};
@@ -90,7 +93,7 @@ struct splat_ctx {
     uint64_t *d_touch = nullptr;
     float *d_kappa = nullptr;
     uint32_t *d_touch_count = nullptr;
-    uint32_t *d_tile_count = nullptr, *d_cta_count = nullptr;
+    uint32_t *d_cta_count = nullptr;
     uint64_t *d_entries = nullptr, *d_entries2 = nullptr;   // tile lists (BinArgs)
     uint8_t *d_blocks = nullptr;
     splat::ListSegment *d_segments = nullptr;
@@ -105,12 +108,12 @@ struct splat_ctx {
     uint32_t rec_cap = 0;           // chunks in the record pool
     float *d_img = nullptr;     // refine: depth, normal(3), alpha  (5 x max_pixels)
     float *d_gimg = nullptr;    // refine: their gradients
-    uint32_t *d_counters = nullptr;   // [0] pairs M, [1] status, [2] queue f, [3] queue b,
-                                      // [4] (view, primitive) pairs that touch a tile,
-                                      // [5] record chunks taken, [6] map-growth draws,
+    uint32_t *d_counters = nullptr;   // [0] pairs M, [1] status, [3] queue b, [6] map-growth draws,
                                       // [7] sampling step, [8..] binning (splat::kBin...)
     unsigned long long *d_grow_sums = nullptr;  // map growth: block sums, Q, offset
-    unsigned long long *d_evals = nullptr;      // [0] forward, [1] backward, [2] rows met
+    unsigned long long *d_bwd_evals = nullptr;
+    // what a render starts from zero, in one piece (kZero... words, then the tiles' list lengths)
+    uint32_t *d_zero = nullptr;
 
     // profiling events: [0,1] forward compositing, [2,3] backward compositing, then one event
     // after the stages of the last profiled render / refinement step: [0] before the
@@ -158,6 +161,7 @@ int check_gaussians(const splat_ctx *ctx, const splat_gaussians *g)
 splat::RenderArgs render_args(splat_ctx *ctx, const splat_gaussians *g)
 {
     splat::RenderArgs a{};
+    a.chain = splat::chained_size(g->n * ctx->n_views);
     a.prim = ctx->d_prim;
     a.n = g->n;
     a.tiles = ctx->d_tileinfo;
@@ -168,7 +172,7 @@ splat::RenderArgs render_args(splat_ctx *ctx, const splat_gaussians *g)
     a.entry_blocks = ctx->d_blocks;
     a.rec = ctx->d_rec;
     a.rec_prev = ctx->d_rec_prev;
-    a.rec_alloc = ctx->d_counters + 5;
+    a.rec_alloc = ctx->d_zero + kZeroChunks;
     a.rec_cap = ctx->rec_cap;
     a.rec_head = ctx->d_rec_head;
     a.rec_fill = ctx->d_rec_fill;
@@ -187,19 +191,16 @@ splat::RenderArgs render_args(splat_ctx *ctx, const splat_gaussians *g)
 }
 
 // forward pipeline: projection -> list layout -> emission -> list sort -> composite
+// refine (nullable): what the refinement step around it starts from, set on the way
 int render_core(splat_ctx *ctx, const splat_gaussians *g, float *depth, float *normal,
-                float *alpha, cudaStream_t st)
+                float *alpha, cudaStream_t st, const splat::RefineStart *refine = nullptr)
 {
     const int64_t n = g->n;
     const int th = ctx->cfg.tile_h, tw = ctx->cfg.tile_w;
     uint32_t *cnt = ctx->d_counters;
-    CK(cudaMemsetAsync(cnt, 0, sizeof(uint32_t), st));           // pair count
-    CK(cudaMemsetAsync(cnt + 4, 0, 2 * sizeof(uint32_t), st));   // touching pairs, chunks
-    CK(cudaMemsetAsync(cnt + 2, 0, sizeof(uint32_t), st));       // forward queue
-    CK(cudaMemsetAsync(ctx->d_evals, 0, sizeof(unsigned long long), st));
-    CK(cudaMemsetAsync(ctx->d_evals + 2, 0, sizeof(unsigned long long), st));
-    CK(cudaMemsetAsync(ctx->d_tile_count, 0,
-                       sizeof(uint32_t) * static_cast<size_t>(ctx->n_tiles), st));
+    uint32_t *zero = ctx->d_zero;
+    CK(cudaMemsetAsync(zero, 0, sizeof(uint32_t) * static_cast<size_t>(kZeroTiles + ctx->n_tiles),
+                       st));
     const uint8_t *active = nullptr;
     if (ctx->samp_draws > 0) {
         CK(splat::launch_sample_views(ctx->n_views, ctx->samp_draws, ctx->d_samp_thr,
@@ -235,8 +236,9 @@ int render_core(splat_ctx *ctx, const splat_gaussians *g, float *depth, float *n
     pa.touch_count = ctx->d_touch_count;
     pa.prim = ctx->d_prim;
     pa.status = cnt + 1;
-    pa.n_valid = cnt + 4;
-    pa.n_rows = ctx->d_evals + 2;
+    pa.n_valid = zero + kZeroTouching;
+    pa.n_rows = reinterpret_cast<unsigned long long *>(zero + kZeroRows);
+    pa.wgrad = refine ? ctx->d_wgrad : nullptr;
     pa.active = active;
     CK(splat::launch_project(pa, st));
     CK(stage_mark(1));
@@ -256,7 +258,7 @@ int render_core(splat_ctx *ctx, const splat_gaussians *g, float *depth, float *n
     ba.touch_count = ctx->d_touch_count;
     ba.max_pairs = ctx->cap.max_pairs;
     ba.max_view_tiles = ctx->max_view_tiles;
-    ba.tile_count = ctx->d_tile_count;
+    ba.tile_count = zero + kZeroTiles;
     ba.cta_count = ctx->d_cta_count;
     ba.ranges = ctx->d_ranges;
     ba.order = ctx->d_tile_order;
@@ -270,7 +272,8 @@ int render_core(splat_ctx *ctx, const splat_gaussians *g, float *depth, float *n
     ba.sms = ctx->sms;
     ba.warps = static_cast<uint32_t>(ctx->grid_fwd) * (splat::kBlock / 32);
     ba.rec_cap = ctx->rec_cap;
-    ba.n_rows = ctx->d_evals + 2;
+    ba.n_rows = pa.n_rows;
+    if (refine) ba.refine = *refine;
     CK(splat::launch_bin_counts(ba, st));
     CK(splat::launch_emit(ba, st));
     CK(stage_mark(3));
@@ -280,8 +283,8 @@ int render_core(splat_ctx *ctx, const splat_gaussians *g, float *depth, float *n
     a.depth = depth;
     a.normal = normal;
     a.alpha = alpha;
-    a.queue = cnt + 2;
-    a.evals = ctx->d_evals;
+    a.queue = zero + kZeroQueue;
+    a.evals = reinterpret_cast<unsigned long long *>(zero + kZeroEvals);
     if (prof) CK(cudaEventRecord(ctx->ev[0], st));
     CK(splat::launch_render_fwd(a, th, tw, ctx->grid_fwd, st));
     if (prof) {
@@ -295,23 +298,36 @@ int render_core(splat_ctx *ctx, const splat_gaussians *g, float *depth, float *n
     return SPLAT_OK;
 }
 
-// backward into the per-primitive world-frame accumulators
+// the counters and accumulators a backward adds to
+splat::RefineStart backward_start(splat_ctx *ctx)
+{
+    splat::RefineStart s{};
+    s.queue = ctx->d_counters + 3;
+    s.evals = ctx->d_bwd_evals;
+    if (ctx->want_pose) {
+        s.pose = ctx->d_pose;
+        s.n_pose = 6 * ctx->n_views;
+    }
+    return s;
+}
+
+// backward into the per-primitive world-frame accumulators; started: they and the counters are
+// already zero
 int backward_core(splat_ctx *ctx, const splat_gaussians *g, const float *gD, const float *gN,
-                  const float *gO, cudaStream_t st)
+                  const float *gO, cudaStream_t st, bool started)
 {
     uint32_t *cnt = ctx->d_counters;
-    CK(cudaMemsetAsync(ctx->d_wgrad, 0, sizeof(float4) * 4 * static_cast<size_t>(g->n), st));
-    if (ctx->want_pose)
-        CK(cudaMemsetAsync(ctx->d_pose, 0, sizeof(float) * 6 * static_cast<size_t>(ctx->n_views),
-                           st));
-    CK(cudaMemsetAsync(cnt + 3, 0, sizeof(uint32_t), st));
-    CK(cudaMemsetAsync(ctx->d_evals + 1, 0, sizeof(unsigned long long), st));
+    if (!started) {
+        CK(splat::launch_backward_start(backward_start(ctx), ctx->d_wgrad, g->n,
+                                        splat::chained_size(g->n * ctx->n_views), st));
+        ctx->launches += 1;
+    }
     splat::RenderArgs a = render_args(ctx, g);
     a.g_depth = gD;
     a.g_normal = gN;
     a.g_alpha = gO;
     a.queue = cnt + 3;
-    a.evals = ctx->d_evals + 1;
+    a.evals = ctx->d_bwd_evals;
     a.pose_grad = ctx->want_pose ? ctx->d_pose : nullptr;
     const bool prof = ctx->profiling && !capturing(st);
     if (prof) CK(cudaEventRecord(ctx->ev[2], st));
@@ -329,11 +345,11 @@ void free_ctx(splat_ctx *c)
 {
     void *ptrs[] = {c->d_views, c->d_frames, c->d_tile_view, c->d_prect, c->d_touch, c->d_kappa,
                     c->d_touch_count,
-                    c->d_tile_count, c->d_cta_count, c->d_entries, c->d_entries2, c->d_blocks, c->d_segments,
+                    c->d_zero, c->d_cta_count, c->d_entries, c->d_entries2, c->d_blocks, c->d_segments,
                     c->d_ranges, c->d_tfinal, c->d_nlast, c->d_wgrad, c->d_prim,
                     c->d_pose, c->d_rec, c->d_rec_prev, c->d_rec_head, c->d_rec_fill,
                     c->d_samp_thr, c->d_active, c->d_grow_sums,
-                    c->d_img, c->d_gimg, c->d_counters, c->d_evals, c->d_pixframes,
+                    c->d_img, c->d_gimg, c->d_counters, c->d_bwd_evals, c->d_pixframes,
                     c->d_tileinfo, c->d_tile_order};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -420,7 +436,7 @@ SPLAT_API int splat_ctx_create(const splat_render_config *cfg, const splat_capac
     if (e == cudaSuccess)
         e = dalloc(&c->d_touch_count,
                    static_cast<size_t>(splat::max_project_blocks(cap->max_gaussians)) * cap->max_views);
-    if (e == cudaSuccess) e = dalloc(&c->d_tile_count, TT);
+    if (e == cudaSuccess) e = dalloc(&c->d_zero, kZeroTiles + static_cast<size_t>(TT));
     if (e == cudaSuccess)
         e = dalloc(&c->d_cta_count, splat::cta_count_words(c->sms, cap->max_views, TT));
     // the forward reads the lists four entries at a time from a 4-aligned index: 128 spare
@@ -454,12 +470,13 @@ SPLAT_API int splat_ctx_create(const splat_render_config *cfg, const splat_capac
     if (e == cudaSuccess) e = dalloc(&c->d_img, static_cast<size_t>(P) * 5);
     if (e == cudaSuccess) e = dalloc(&c->d_gimg, static_cast<size_t>(P) * 5);
     if (e == cudaSuccess) e = dalloc(&c->d_counters, kCounters);
-    if (e == cudaSuccess) e = dalloc(&c->d_evals, 3);
+    if (e == cudaSuccess) e = dalloc(&c->d_bwd_evals, 1);
     for (int k = 0; k < 4 && e == cudaSuccess; ++k) e = cudaEventCreate(&c->ev[k]);
     for (int k = 0; k < splat_ctx::kStageEvents && e == cudaSuccess; ++k)
         e = cudaEventCreate(&c->stage_ev[k]);
     if (e == cudaSuccess) e = cudaMemset(c->d_counters, 0, kCounters * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMemset(c->d_evals, 0, 3 * sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMemset(c->d_bwd_evals, 0, sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMemset(c->d_zero, 0, kZeroTiles * sizeof(uint32_t));
     if (e == cudaSuccess) e = splat::prepare_lists();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
@@ -685,7 +702,7 @@ SPLAT_API int splat_render_views_backward(splat_ctx *ctx, const splat_gaussians 
     if (!ctx->rendered || g->n != ctx->last_n) return SPLAT_ERR_STATE;
     if (!g_pos_logit || !g_quat || !g_log_scale) return SPLAT_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    r = backward_core(ctx, g, dL_ddepth, dL_dnormal, dL_dalpha, st);
+    r = backward_core(ctx, g, dL_ddepth, dL_dnormal, dL_dalpha, st, false);
     if (r) return r;
     CK(splat::launch_param_grads(reinterpret_cast<const float4 *>(g->pos_logit),
                                  reinterpret_cast<const float4 *>(g->quat_wxyz),
@@ -802,7 +819,7 @@ SPLAT_API int splat_loss(const float *depth, const float *normal, const float *a
         return SPLAT_ERR_INVALID_ARG;
     CK(splat::launch_loss(depth, normal, alpha, target_depth, target_normal, n_pixels,
                           cfg->lambda_n, cfg->lambda_o, cfg->o_eps, cfg->rho_exp, dL_ddepth, dL_dnormal,
-                          dL_dalpha, loss_out, static_cast<cudaStream_t>(stream)));
+                          dL_dalpha, loss_out, static_cast<cudaStream_t>(stream), false));
     return SPLAT_OK;
 }
 
@@ -824,7 +841,7 @@ SPLAT_API int splat_view_loss(splat_ctx *ctx, const float *depth, const float *n
     if (ctx->n_views < 1) return SPLAT_ERR_STATE;
     CK(splat::launch_loss(depth, normal, alpha, target_depth, target_normal, ctx->n_pixels,
                           cfg->lambda_n, cfg->lambda_o, cfg->o_eps, cfg->rho_exp, dL_ddepth, dL_dnormal,
-                          dL_dalpha, loss_out, static_cast<cudaStream_t>(stream), ctx->d_views,
+                          dL_dalpha, loss_out, static_cast<cudaStream_t>(stream), false, ctx->d_views,
                           ctx->n_views, nullptr, cfg->normal_mode));
     return SPLAT_OK;
 }
@@ -887,12 +904,16 @@ SPLAT_API int splat_refine_step(splat_ctx *ctx, float *pos_logit, float *quat, f
     const int64_t P = ctx->n_pixels;
     float *depth = ctx->d_img, *normal = ctx->d_img + P, *alpha = ctx->d_img + 4 * P;
     float *gd = ctx->d_gimg, *gn = ctx->d_gimg + P, *ga = ctx->d_gimg + 4 * P;
-    r = render_core(ctx, &g, depth, normal, alpha, st);
+    // the accumulators, the loss and the backward's counters are zeroed and the step is counted by
+    // kernels of the render
+    splat::RefineStart start = backward_start(ctx);
+    start.loss = loss_out;
+    start.step = step;
+    r = render_core(ctx, &g, depth, normal, alpha, st, &start);
     if (r) return r;
-    CK(cudaMemsetAsync(loss_out, 0, sizeof(double), st));
     CK(splat::launch_loss(depth, normal, alpha, target_depth, target_normal, P, loss_cfg->lambda_n,
                           loss_cfg->lambda_o, loss_cfg->o_eps, loss_cfg->rho_exp, gd, gn, ga,
-                          loss_out, st,
+                          loss_out, st, splat::chained_size(n * ctx->n_views),
                           ctx->d_views, ctx->n_views,
                           ctx->samp_draws > 0 ? ctx->d_active : nullptr,
                           loss_cfg->normal_mode));
@@ -901,7 +922,7 @@ SPLAT_API int splat_refine_step(splat_ctx *ctx, float *pos_logit, float *quat, f
         CK(cudaEventRecord(ctx->stage_ev[6], st));
         ctx->stage_rec[6] = true;
     }
-    r = backward_core(ctx, &g, gd, gn, ga, st);
+    r = backward_core(ctx, &g, gd, gn, ga, st, true);
     if (r) return r;
     splat::AdamArgs a{};
     a.pos_logit = reinterpret_cast<float4 *>(pos_logit);
@@ -925,13 +946,13 @@ SPLAT_API int splat_refine_step(splat_ctx *ctx, float *pos_logit, float *quat, f
     a.lambda_s = loss_cfg->lambda_s;
     a.tau_s = loss_cfg->tau_s;
     a.loss_out = loss_out;
+    a.chain = splat::chained_size(n * ctx->n_views);
     CK(splat::launch_adam_fused(a, ctx->d_wgrad, st));
     if (prof) {
         CK(cudaEventRecord(ctx->stage_ev[7], st));
         ctx->stage_rec[7] = true;
     }
-    CK(splat::launch_step_inc(step, st));
-    ctx->launches += 3;   // loss, fused Adam, step counter
+    ctx->launches += 2;   // loss, fused Adam
     return SPLAT_OK;
 }
 
@@ -1014,14 +1035,16 @@ SPLAT_API int splat_get_stats(splat_ctx *ctx, splat_stats *out)
 {
     if (!ctx || !out) return SPLAT_ERR_INVALID_ARG;
     CK(cudaDeviceSynchronize());
-    uint32_t c[5] = {0, 0, 0, 0, 0};
-    unsigned long long ev[2] = {0, 0};
-    CK(cudaMemcpy(c, ctx->d_counters, sizeof c, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(ev, ctx->d_evals, sizeof ev, cudaMemcpyDeviceToHost));
-    out->n_pairs = c[0];
-    out->n_touching = c[4];
-    out->fwd_evals = static_cast<int64_t>(ev[0]);
-    out->bwd_evals = static_cast<int64_t>(ev[1]);
+    uint32_t pairs = 0, zero[kZeroTiles] = {};
+    unsigned long long fwd = 0, bwd = 0;
+    CK(cudaMemcpy(&pairs, ctx->d_counters, sizeof pairs, cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(zero, ctx->d_zero, sizeof zero, cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(&bwd, ctx->d_bwd_evals, sizeof bwd, cudaMemcpyDeviceToHost));
+    std::memcpy(&fwd, zero + kZeroEvals, sizeof fwd);
+    out->n_pairs = pairs;
+    out->n_touching = zero[kZeroTouching];
+    out->fwd_evals = static_cast<int64_t>(fwd);
+    out->bwd_evals = static_cast<int64_t>(bwd);
     out->n_pixels = ctx->n_pixels;
     out->n_tiles = ctx->n_tiles;
     out->kernel_launches = ctx->launches;

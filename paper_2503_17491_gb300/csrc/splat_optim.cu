@@ -127,6 +127,7 @@ __global__ void __launch_bounds__(256) k_loss(const float *__restrict__ depth,
                                               const ViewDesc *__restrict__ views, int n_views,
                                               const uint8_t *__restrict__ active)
 {
+    chain_wait();
     __shared__ double s_part[8];
     float acc = 0.0f;
     for (int64_t p = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; p < n;
@@ -200,9 +201,10 @@ struct AdamScalars {
     float c1, c2;   // bias corrections 1 - beta^t
 };
 
-__device__ __forceinline__ AdamScalars adam_scalars(const AdamArgs &a)
+// step: the number of this step, from 1
+__device__ __forceinline__ AdamScalars adam_scalars(const AdamArgs &a, int32_t step)
 {
-    const float t = static_cast<float>(*a.step + 1);
+    const float t = static_cast<float>(step);
     return AdamScalars{1.0f - powf(a.beta1, t), 1.0f - powf(a.beta2, t)};
 }
 
@@ -248,12 +250,13 @@ __global__ void __launch_bounds__(256) k_adam(const AdamArgs a, const float4 *__
 {
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= a.n) return;
-    adam_prim(a, i, g_pl[i], g_q[i], g_ls[i], adam_scalars(a));
+    adam_prim(a, i, g_pl[i], g_q[i], g_ls[i], adam_scalars(a, *a.step + 1));
 }
 
 __global__ void __launch_bounds__(256) k_adam_fused(const AdamArgs a,
                                                     const float4 *__restrict__ wgrad)
 {
+    chain_wait();
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= a.n) return;
     float4 gp, gq;
@@ -276,7 +279,23 @@ __global__ void __launch_bounds__(256) k_adam_fused(const AdamArgs a,
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(am, acc, o);
         if ((threadIdx.x & 31) == __ffs(am) - 1 && acc != 0.0) atomicAdd(a.loss_out, acc);
     }
-    adam_prim(a, i, gp, gq, gl, adam_scalars(a));
+    adam_prim(a, i, gp, gq, gl, adam_scalars(a, *a.step));
+}
+
+// One launch instead of a memset for each: the accumulators by the grid, the rest by its first CTA.
+__global__ void __launch_bounds__(256) k_backward_start(const RefineStart s,
+                                                        float4 *__restrict__ wgrad, int64_t n4)
+{
+    chain_wait();
+    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (i < n4) wgrad[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (blockIdx.x == 0) {
+        for (int k = threadIdx.x; k < s.n_pose; k += blockDim.x) s.pose[k] = 0.0f;
+        if (threadIdx.x == 0) {
+            *s.queue = 0u;
+            *s.evals = 0ull;
+        }
+    }
 }
 
 __global__ void k_step_inc(int32_t *step)
@@ -290,7 +309,7 @@ cudaError_t launch_loss(const float *depth, const float *normal, const float *al
                         const float *t_depth, const float *t_normal, int64_t n_pixels,
                         float lambda_n, float lambda_o, float o_eps, float rho_exp,
                         float *g_depth, float *g_normal, float *g_alpha, double *loss_out,
-                        cudaStream_t st, const ViewDesc *views, int n_views,
+                        cudaStream_t st, bool chain, const ViewDesc *views, int n_views,
                         const uint8_t *active, int normal_mode)
 {
     if (n_pixels <= 0) return cudaSuccess;
@@ -299,12 +318,9 @@ cudaError_t launch_loss(const float *depth, const float *normal, const float *al
     int64_t blocks = (n_pixels + 255) / 256;
     if (blocks > 4096) blocks = 4096;
     auto kern = normal_mode == 1 ? k_loss<1> : k_loss<0>;
-    kern<<<static_cast<unsigned>(blocks), 256, 0, st>>>(depth, normal, alpha, t_depth, t_normal,
-                                                        n_pixels, lambda_n, lambda_o, o_eps,
-                                                        rho_exp, g_depth, g_normal, g_alpha,
-                                                        loss_out,
-                                                        views, n_views, active);
-    return cudaGetLastError();
+    return launch_chained(chain, kern, dim3(static_cast<unsigned>(blocks)), 256, 0, st, depth, normal,
+                          alpha, t_depth, t_normal, n_pixels, lambda_n, lambda_o, o_eps, rho_exp,
+                          g_depth, g_normal, g_alpha, loss_out, views, n_views, active);
 }
 
 cudaError_t launch_adam(const AdamArgs &a, const float4 *g_pl, const float4 *g_q,
@@ -318,8 +334,16 @@ cudaError_t launch_adam(const AdamArgs &a, const float4 *g_pl, const float4 *g_q
 cudaError_t launch_adam_fused(const AdamArgs &a, const float4 *wgrad, cudaStream_t st)
 {
     if (a.n <= 0) return cudaSuccess;
-    k_adam_fused<<<static_cast<unsigned>((a.n + 255) / 256), 256, 0, st>>>(a, wgrad);
-    return cudaGetLastError();
+    return launch_chained(a.chain, k_adam_fused, dim3(static_cast<unsigned>((a.n + 255) / 256)), 256, 0, st,
+                          a, wgrad);
+}
+
+cudaError_t launch_backward_start(const RefineStart &s, float4 *wgrad, int64_t n, bool chain,
+                                  cudaStream_t st)
+{
+    const int64_t n4 = 4 * n;
+    return launch_chained(chain, k_backward_start, dim3(static_cast<unsigned>(n4 > 0 ? (n4 + 255) / 256 : 1)),
+                          256, 0, st, s, wgrad, n4);
 }
 
 cudaError_t launch_step_inc(int32_t *step, cudaStream_t st)

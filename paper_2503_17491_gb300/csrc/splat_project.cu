@@ -505,6 +505,7 @@ struct ProjectShared {
 
 __global__ void __launch_bounds__(kProjectThreads, 3) k_project(const ProjectArgs A)
 {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char s_raw[];
     ProjectShared &sh = *reinterpret_cast<ProjectShared *>(s_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -625,6 +626,11 @@ __global__ void __launch_bounds__(kProjectThreads, 3) k_project(const ProjectArg
             e[1] = make_float4(sb * tb.x, sb * tb.y, sb * tb.z, ok ? 1.0f : 0.0f);
             e[2] = make_float4(tn.x, tn.y, tn.z, 0.0f);
             e[3] = make_float4(mu.x, mu.y, mu.z, 0.0f);
+            if (A.wgrad) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    A.wgrad[4 * i + k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            }
         }
 
         for (int v = 0; v < A.n_views; ++v) {
@@ -741,9 +747,8 @@ cudaError_t launch_project(const ProjectArgs &a, cudaStream_t st)
     if (a.n <= 0) return cudaSuccess;
     ProjectArgs b = a;
     b.block_prims = block_prims(a.n);
-    k_project<<<static_cast<unsigned>(project_blocks(a.n)), kProjectThreads, sizeof(ProjectShared),
-                st>>>(b);
-    return cudaGetLastError();
+    return launch_chained(chained_size(a.n * a.n_views), k_project, dim3(static_cast<unsigned>(project_blocks(a.n))),
+                          kProjectThreads, sizeof(ProjectShared), st, b);
 }
 
 cudaError_t launch_records(int64_t n, int n_views, const ViewDesc *views, int flip_normals,

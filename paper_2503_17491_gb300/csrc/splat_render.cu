@@ -511,6 +511,7 @@ struct FwdShared {
 template <int TH, int TW>
 __global__ void __launch_bounds__(kBlock, 3) k_render_fwd(const RenderArgs A)
 {
+    chain_wait();
     static_assert(TH * TW == kBlock && TH % 4 == 0 && TW % 8 == 0, "4x8 warp blocks");
     extern __shared__ __align__(16) unsigned char s_raw[];
     FwdShared &sh = *reinterpret_cast<FwdShared *>(s_raw);
@@ -752,6 +753,7 @@ struct BwdShared {
 template <int TH, int TW>
 __global__ void __launch_bounds__(kBlock, 3) k_render_bwd(const RenderArgs A)
 {
+    chain_wait();
     static_assert(TH * TW == kBlock && TH % 4 == 0 && TW % 8 == 0, "4x8 warp blocks");
     extern __shared__ __align__(16) unsigned char s_raw[];
     BwdShared &sh = *reinterpret_cast<BwdShared *>(s_raw);
@@ -1077,6 +1079,7 @@ __global__ void k_param_grads(const float4 *__restrict__ pos_logit, const float4
                               float4 *__restrict__ g_pl, float4 *__restrict__ g_q,
                               float2 *__restrict__ g_ls, int accumulate)
 {
+    chain_wait();
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= n) return;
     float4 a, b;
@@ -1132,8 +1135,7 @@ cudaError_t launch_render_fwd(const RenderArgs &a, int tile_h, int tile_w, int g
         constexpr int h = decltype(TH)::value, w = decltype(TW)::value;
         const cudaError_t e = fwd_prepare<h, w>();
         if (e != cudaSuccess) return e;
-        k_render_fwd<h, w><<<grid, kBlock, sizeof(FwdShared), st>>>(a);
-        return cudaGetLastError();
+        return launch_chained(a.chain, k_render_fwd<h, w>, dim3(grid), kBlock, sizeof(FwdShared), st, a);
     });
 }
 
@@ -1144,8 +1146,7 @@ cudaError_t launch_render_bwd(const RenderArgs &a, int tile_h, int tile_w, int g
         constexpr int h = decltype(TH)::value, w = decltype(TW)::value;
         const cudaError_t e = bwd_prepare<h, w>();
         if (e != cudaSuccess) return e;
-        k_render_bwd<h, w><<<grid, kBlock, sizeof(BwdShared), st>>>(a);
-        return cudaGetLastError();
+        return launch_chained(a.chain, k_render_bwd<h, w>, dim3(grid), kBlock, sizeof(BwdShared), st, a);
     });
 }
 
@@ -1174,9 +1175,8 @@ cudaError_t launch_param_grads(const float4 *pos_logit, const float4 *quat, cons
 {
     (void)log_scale;
     if (n <= 0) return cudaSuccess;
-    k_param_grads<<<static_cast<unsigned>((n + 255) / 256), 256, 0, st>>>(
-        pos_logit, quat, wgrad, n, g_pos_logit, g_quat, g_log_scale, accumulate);
-    return cudaGetLastError();
+    return launch_chained(chained_size(n), k_param_grads, dim3(static_cast<unsigned>((n + 255) / 256)), 256, 0, st,
+                          pos_logit, quat, wgrad, n, g_pos_logit, g_quat, g_log_scale, accumulate);
 }
 
 }  // namespace splat

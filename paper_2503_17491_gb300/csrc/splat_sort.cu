@@ -113,8 +113,9 @@ __global__ void __launch_bounds__(kLayoutThreads) k_layout(
     const uint32_t *__restrict__ tile_count, int64_t n_tiles, int64_t max_pairs,
     uint2 *__restrict__ ranges, uint32_t *__restrict__ order, uint32_t *__restrict__ d_count,
     uint32_t *status, uint32_t *__restrict__ bin, uint32_t warps, uint32_t rec_cap,
-    const unsigned long long *n_rows)
+    const unsigned long long *n_rows, const RefineStart start)
 {
+    chain_wait();
     __shared__ unsigned long long s_warp[33];
     __shared__ uint32_t s_cnt[kBuckets], s_off[kBuckets];
     const int tid = threadIdx.x, lane = tid & 31;
@@ -160,10 +161,15 @@ __global__ void __launch_bounds__(kLayoutThreads) k_layout(
         if (rec_cap && *n_rows / 32 + items > rec_cap) n4 = n2 = 0u;
         bin[kBinSplit4] = n4;
         bin[kBinSplit2] = n2;
+        if (start.queue) *start.queue = 0u;
+        if (start.evals) *start.evals = 0ull;
+        if (start.loss) *start.loss = 0.0;
+        if (start.step) *start.step += 1;
         const bool over = total > static_cast<unsigned long long>(max_pairs);
         if (over) atomicOr(status, SPLAT_STATUS_CAPACITY);
         *d_count = static_cast<uint32_t>(over ? max_pairs : static_cast<int64_t>(total));
     }
+    for (int k = tid; k < start.n_pose; k += kLayoutThreads) start.pose[k] = 0.0f;
     __syncthreads();
     // past the capacity a list keeps the places below it (the status bit marks the result)
     const unsigned long long cap = static_cast<unsigned long long>(max_pairs);
@@ -320,6 +326,7 @@ __device__ __forceinline__ void for_each_entry(const Chunk &c, F f)
 template <bool kShared>
 __global__ void __launch_bounds__(kChunkThreads) k_count(const BinArgs A)
 {
+    chain_wait();
     extern __shared__ uint32_t s_cnt[];
     const int v = blockIdx.y;
     if (A.active && !A.active[v]) return;
@@ -343,6 +350,7 @@ __global__ void __launch_bounds__(kChunkThreads) k_count(const BinArgs A)
 template <bool kShared>
 __global__ void __launch_bounds__(kChunkThreads) k_emit(const BinArgs A)
 {
+    chain_wait();
     extern __shared__ uint32_t s_cnt[];
     const int v = blockIdx.y;
     if (A.active && !A.active[v]) return;
@@ -405,6 +413,7 @@ __device__ __forceinline__ void for_each_key(const uint64_t *src, uint32_t n, F 
 // memory).
 __global__ void __launch_bounds__(kSplitThreads) k_split(const BinArgs A)
 {
+    chain_wait();
     __shared__ uint32_t s_bin[kSplitBins];
     __shared__ uint32_t s_start[kSplitBins + 1];
     __shared__ uint32_t s_warp[33];
@@ -778,6 +787,7 @@ __device__ __noinline__ void sort_oversized(const BinArgs &A, const ListSegment 
 // warps take the shorter lists.
 __global__ void __launch_bounds__(kListThreads, kListCtas) k_lists(const BinArgs A)
 {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char s_raw[];
     ListShared &sh = *reinterpret_cast<ListShared *>(s_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -831,6 +841,8 @@ dim3 chunk_grid(BinArgs &a)
                 static_cast<unsigned>(a.n_views));
 }
 
+bool chained(const BinArgs &a) { return chained_size(a.n * a.n_views); }
+
 }  // namespace
 
 // k_lists' shared memory is above the 48 KB static limit: allow it once
@@ -848,15 +860,15 @@ cudaError_t launch_bin_counts(const BinArgs &args, cudaStream_t st)
     BinArgs a = args;
     if (a.n > 0) {
         const dim3 grid = chunk_grid(a);
-        if (a.max_view_tiles <= kMaxSharedTiles)
-            k_count<true><<<grid, kChunkThreads, 4 * a.max_view_tiles, st>>>(a);
-        else
-            k_count<false><<<grid, kChunkThreads, 0, st>>>(a);
+        const bool shared = a.max_view_tiles <= kMaxSharedTiles;
+        const cudaError_t e = launch_chained(chained(a), shared ? k_count<true> : k_count<false>, grid,
+                                             kChunkThreads, shared ? 4 * a.max_view_tiles : 0, st,
+                                             a);
+        if (e != cudaSuccess) return e;
     }
-    k_layout<<<1, kLayoutThreads, 0, st>>>(a.tile_count, a.n_tiles, a.max_pairs, a.ranges, a.order,
-                                           a.d_count, a.status, a.bin, a.warps, a.rec_cap,
-                                           a.n_rows);
-    return cudaGetLastError();
+    return launch_chained(chained(a), k_layout, dim3(1), kLayoutThreads, 0, st, a.tile_count, a.n_tiles,
+                          a.max_pairs, a.ranges, a.order, a.d_count, a.status, a.bin, a.warps,
+                          a.rec_cap, a.n_rows, a.refine);
 }
 
 cudaError_t launch_emit(const BinArgs &args, cudaStream_t st)
@@ -864,22 +876,23 @@ cudaError_t launch_emit(const BinArgs &args, cudaStream_t st)
     BinArgs a = args;
     if (a.n <= 0) return cudaSuccess;
     const dim3 grid = chunk_grid(a);
-    if (a.max_view_tiles <= kMaxSharedTiles)
-        k_emit<true><<<grid, kChunkThreads, 4 * a.max_view_tiles, st>>>(a);
-    else
-        k_emit<false><<<grid, kChunkThreads, 0, st>>>(a);
-    return cudaGetLastError();
+    const bool shared = a.max_view_tiles <= kMaxSharedTiles;
+    return launch_chained(chained(a), shared ? k_emit<true> : k_emit<false>, grid, kChunkThreads,
+                          shared ? 4 * a.max_view_tiles : 0, st, a);
 }
 
 cudaError_t launch_lists(const BinArgs &a, cudaStream_t st)
 {
     if (a.n <= 0) return cudaSuccess;
-    const cudaError_t e = prepare_lists();
+    cudaError_t e = prepare_lists();
     if (e != cudaSuccess) return e;
     // a list holds each primitive once: below kListCap primitives none is long
-    if (a.n >= kListCap) k_split<<<2 * a.sms, kSplitThreads, 0, st>>>(a);
-    k_lists<<<kListCtas * a.sms, kListThreads, sizeof(ListShared), st>>>(a);
-    return cudaGetLastError();
+    if (a.n >= kListCap) {
+        e = launch_chained(chained(a), k_split, dim3(2 * a.sms), kSplitThreads, 0, st, a);
+        if (e != cudaSuccess) return e;
+    }
+    return launch_chained(chained(a), k_lists, dim3(kListCtas * a.sms), kListThreads, sizeof(ListShared), st,
+                          a);
 }
 
 }  // namespace splat
