@@ -41,7 +41,8 @@ __device__ __forceinline__ uint32_t grow_weight(const GrowArgs &a, int64_t p)
     }
     const ViewDesc &vd = a.views[view_of(a.views, a.n_views, p)];
     const int64_t local = p - vd.pixel_offset;
-    const int r = static_cast<int>(local / vd.cols), c = static_cast<int>(local % vd.cols);
+    int r, c;
+    row_col(local, vd.cols, r, c);
     const float dx = a.t_depth[p - c + (c + 1 == vd.cols ? 0 : c + 1)];
     const float gx = dx > 0.0f ? __fsub_rn(dx, dt) : 0.0f;
     float gy = 0.0f;
@@ -131,16 +132,29 @@ __global__ void __launch_bounds__(1024) k_grow_top(const GrowArgs a)
     }
 }
 
-// #{j < n_d : floor((j Q + o) / n_d) < X} = clamp(ceil((X n_d - o) / Q), 0, n_d)
+// #{j < n_d : floor((j Q + o) / n_d) < X} = clamp(ceil((X n_d - o) / Q), 0, n_d).  The quotient
+// is at most about 2^24: a binary32 estimate (inv_q = 1 / Q) is within a few units of it, and the
+// exact remainder corrects it, at a third of a 64-bit division's instructions.
 __device__ __forceinline__ unsigned long long samples_below(unsigned long long X,
                                                             unsigned long long n_d,
                                                             unsigned long long Q,
-                                                            unsigned long long o)
+                                                            unsigned long long o, float inv_q)
 {
     const unsigned long long xn = X * n_d;
     if (xn <= o) return 0ull;
-    const unsigned long long c = (xn - o + Q - 1ull) / Q;
-    return c < n_d ? c : n_d;
+    const unsigned long long num = xn - o + Q - 1ull;
+    long long c = static_cast<long long>(static_cast<float>(num) * inv_q);
+    long long rem = static_cast<long long>(num) - c * static_cast<long long>(Q);
+    while (rem < 0) {
+        --c;
+        rem += static_cast<long long>(Q);
+    }
+    while (rem >= static_cast<long long>(Q)) {
+        ++c;
+        rem -= static_cast<long long>(Q);
+    }
+    const unsigned long long u = static_cast<unsigned long long>(c);
+    return u < n_d ? u : n_d;
 }
 
 __device__ __forceinline__ void write_empty(const GrowArgs &a, int64_t j)
@@ -156,7 +170,8 @@ __device__ __forceinline__ void write_primitive(const GrowArgs &a, int64_t j, in
 {
     const ViewDesc &vd = a.views[view_of(a.views, a.n_views, p)];
     const int64_t local = p - vd.pixel_offset;
-    const int r = static_cast<int>(local / vd.cols), c = static_cast<int>(local % vd.cols);
+    int r, c;
+    row_col(local, vd.cols, r, c);
     const float d = a.t_depth[p];
     const float3 v = pixel_ray(vd, r, c);
     const float *R = vd.R_hi;   // T^c_w: p_s = R p_w + t, so p_w = R^T (p_s - t)
@@ -200,15 +215,19 @@ __global__ void __launch_bounds__(kGrowThreads) k_grow_select(const GrowArgs a)
     const int64_t lo = static_cast<int64_t>(blockIdx.x) * a.chunk;
     const int64_t hi = lo + a.chunk < a.n_pixels ? lo + a.chunk : a.n_pixels;
     unsigned long long base = a.block_sums[blockIdx.x];
+    const float inv_q = 1.0f / static_cast<float>(Q);
     for (int64_t p0 = lo; p0 < hi; p0 += kGrowThreads) {   // uniform trip count per block
         const int64_t p = p0 + threadIdx.x;
         const unsigned long long q = p < hi ? a.q[p] : 0u;
         unsigned long long tile_total;
         const unsigned long long C = base + block_exclusive_scan(q, s_warp, &tile_total);
         base += tile_total;
+        // a pixel's samples begin where its predecessor's end: one quotient a pixel, one more for
+        // each warp's first
+        const unsigned long long j1 = samples_below(C + q, n_d, Q, o, inv_q);
+        unsigned long long j0 = __shfl_up_sync(0xFFFFFFFFu, j1, 1);
+        if ((threadIdx.x & 31) == 0) j0 = samples_below(C, n_d, Q, o, inv_q);
         if (q == 0ull) continue;
-        const unsigned long long j0 = samples_below(C, n_d, Q, o);
-        const unsigned long long j1 = samples_below(C + q, n_d, Q, o);
         if (j1 > j0) {
             write_primitive(a, static_cast<int64_t>(j0), p);
             for (unsigned long long j = j0 + 1; j < j1; ++j) write_empty(a, static_cast<int64_t>(j));

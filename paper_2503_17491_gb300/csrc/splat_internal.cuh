@@ -71,6 +71,16 @@ struct ViewDesc {
     float cull_t_top, cull_l_top, cull_t_bot, cull_l_bot;
 };
 
+// Row and column of pixel `local` of a view: a view has at most 32,767^2 pixels, so the quotient
+// is a 32-bit one (a 64-bit one costs about four times the instructions).
+__device__ __forceinline__ void row_col(int64_t local, int cols, int &r, int &c)
+{
+    const uint32_t l = static_cast<uint32_t>(local), w = static_cast<uint32_t>(cols);
+    const uint32_t q = l / w;
+    r = static_cast<int>(q);
+    c = static_cast<int>(l - q * w);
+}
+
 // Pixel-centre ray of pixel (r, c) of a view (Sec. 3.1), binary32.
 __device__ __forceinline__ float3 pixel_ray(const ViewDesc &vd, int r, int c)
 {

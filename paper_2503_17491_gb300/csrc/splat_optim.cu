@@ -160,7 +160,8 @@ __global__ void __launch_bounds__(256) k_loss(const float *__restrict__ depth,
         if (kNormalMode == 1 && view_on && lambda_n != 0.0f) {
             const ViewDesc &vd = views[v];
             const int64_t local = p - vd.pixel_offset;
-            const int r = static_cast<int>(local / vd.cols), c = static_cast<int>(local % vd.cols);
+            int r, c;
+            row_col(local, vd.cols, r, c);
             const Rays3x3 rays = rays_around(vd, r, c);
             const float3 vp = rays.ray(1, 1);
             const Stencil s0 = normal_stencil(vd, r, c, rays, 1, 1, depth, normal, t_depth, n,
@@ -371,7 +372,8 @@ __global__ void k_backproject(const ViewDesc *__restrict__ views, int n_views, i
     while (v + 1 < n_views && views[v + 1].pixel_offset <= k) ++v;
     const ViewDesc &vd = views[v];
     const int64_t local = k - vd.pixel_offset;
-    const int r = static_cast<int>(local / vd.cols), c = static_cast<int>(local % vd.cols);
+    int r, c;
+    row_col(local, vd.cols, r, c);
     const float O = alpha[k];
     float px = __int_as_float(0x7FC00000), py = px, pz = px;
     if (O >= o_min) {
