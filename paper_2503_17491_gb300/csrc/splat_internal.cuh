@@ -64,7 +64,6 @@ struct ViewDesc {
     int32_t tiles_r, tiles_c;     // tile rows / columns of this view
     int64_t tile_offset;          // first global tile id of the view
     int64_t pixel_offset;         // first pixel of the view in the packed buffers
-    int32_t table_offset;         // into the frame table: tiles_r rows then tiles_c columns
     int32_t pix_offset;           // into the pixel-frame table: tiles_r x 256 entries
     // cones two rows (and a milliradian) beyond the top and bottom rows: z = t |xy|, with
     // l = sqrt(1 + t^2) the Lipschitz constant of z - t |xy| (l = inf: no cone)
@@ -169,12 +168,6 @@ inline void set_cull_cones(ViewDesc &vd, double emin, double emax, double dtheta
                                                     1.0001)
                                : INFINITY;
 }
-
-// Frame table entry (float pairs of FP64 sin / cos): per tile row sin/cos of the reference
-// elevation theta0, per tile column sin/cos of the reference azimuth gamma0.
-struct SinCos2 {
-    float s_hi, s_lo, c_hi, c_lo;
-};
 
 // Pixel ray planes of one pixel in its tile's frame (FP64 values as float pairs): h_x, h_y
 // (hi parts and the remainders) and the ray direction v (hi only).  One entry per (view, tile

@@ -140,7 +140,6 @@ int build_tables(const double *T, const splat_lidar_intrinsics &in, int th, int 
     vd.tiles_c = tiles_c;
     vd.tile_offset = 0;
     vd.pixel_offset = 0;
-    vd.table_offset = 0;
     vd.pix_offset = 0;
     for (int tr = 0; tr < tiles_r; ++tr) {
         const double t0 = emax - (tr * th + 0.5 * (th - 1)) * dth;
