@@ -102,7 +102,7 @@ struct splat_ctx {
     // workspace
     uint64_t *d_prect = nullptr;   // pair pixel rectangles with the normal-flip bit
     // touching pairs by view and block of primitives: tile rectangles, range keys, counts
-    uint64_t *d_touch = nullptr;
+    uint2 *d_touch = nullptr;
     float *d_kappa = nullptr;
     uint32_t *d_touch_count = nullptr;
     uint32_t *d_cta_count = nullptr;

@@ -256,20 +256,20 @@ inline int64_t max_project_blocks(int64_t n)
 }
 
 // A touching pair in its block's segment: its tile rectangle and its primitive's place in the
-// block, 64 bits.  Images have at most 32,767 rows and columns and tiles at least 4 rows and 8
-// columns: at most 8,192 tile rows and 4,096 tile columns.
-__device__ __forceinline__ uint64_t pack_touch(const TileRect &t, uint32_t local)
+// block, in two 32-bit words.  Images have at most 32,767 rows and columns and tiles at least 4
+// rows and 8 columns: at most 8,192 tile rows and 4,096 tile columns.
+__device__ __forceinline__ uint2 pack_touch(const TileRect &t, uint32_t local)
 {
-    return static_cast<uint64_t>(t.r0) | static_cast<uint64_t>(t.nr) << 13 |
-           static_cast<uint64_t>(t.c0) << 27 | static_cast<uint64_t>(t.nc) << 39 |
-           static_cast<uint64_t>(local) << 52;
+    return make_uint2(static_cast<uint32_t>(t.r0) | static_cast<uint32_t>(t.nr) << 13 | local << 27,
+                      static_cast<uint32_t>(t.c0) | static_cast<uint32_t>(t.nc) << 12 |
+                          local >> 5 << 25);
 }
 
-__device__ __forceinline__ TileRect unpack_touch(uint64_t w, uint32_t &local)
+__device__ __forceinline__ TileRect unpack_touch(uint2 w, uint32_t &local)
 {
-    local = static_cast<uint32_t>(w >> 52);
-    return TileRect{static_cast<int>(w & 0x1FFFu), static_cast<int>(w >> 13 & 0x3FFFu),
-                    static_cast<int>(w >> 27 & 0xFFFu), static_cast<int>(w >> 39 & 0x1FFFu)};
+    local = w.x >> 27 | w.y >> 25 << 5;
+    return TileRect{static_cast<int>(w.x & 0x1FFFu), static_cast<int>(w.x >> 13 & 0x3FFFu),
+                    static_cast<int>(w.y & 0xFFFu), static_cast<int>(w.y >> 12 & 0x1FFFu)};
 }
 
 // the tiles a record's pixel rectangle meets: columns c0 .. c0 + nc - 1 (mod W), wrapping past
@@ -443,7 +443,7 @@ struct ProjectArgs {
     int block_prims;        // set by the launcher
     // per (view, block): its touching pairs from place view * n + block's first primitive on,
     // their range keys, and how many there are (view * project_blocks(n) + block)
-    uint64_t *touch;
+    uint2 *touch;
     float *kappa;
     uint32_t *touch_count;
     float4 *prim;
@@ -479,7 +479,8 @@ struct BinArgs {
     int tile_h, tile_w;
     int64_t n_tiles;
     const TileInfo *tiles;
-    const uint64_t *prect, *touch;
+    const uint64_t *prect;
+    const uint2 *touch;
     const float *kappa;
     const uint32_t *touch_count;
     int64_t max_pairs;
@@ -513,7 +514,10 @@ inline int64_t cta_count_words(int sms, int max_views, int64_t max_tiles)
            (max_tiles < kMaxSharedTiles ? max_tiles : kMaxSharedTiles);
 }
 // kBinSplit4, kBinSplit2: RenderArgs::split
-enum { kBinLong = 0, kBinMid, kBinSegments, kBinQueueSeg, kBinSplit4, kBinSplit2, kBinWords };
+// kBinOver: the entries exceed the capacity
+enum {
+    kBinLong = 0, kBinMid, kBinSegments, kBinQueueSeg, kBinSplit4, kBinSplit2, kBinOver, kBinWords
+};
 cudaError_t prepare_lists();    // before the first launch_lists on a device
 int bin_launches(int64_t n);    // kernels these three run for n primitives
 cudaError_t launch_bin_counts(const BinArgs &a, cudaStream_t st);   // count and layout

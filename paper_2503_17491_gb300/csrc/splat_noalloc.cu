@@ -280,7 +280,7 @@ extern "C" SPLAT_API int splat_render_noalloc(const splat_gaussians *g,
     pa.tile_w = tw;
     pa.flip_normals = cfg.flip_normals;
     pa.prect = reinterpret_cast<uint64_t *>(base + kOffPrect);
-    pa.touch = reinterpret_cast<uint64_t *>(base + kOffTouch);
+    pa.touch = reinterpret_cast<uint2 *>(base + kOffTouch);
     pa.kappa = reinterpret_cast<float *>(base + kOffKappa);
     pa.touch_count = reinterpret_cast<uint32_t *>(base + kOffTouchCount);
     pa.prim = prim;
