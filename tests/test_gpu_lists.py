@@ -103,3 +103,63 @@ def test_split_blocks(tile):
     assert ctx.status() == 0 and whole.status() == 0
     for x, y in zip(ga, gb):
         assert (x - y).abs().max() <= 1e-5 * y.abs().max()
+
+
+def test_many_tiles():
+    """A view of more tiles than the shared-memory counters hold (14,000), beside one of few: both
+    in one call."""
+    s = scenes.tiny_scene(3000, 5, rows=112, cols=32_000, dist=(0.6, 9.0), log_scale=(-5.0, -1.0))
+    few = scenes.View(np.eye(4), 16, 64, scenes.deg(-20), scenes.deg(20))
+    views = [s.views[0], few]
+    ctx = make_ctx(s.n, views, (16, 16), max_pairs=1 << 21)
+    ctx.render(*to_dev(s))
+    assert ctx.status() == 0
+    assert check_lists(ctx, s, views, (16, 16)) > s.n
+
+
+def _rotation(rng):
+    q = rng.normal(size=4)
+    w, x, y, z = q / np.linalg.norm(q)
+    return np.array([[1 - 2 * (y * y + z * z), 2 * (x * y - w * z), 2 * (x * z + w * y)],
+                     [2 * (x * y + w * z), 1 - 2 * (x * x + z * z), 2 * (y * z - w * x)],
+                     [2 * (x * z - w * y), 2 * (y * z + w * x), 1 - 2 * (x * x + y * y)]])
+
+
+@pytest.mark.parametrize("kind", ["edge_on", "thin", "near", "far", "axes", "boundaries"])
+@pytest.mark.parametrize("tile", [(16, 16), (4, 64)])
+def test_boxes(kind, tile):
+    """The projection's approximate box against the contract's where the bounds lie badly: planes
+    seen edge on, slivers, primitives around and behind the sensor, far below a pixel, centres on
+    the axes, poles and seam, and centres on pixel boundaries; from a level and two tilted poses,
+    a narrow, a wide and a whole-sphere field of view."""
+    rng = np.random.default_rng(len(kind) + tile[0])
+    n = 6000
+    g = rng.uniform(-math.pi, math.pi, n)
+    th = np.arcsin(rng.uniform(-1, 1, n))
+    r = np.exp(rng.uniform(math.log(0.05 if kind == "near" else 1.0),
+                           math.log({"near": 1.5, "far": 400.0}.get(kind, 40.0)), n))
+    if kind == "axes":
+        g = rng.integers(-2, 3, n) * (math.pi / 2)
+        th = rng.choice([0.0, 0.0, math.pi / 2, -math.pi / 2], n)
+    if kind == "boundaries":
+        g = math.pi - 2 * math.pi * rng.integers(0, 333, n) / 333
+        th = math.radians(20) - math.radians(40) * rng.integers(0, 46, n) / 45
+    p = np.stack([np.cos(th) * np.cos(g), np.cos(th) * np.sin(g), np.sin(th)], 1) * r[:, None]
+    nrm = np.cross(p, rng.normal(size=(n, 3))) if kind == "edge_on" else rng.normal(size=(n, 3))
+    pl, q, ls = scenes.gaussians_on(
+        p, nrm, rng, jitter=0.0, quat_noise=0.0 if kind == "edge_on" else 0.05,
+        log_scale=(-5.0, -2.5) if kind == "far" else (-3.5, -0.5))
+    if kind == "thin":
+        ls[:, 1] -= 6.0
+    views = []
+    for k, (rows, cols, fov) in enumerate([(45, 333, 20), (64, 128, 89), (33, 1000, 89.9)]):
+        T = np.eye(4)
+        if k:
+            T[:3, :3] = _rotation(rng)
+            T[:3, 3] = rng.normal(0, 0.3, 3)
+        views.append(scenes.View(T, rows, cols, scenes.deg(-fov), scenes.deg(fov)))
+    s = scenes.Scene(f"boxes_{kind}", pl, q, ls, views)
+    ctx = make_ctx(s.n, views, tile, max_pairs=1 << 22)
+    ctx.render(*to_dev(s))
+    assert ctx.status() == 0
+    assert check_lists(ctx, s, views, tile) > 0
