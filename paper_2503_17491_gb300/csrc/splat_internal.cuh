@@ -458,9 +458,9 @@ cudaError_t launch_records(int64_t n, int n_views, const ViewDesc *views, int fl
                            int tile_h, int tile_w, const float4 *prim, const uint64_t *prect,
                            const uint8_t *active, PairRec *recs, cudaStream_t st);
 
-// Binning (splat_sort.cu): from the projection's pixel rectangles to the per-tile lists in (range, id)
-// order, [start, end) per tile and the work order.  A list of more than kListCap entries is cut
-// into segments of at most kListCap before it is sorted.
+// Binning (splat_sort.cu): from the projection's pixel rectangles to the per-tile lists in
+// (range, id) order, [start, end) per tile and the work order.  A list of more than kListCap
+// entries is cut into segments of at most kListCap before it is sorted.
 constexpr int kListCap = 4096;
 constexpr int kSegTarget = kListCap / 2;
 struct ListSegment {

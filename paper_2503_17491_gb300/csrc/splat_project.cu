@@ -1,7 +1,7 @@
 // K1: per-primitive projection for every registered view -- the range key, the sign that turns
 // the normal towards the sensor, and the conservative spherical bounding box of the region of the
-// 3-sigma box where the primitive can reach alpha_min, with its tile rectangle (Sec. 3.2.1 tiles and range sort; Sec. 3.2.3 bounding
-// box computation; Supp. B).
+// 3-sigma box where the primitive can reach alpha_min, with its tile rectangle (Sec. 3.2.1 tiles
+// and range sort; Sec. 3.2.3 bounding box computation; Supp. B).
 //
 // Everything in this file takes integer decisions (which tiles, which order, which sign), so it
 // follows a fixed binary32 contract: every value is produced by the same sequence of correctly
@@ -17,9 +17,10 @@
 // integers, and wherever the approximate bounds of all four lie clear of the next pixel by more
 // than both computations' errors the integers are already known.  The few pairs left (a bound
 // within a few thousandths of a pixel of a boundary, near or steep primitives: 1 % of the
-// pairs along a long street, 3-4 % in a street or block) are queued per warp
-// and boxed by the contract 32 at a time.  Projection of 12 x 500 k pairs: 0.214
-// -> 0.181 ms; of 8 x 1 M pairs along a 600 m street: 0.278 -> 0.188 ms.
+// pairs along a long street, 3-4 % in a street or block) are queued per warp and boxed by the
+// contract 32 at a time.  Projection of 12 x 500 k pairs: 0.214 -> 0.19 ms, in a refinement with
+// the gradient accumulators zeroed on the way; of 8 x 1 M pairs along a 600 m street: 0.278
+// -> 0.188 ms.  Issue bound (74 % of the slots, 640 instructions per warp and view).
 //
 // A pair leaves its pixel rectangle with the normal-flip bit (8 bytes, zero when it touches no
 // tile).  A pair that touches a tile also appends its tile rectangle and range key (12 bytes) to
@@ -747,7 +748,8 @@ cudaError_t launch_project(const ProjectArgs &a, cudaStream_t st)
     if (a.n <= 0) return cudaSuccess;
     ProjectArgs b = a;
     b.block_prims = block_prims(a.n);
-    return launch_chained(chained_size(a.n * a.n_views), k_project, dim3(static_cast<unsigned>(project_blocks(a.n))),
+    return launch_chained(chained_size(a.n * a.n_views), k_project,
+                          dim3(static_cast<unsigned>(project_blocks(a.n))),
                           kProjectThreads, sizeof(ProjectShared), st, b);
 }
 

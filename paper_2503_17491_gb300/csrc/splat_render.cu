@@ -9,11 +9,11 @@
 // list is one serial chain (the transmittance), so a block's time grows with its list: the blocks
 // of the lists that are long against a warp's share of the frame go to two or four warps, each
 // with its own pixels (one 64 x 1024 scan over 100,000 primitives: forward 0.125 -> 0.066 ms,
-// backward 0.112 -> 0.048 ms; eight 128 x 1024 scans along a street: forward 0.446 -> 0.319 ms).  Warps never wait for
-// one another.  A warp walks its tile's slice of the sorted list (Sec. 3.2.1) 32 entries at a
-// time -- every lane reads one entry's projection record and tests whether the primitive's pixel
-// rectangle meets the warp's block -- and stages the entries that do, 32 at a time, into shared
-// memory.  A staged batch is then evaluated pair-parallel: the (primitive, pixel) candidates --
+// backward 0.112 -> 0.048 ms; eight 128 x 1024 scans along a street: forward 0.446 -> 0.319 ms).
+// Warps never wait for one another.  A warp walks its tile's slice of the sorted list (Sec. 3.2.1),
+// tests each entry's packed rectangle inside the tile against its block, and stages the entries
+// that meet it, 32 at a time, into shared memory.  A staged batch is then evaluated
+// pair-parallel: the (primitive, pixel) candidates --
 // every pixel of the block inside a staged primitive's rectangle that is still live -- are
 // numbered primitive-major (a prefix sum of the per-primitive counts; each primitive's lane
 // writes its candidates into a shared list), and each round gives one candidate to every lane,
@@ -352,7 +352,8 @@ __device__ __forceinline__ uint32_t next_item(uint32_t *queue, int lane)
 
 // Work items of the frame: the first n4 tiles of the work order give 32 items each, the next n2
 // tiles 16, the rest 8: a tile's eight 4 x 8 blocks, whole, in halves of two rows or row by row
-// (the layout kernel of the binning chooses).  An item's pixels are those of the lanes with lane >> shift == sub.
+// (the layout kernel of the binning chooses).  An item's pixels are those of the lanes with
+// lane >> shift == sub.
 struct Item {
     uint32_t place;   // of the tile in the work order
     int blk, sub, shift;

@@ -19,8 +19,8 @@
 // Why not a global radix sort: sorting all pairs by range and the entries by tile takes four plus
 // two passes of three launches each, whose per-tile ranking is one serial chain of shared memory
 // per warp; here an entry is written once and read by the list sort, in five launches.  From
-// pairs to lists, 12 views x 500 k primitives (5.3 M entries): 0.51 ms in 24 launches -> 0.22 ms
-// (count 0.031, layout 0.007, emission 0.066, split 0.025, lists 0.105); 64 tiles of 1,500
+// pairs to lists, 12 views x 500 k primitives (5.3 M entries): 0.51 ms in 24 launches -> 0.23 ms
+// (count 0.032, layout 0.010, emission 0.062, split 0.024, lists 0.097); 64 tiles of 1,500
 // entries: 0.13 -> 0.022 ms.  The lists stage is bound by the shared-memory latency of its four
 // passes over the keys, the counting stages by instruction issue.
 // Everything runs on counts that stay on the device, with fixed launch shapes, so the pipeline
@@ -681,9 +681,9 @@ __device__ __forceinline__ uint32_t get_bin(const uint32_t *bins, uint32_t b)
 // then ranked against the other keys of its bin -- one or two on lists whose ranges spread.  A
 // list with a bin above kMaxInBin (a wall behind a near object) is merge sorted.  The keys are
 // read three times rather than held: they stay in L1, and short loops keep the code in the
-// instruction cache.  24 warps with 52 KB a CTA leave 72 KB of L1, which bounds the misses in flight:
-// with the rectangles gathered into shared memory as well (68 KB a CTA) the stage took 0.178 ms
-// instead of 0.121 on 5.3 M entries, with four CTAs per SM 0.157.
+// instruction cache.  24 warps with 52 KB a CTA leave 72 KB of L1, which bounds the misses in
+// flight: with the rectangles gathered into shared memory as well (68 KB a CTA) the stage took
+// 0.178 ms instead of 0.121 on 5.3 M entries, with four CTAs per SM 0.157.
 template <int G>
 __device__ __forceinline__ void sort_list(const BinArgs &A, const uint64_t *src, uint32_t start,
                                           int n, uint32_t tile, uint64_t *key,
