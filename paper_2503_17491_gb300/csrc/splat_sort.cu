@@ -101,12 +101,15 @@ __device__ __forceinline__ T block_excl_scan(T v, T *s_warp, T *total)
 //   eight 128x1024 along a street, 3 shares             .446      | .315      | .318
 //   128x2048, 1 M, urban block, 2.1 shares              .249 .225 |           | .274 .250
 //   12 keyframes, 500 k, 1.8 shares                     .729 .816 |           | .768 .842
-// Where even the longest list is below about kSplitFrom shares (the last two) the queue evens the
-// warps out by itself and splitting only costs, so such a frame is left whole.
+// Where even the longest list is below kSplitFrom shares the queue evens the warps out by itself
+// and splitting only costs, so such a frame is left whole: the whole pass at 2.44 and 2.51 shares
+// (128x2048, 1 M, forward and backward) 0.66 whole, 0.69 split; at 2.76 and 2.78 (eight 128x1024,
+// forward) 0.76 whole, 0.69 split.  The longest list is taken exactly: rounded up to a bucket the
+// line lay anywhere up to 3.1 shares.
 // A split block keeps one contributor record per part and primitive, so nothing is split when the
 // record pool might not hold one record for every row of 8 pixels that every pair meets (n_rows
 // counts those): the pool then overflows for no frame that it held unsplit.
-constexpr float kSplit2Share = 0.4f, kSplit4Share = 0.8f, kSplitFrom = 2.5f;
+constexpr float kSplit2Share = 0.4f, kSplit4Share = 0.8f, kSplitFrom = 2.65f;
 constexpr uint32_t kSplitLeast = 64;
 
 __global__ void __launch_bounds__(kLayoutThreads) k_layout(
@@ -117,23 +120,28 @@ __global__ void __launch_bounds__(kLayoutThreads) k_layout(
 {
     chain_wait();
     __shared__ unsigned long long s_warp[33];
-    __shared__ uint32_t s_cnt[kBuckets], s_off[kBuckets];
+    __shared__ uint32_t s_cnt[kBuckets], s_off[kBuckets], s_longest;
     const int tid = threadIdx.x, lane = tid & 31;
     if (tid < kBuckets) s_cnt[tid] = 0;
+    if (tid == 0) s_longest = 0;
     __syncthreads();
     // each thread takes a run of consecutive tiles; the loop bounds are uniform so that the
     // whole warp takes part in the matches
     const int64_t per = (n_tiles + kLayoutThreads - 1) / kLayoutThreads;
     const int64_t t0 = per * tid;
     unsigned long long sum = 0;
+    uint32_t longest = 0;
     for (int64_t k = 0; k < per; ++k) {
         const bool in = t0 + k < n_tiles;
         const uint32_t len = in ? tile_count[t0 + k] : 0u;
         sum += len;
+        longest = max(longest, len);
         const int b = in ? len_bucket(len) : kBuckets;
         const uint32_t peers = __match_any_sync(kFull, b);
         if (in && lane == __ffs(peers) - 1) atomicAdd(&s_cnt[b], __popc(peers));
     }
+    longest = __reduce_max_sync(kFull, longest);
+    if (lane == 0 && longest) atomicMax(&s_longest, longest);
     unsigned long long total;
     const unsigned long long run0 = block_excl_scan<kLayoutThreads>(sum, s_warp, &total);
     __syncthreads();
@@ -155,7 +163,7 @@ __global__ void __launch_bounds__(kLayoutThreads) k_layout(
                                                          fminf(share * x, 2147483647.0f))))];
         };
         uint32_t n4 = tiles_above(kSplit4Share), n2 = tiles_above(kSplit2Share) - n4;
-        if (tiles_above(kSplitFrom) == 0u) n4 = n2 = 0u;
+        if (static_cast<float>(s_longest) < share * kSplitFrom) n4 = n2 = 0u;
         const unsigned long long items =
             8ull * (static_cast<unsigned long long>(n_tiles) + n2 + 3ull * n4);
         if (rec_cap && *n_rows / 32 + items > rec_cap) n4 = n2 = 0u;
