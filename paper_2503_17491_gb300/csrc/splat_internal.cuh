@@ -1,6 +1,7 @@
 // Internal definitions shared by the translation units of libsplatloam (not part of the ABI).
 #pragma once
 
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -48,6 +49,30 @@ cudaError_t launch_chained(bool chain, void (*kernel)(P...), dim3 grid, unsigned
     cfg.numAttrs = chain ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
+
+// Raises a kernel's dynamic shared memory limit above the default 48 KB, once on each device: the
+// attribute belongs to the current device's copy of the kernel.  One static object per kernel; a
+// failed call is tried again by the next one.
+class SharedLimit {
+public:
+    template <typename Kernel>
+    cudaError_t raise(Kernel *kernel, size_t bytes)
+    {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        const bool known = dev >= 0 && dev < kDevices;
+        if (known && done_[dev].load(std::memory_order_acquire)) return cudaSuccess;
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 static_cast<int>(bytes));
+        if (e == cudaSuccess && known) done_[dev].store(true, std::memory_order_release);
+        return e;
+    }
+
+private:
+    static constexpr int kDevices = 64;
+    std::atomic<bool> done_[kDevices] = {};
+};
 
 // ---------------------------------------------------------------------------------------------
 // per-view descriptor (device)
@@ -518,7 +543,7 @@ inline int64_t cta_count_words(int sms, int max_views, int64_t max_tiles)
 enum {
     kBinLong = 0, kBinMid, kBinSegments, kBinQueueSeg, kBinSplit4, kBinSplit2, kBinOver, kBinWords
 };
-cudaError_t prepare_lists();    // before the first launch_lists on a device
+cudaError_t prepare_lists();    // once per device, before its first launch_lists
 int bin_launches(int64_t n);    // kernels these three run for n primitives
 cudaError_t launch_bin_counts(const BinArgs &a, cudaStream_t st);   // count and layout
 cudaError_t launch_emit(const BinArgs &a, cudaStream_t st);

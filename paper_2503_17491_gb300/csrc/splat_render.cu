@@ -1110,23 +1110,19 @@ cudaError_t dispatch(int th, int tw, K k)
 
 }  // namespace
 
-// both kernels' shared memory is above the 48 KB static limit: allow it once per instantiation
+// both kernels' shared memory is above the 48 KB static limit: allow it for every instantiation
 template <int TH, int TW>
 cudaError_t fwd_prepare()
 {
-    static cudaError_t e = cudaFuncSetAttribute(k_render_fwd<TH, TW>,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                static_cast<int>(sizeof(FwdShared)));
-    return e;
+    static SharedLimit limit;
+    return limit.raise(k_render_fwd<TH, TW>, sizeof(FwdShared));
 }
 
 template <int TH, int TW>
 cudaError_t bwd_prepare()
 {
-    static cudaError_t e = cudaFuncSetAttribute(k_render_bwd<TH, TW>,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                static_cast<int>(sizeof(BwdShared)));
-    return e;
+    static SharedLimit limit;
+    return limit.raise(k_render_bwd<TH, TW>, sizeof(BwdShared));
 }
 
 cudaError_t launch_render_fwd(const RenderArgs &a, int tile_h, int tile_w, int grid,

@@ -878,12 +878,11 @@ bool chained(const BinArgs &a) { return chained_size(a.n * a.n_views); }
 
 }  // namespace
 
-// k_lists' shared memory is above the 48 KB static limit: allow it once
+// k_lists' shared memory is above the 48 KB static limit
 cudaError_t prepare_lists()
 {
-    static const cudaError_t e = cudaFuncSetAttribute(
-        k_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(ListShared)));
-    return e;
+    static SharedLimit limit;
+    return limit.raise(k_lists, sizeof(ListShared));
 }
 
 int bin_launches(int64_t n) { return n >= kListCap ? 5 : 4; }
