@@ -636,7 +636,7 @@ int render_occupancy(int tile_h, int tile_w, bool backward);
 
 cudaError_t launch_param_grads(const float4 *pos_logit, const float4 *quat, const float2 *log_scale,
                                const float4 *wgrad, int64_t n, float4 *g_pos_logit, float4 *g_quat,
-                               float2 *g_log_scale, int accumulate, cudaStream_t st);
+                               float2 *g_log_scale, int accumulate, cudaStream_t st, bool chain);
 
 // active (nullable): pixels of views with active[v] == 0 count as invalid (views: the registered
 // views, for the pixel -> view lookup).  normal_mode 0: normal term against t_normal; 1:
