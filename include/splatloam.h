@@ -411,9 +411,10 @@ SPLAT_API int splat_get_stats(splat_ctx *ctx, splat_stats *out);
 SPLAT_API int splat_set_profiling(splat_ctx *ctx, int enable);
 SPLAT_API int splat_kernel_times(splat_ctx *ctx, float *fwd_ms, float *bwd_ms);
 /* With profiling enabled: the durations (ms, waiting for the events) of the stages of the last
- * profiled render and refinement step, ms[7] = projection, (no stage), emission (count, layout,
- * emit), list sort, (no stage), loss, fused Adam; -1 for a stage not recorded since profiling was
- * enabled (the last two come from splat_refine_step only) and for the two places without a stage.
+ * profiled render and refinement step, ms[7] = projection, range sort, emission (count, layout,
+ * emit), list sort, tile ranges, loss, fused Adam; -1 for a stage not recorded since profiling was
+ * enabled (the last two come from splat_refine_step only).  The lists are sorted tile by tile:
+ * range sort and tile ranges are not passes of their own and give 0.
  * Errors: INVALID_ARG, CUDA. */
 SPLAT_API int splat_stage_times(splat_ctx *ctx, float *ms);
 

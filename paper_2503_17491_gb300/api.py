@@ -327,8 +327,8 @@ class SplatContext:
 
     def stage_times(self) -> dict:
         """Durations (ms) of the stages of the last profiled render / refinement step
-        (splat_stage_times); None for a stage not recorded ("range sort" and "tile ranges" name
-        no stage any more: the lists are sorted per tile)."""
+        (splat_stage_times); None for a stage not recorded.  "range sort" and "tile ranges" take
+        no time: the lists are sorted tile by tile."""
         ms = (ctypes.c_float * 7)()
         _lib.check(self.lib.splat_stage_times(self.h, ms), "splat_stage_times")
         return {k: (float(v) if v >= 0 else None) for k, v in zip(self.STAGES, ms)}

@@ -1086,25 +1086,25 @@ SPLAT_API int splat_stage_times(splat_ctx *ctx, float *ms)
 {
     if (!ctx || !ms) return SPLAT_ERR_INVALID_ARG;
     // the loss runs between the end of the forward compositing and event 6, the fused Adam
-    // between the end of the backward and event 7; binning has no global range sort and no
-    // separate ranges pass
+    // between the end of the backward and event 7; the binning has no global range sort and no
+    // separate ranges pass, which take no time in a render that was profiled
     struct Span {
         cudaEvent_t a, b;
         bool ok;
     };
-    const Span none{nullptr, nullptr, false};
+    const Span binning{nullptr, nullptr, ctx->stage_rec[0] && ctx->stage_rec[4]};
     const Span spans[7] = {
         {ctx->stage_ev[0], ctx->stage_ev[1], ctx->stage_rec[0] && ctx->stage_rec[1]},
-        none,
+        binning,
         {ctx->stage_ev[1], ctx->stage_ev[3], ctx->stage_rec[1] && ctx->stage_rec[3]},
         {ctx->stage_ev[3], ctx->stage_ev[4], ctx->stage_rec[3] && ctx->stage_rec[4]},
-        none,
+        binning,
         {ctx->ev[1], ctx->stage_ev[6], ctx->rec_fwd && ctx->stage_rec[6]},
         {ctx->ev[3], ctx->stage_ev[7], ctx->rec_bwd && ctx->stage_rec[7]},
     };
     for (int k = 0; k < 7; ++k) {
-        ms[k] = -1.0f;
-        if (!spans[k].ok) continue;
+        ms[k] = spans[k].ok ? 0.0f : -1.0f;
+        if (!spans[k].ok || !spans[k].a) continue;
         CK(cudaEventSynchronize(spans[k].b));
         CK(cudaEventElapsedTime(&ms[k], spans[k].a, spans[k].b));
     }

@@ -105,3 +105,14 @@ def test_chained_launches_follow_the_pairs(host, n, views, chained):
     host.lib.fake_clear()
     assert host.render() == 0 and host.backward() == 0
     assert {x["chained"] for x in host.launches()} == {chained}
+
+
+def test_stage_times_of_a_profiled_render_add_up(host):
+    """Every stage of a profiled render has a time (the two that the binning no longer has take
+    none), so that the values can be summed; what was not recorded gives -1."""
+    assert host.create(100) == 0
+    ms = (ctypes.c_float * 7)()
+    assert host.lib.splat_stage_times(host.ctx, ms) == 0 and list(ms) == [-1.0] * 7
+    assert host.lib.splat_set_profiling(host.ctx, 1) == 0 and host.render() == 0
+    assert host.lib.splat_stage_times(host.ctx, ms) == 0
+    assert list(ms) == [1.0, 0.0, 1.0, 1.0, 0.0, -1.0, -1.0]
