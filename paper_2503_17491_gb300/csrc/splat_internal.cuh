@@ -34,29 +34,46 @@ constexpr int64_t kChainPairs = int64_t{1} << 19;
 inline bool chained_size(int64_t pairs) { return pairs <= kChainPairs; }
 
 template <typename... P, typename... A>
-cudaError_t launch_chained(bool chain, void (*kernel)(P...), dim3 grid, unsigned block, size_t smem,
-                           cudaStream_t st, const A &...args)
+cudaError_t launch_cluster(bool chain, int cluster, void (*kernel)(P...), dim3 grid, unsigned block,
+                           size_t smem, cudaStream_t st, const A &...args)
 {
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2] = {};
+    unsigned n = 0;
+    if (chain) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = static_cast<unsigned>(cluster);
+        attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
+        ++n;
+    }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cfg.attrs = &attr;
-    cfg.numAttrs = chain ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
+template <typename... P, typename... A>
+cudaError_t launch_chained(bool chain, void (*kernel)(P...), dim3 grid, unsigned block, size_t smem,
+                           cudaStream_t st, const A &...args)
+{
+    return launch_cluster(chain, 1, kernel, grid, block, smem, st, args...);
+}
+
 // Raises a kernel's dynamic shared memory limit above the default 48 KB, once on each device: the
-// attribute belongs to the current device's copy of the kernel.  One static object per kernel; a
-// failed call is tried again by the next one.
+// attribute belongs to the current device's copy of the kernel.  carveout (percent, negative for
+// the driver's choice): how much of an SM's memory is shared, the rest is L1.  One static object
+// per kernel; a failed call is tried again by the next one.
 class SharedLimit {
 public:
     template <typename Kernel>
-    cudaError_t raise(Kernel *kernel, size_t bytes)
+    cudaError_t raise(Kernel *kernel, size_t bytes, int carveout = -1)
     {
         int dev = 0;
         cudaError_t e = cudaGetDevice(&dev);
@@ -65,6 +82,9 @@ public:
         if (known && done_[dev].load(std::memory_order_acquire)) return cudaSuccess;
         e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  static_cast<int>(bytes));
+        if (e == cudaSuccess && carveout >= 0)
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     carveout);
         if (e == cudaSuccess && known) done_[dev].store(true, std::memory_order_release);
         return e;
     }
@@ -484,16 +504,25 @@ cudaError_t launch_records(int64_t n, int n_views, const ViewDesc *views, int fl
                            const uint8_t *active, PairRec *recs, cudaStream_t st);
 
 // Binning (splat_sort.cu): from the projection's pixel rectangles to the per-tile lists in
-// (range, id) order, [start, end) per tile and the work order.  A list of more than kListCap
-// entries is cut into segments of at most kListCap before it is sorted.
+// (range, id) order, [start, end) per tile and the work order.  A list of kListCap entries or more
+// is cut into segments of at most kListCap before it is sorted, one of kHugeList or more by a
+// cluster of kSplitCluster CTAs: one list of 1 M entries 0.794 -> 0.221 ms (clusters of two 0.406,
+// of eight 0.146), sixteen of 68,000 0.065 -> 0.036 (0.042, 0.098: clusters of eight do not all fit
+// on the chip at once, which also costs frames without such lists 6 us; of four nothing).
 constexpr int kListCap = 4096;
 constexpr int kSegTarget = kListCap / 2;
+constexpr int kHugeList = 32768, kSplitCluster = 4;
+constexpr int kSplitLevels = 6;   // cuts of one list, at most (split_list)
 struct ListSegment {
     uint32_t start, len, tile;
+    uint32_t in_entries;   // its keys lie in BinArgs::entries (1) or entries2 (0)
 };
-inline int64_t max_segments(int64_t max_pairs)   // ceil(len / target) of lists above the cap
+// A cut of len entries leaves at most len / kSegTarget + 1 stretches and one more segment for each
+// bin above kSegTarget; at every level the lists and segments that are cut have kListCap entries
+// or more.
+constexpr int64_t max_segments(int64_t max_pairs)
 {
-    return max_pairs / kSegTarget + max_pairs / kListCap + 2;
+    return kSplitLevels * (2 * (max_pairs / kSegTarget) + max_pairs / kListCap + 4);
 }
 struct BinArgs {
     const ViewDesc *views;
@@ -515,7 +544,7 @@ struct BinArgs {
     uint2 *ranges;
     uint32_t *order;            // tiles by decreasing bucket of list length, four an octave
     uint64_t *entries;          // emitted (range key << 32 | pair id), then the sorted entries
-    uint64_t *entries2;         // scratch of the same size (needed when n > kListCap)
+    uint64_t *entries2;         // scratch of the same size (needed when n >= kListCap)
     uint8_t *entry_blocks;
     ListSegment *segments;      // max_segments(max_pairs)
     uint32_t *d_count;          // out: list entries
@@ -529,7 +558,6 @@ struct BinArgs {
     int block_prims, blocks;    // the projection's blocks; these and chunk (blocks a counting CTA
     int chunk;                  // takes) are set by the launchers
 };
-// kBinLong, kBinMid: tiles (in work order) with at least kListCap and at least 256 entries;
 constexpr int kBinCtas = 4;              // counting and emitting CTAs per SM
 constexpr int kMinChunk = kLargeBlock;   // primitives each takes at least
 constexpr int kMaxSharedTiles = 12288;   // views up to this are counted in shared memory (48 KB)
@@ -538,10 +566,11 @@ inline int64_t cta_count_words(int sms, int max_views, int64_t max_tiles)
     return (int64_t{kBinCtas} * sms + max_views) *
            (max_tiles < kMaxSharedTiles ? max_tiles : kMaxSharedTiles);
 }
-// kBinSplit4, kBinSplit2: RenderArgs::split
-// kBinOver: the entries exceed the capacity
+// kBinHuge, kBinLong, kBinMid: tiles (in work order) with at least kHugeList, kListCap and 256
+// entries; kBinSplit4, kBinSplit2: RenderArgs::split; kBinOver: the entries exceed the capacity
 enum {
-    kBinLong = 0, kBinMid, kBinSegments, kBinQueueSeg, kBinSplit4, kBinSplit2, kBinOver, kBinWords
+    kBinLong = 0, kBinMid, kBinSegments, kBinQueueSeg, kBinSplit4, kBinSplit2, kBinOver, kBinHuge,
+    kBinWords
 };
 cudaError_t prepare_lists();    // once per device, before its first launch_lists
 int bin_launches(int64_t n);    // kernels these three run for n primitives

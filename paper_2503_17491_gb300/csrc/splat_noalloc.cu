@@ -59,8 +59,7 @@ constexpr size_t kOffEntries2 = align256(kOffEntries + 8 * (kMaxPairs + 128));
 constexpr size_t kOffBlocks = align256(kOffEntries2 + 8 * kMaxPairs);
 constexpr size_t kOffSegments = align256(kOffBlocks + kMaxPairs + 128);
 constexpr size_t kOffRanges =
-    align256(kOffSegments + sizeof(splat::ListSegment) *
-                                (kMaxPairs / splat::kSegTarget + kMaxPairs / splat::kListCap + 2));
+    align256(kOffSegments + sizeof(splat::ListSegment) * splat::max_segments(kMaxPairs));
 constexpr size_t kOffOrder = align256(kOffRanges + 8 * size_t{kMaxTiles});
 constexpr size_t kOffTiles = align256(kOffOrder + 4 * size_t{kMaxTiles});
 constexpr size_t kOffPix = align256(kOffTiles + sizeof(TileInfo) * kMaxTiles);

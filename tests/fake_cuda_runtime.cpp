@@ -103,13 +103,14 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *fn, voi
                    c->attrs[k].val.programmaticStreamSerializationAllowed;
     return launch(fn, c->gridDim, c->blockDim, c->dynamicSmemBytes, chained);
 }
-cudaError_t cudaFuncSetAttribute(const void *fn, cudaFuncAttribute, int value)
+cudaError_t cudaFuncSetAttribute(const void *fn, cudaFuncAttribute attr, int value)
 {
     if (g_failing_attributes > 0) {
         --g_failing_attributes;
         return cudaErrorUnknown;
     }
-    g_limit[{g_device, fn}] = static_cast<size_t>(value);
+    if (attr == cudaFuncAttributeMaxDynamicSharedMemorySize)
+        g_limit[{g_device, fn}] = static_cast<size_t>(value);
     return cudaSuccess;
 }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *, int, size_t,

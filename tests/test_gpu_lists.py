@@ -163,3 +163,63 @@ def test_boxes(kind, tile):
     ctx.render(*to_dev(s))
     assert ctx.status() == 0
     assert check_lists(ctx, s, views, tile) > 0
+
+
+@pytest.mark.parametrize("n,kind", [(70_000, "spread"), (65_536, "equal"), (70_000, "wall"),
+                                    (70_001, "mixed"), (9000, "far"), (66_000, "far"),
+                                    (30_000, "nested")])
+def test_segments(n, kind):
+    """Lists cut by one CTA and by a cluster, and segments that have to be cut again: all at one
+    place (only the ids differ), a thin wall, a wall beside a spread, ranges past the last bin of
+    the first cut, and clumps inside clumps that take several cuts."""
+    rng = np.random.default_rng(n)
+    r = rng.uniform(2.0, 60.0, n)
+    if kind == "equal":
+        r[:] = 7.0
+    if kind == "wall":
+        r = 30.0 + 1e-4 * rng.uniform(0, 1, n)
+    if kind == "mixed":
+        r[::3] = 12.0 + 1e-5 * rng.uniform(0, 1, len(r[::3]))
+    if kind == "far":
+        r = np.exp(rng.uniform(math.log(2.0 ** 21), math.log(2.0 ** 24), n))
+    if kind == "nested":
+        r = 16.0 + 8.0 * 2.0 ** -rng.integers(0, 22, n)
+    s = _one_tile(n, r, 3)
+    if kind == "equal":
+        s.pos_logit[:, :3] = s.pos_logit[0, :3]
+    assert _check(s)[1] == n
+
+
+def _stage(s, name, runs=9, max_pairs=None):
+    """Median time (ms) of a stage of a forward render."""
+    ctx = make_ctx(s.n, s.views, max_pairs=max_pairs)
+    dev = to_dev(s)
+    ctx.set_profiling(True)
+    ms = []
+    for k in range(runs + 3):
+        ctx.render(*dev)
+        ms.append(ctx.stage_times()[name])
+    assert ctx.status() == 0
+    ctx.close()
+    return float(np.median(ms[3:]))
+
+
+def test_equal_ranges_cost_no_cliff():
+    """150,000 primitives of one tile within a tenth of a millimetre of range are sorted in the
+    order of time of as many spread over 60 m: they take one more cut (three more passes over the
+    keys) and the same list sort.  Merging them in one CTA took 26 times as long."""
+    rng = np.random.default_rng(1)
+    n = 150_000
+    wall = _stage(_one_tile(n, 30.0 + 1e-4 * rng.uniform(0, 1, n), 1), "tile sort")
+    spread = _stage(_one_tile(n, rng.uniform(2.0, 60.0, n), 1), "tile sort")
+    assert wall <= 5 * spread, (wall, spread)
+
+
+def test_one_long_list_takes_several_ctas():
+    """A list of 600,000 entries, cut by a cluster of CTAs, against one of 30,000 that one CTA cuts:
+    twenty times the keys on four times the CTAs is five times as long, and the sort of the segments
+    spreads over the SMs and adds less than that.  Cut by one CTA it took ten times as long."""
+    rng = np.random.default_rng(2)
+    t = {n: _stage(_one_tile(n, rng.uniform(2.0, 60.0, n), 1), "tile sort")
+         for n in (30_000, 600_000)}
+    assert t[600_000] <= 7 * t[30_000], t
