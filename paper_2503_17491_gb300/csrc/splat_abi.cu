@@ -90,7 +90,7 @@ struct splat_ctx {
     int n_views = 0;
     std::vector<ViewDesc> views;
     int64_t n_pixels = 0, n_tiles = 0;
-    int max_view_tiles = 0;
+    int bands = 0, max_view_bands = 0, max_band_tiles = 0;   // of the binning (splat::view_bands)
     ViewDesc *d_views = nullptr;
     PixFrame *d_pixframes = nullptr;   // grown by splat_set_views
     int64_t pixframe_cap = 0;
@@ -258,7 +258,10 @@ int render_core(splat_ctx *ctx, const splat_gaussians *g, float *depth, float *n
     ba.views = ctx->d_views;
     ba.n_views = ctx->n_views;
     ba.active = active;
-    ba.max_active = active ? std::min(ctx->samp_draws, ctx->n_views) : ctx->n_views;
+    ba.bands = ba.max_active_bands = ctx->bands;
+    if (active)
+        ba.max_active_bands =
+            std::min(ctx->bands, std::min(ctx->samp_draws, ctx->n_views) * ctx->max_view_bands);
     ba.n = n;
     ba.tile_h = th;
     ba.tile_w = tw;
@@ -269,7 +272,7 @@ int render_core(splat_ctx *ctx, const splat_gaussians *g, float *depth, float *n
     ba.kappa = ctx->d_kappa;
     ba.touch_count = ctx->d_touch_count;
     ba.max_pairs = ctx->cap.max_pairs;
-    ba.max_view_tiles = ctx->max_view_tiles;
+    ba.max_band_tiles = ctx->max_band_tiles;
     ba.tile_count = zero + kZeroTiles;
     ba.cta_count = ctx->d_cta_count;
     ba.ranges = ctx->d_ranges;
@@ -669,9 +672,14 @@ SPLAT_API int splat_set_views(splat_ctx *ctx, int32_t n_views, const double *T_w
     ctx->n_views = n_views;
     ctx->n_pixels = pix;
     ctx->n_tiles = tiles;
-    ctx->max_view_tiles = 0;
-    for (const ViewDesc &v : views)
-        ctx->max_view_tiles = std::max(ctx->max_view_tiles, v.tiles_r * v.tiles_c);
+    ctx->bands = ctx->max_view_bands = ctx->max_band_tiles = 0;
+    for (const ViewDesc &v : views) {
+        const int bands = splat::view_bands(v.tiles_r, v.tiles_c);
+        ctx->bands += bands;
+        ctx->max_view_bands = std::max(ctx->max_view_bands, bands);
+        ctx->max_band_tiles = std::max(
+            ctx->max_band_tiles, std::min(v.tiles_r, splat::band_rows(v.tiles_c)) * v.tiles_c);
+    }
     ctx->rendered = false;
     ctx->have_pose = false;
     ctx->samp_draws = 0;   // the sampling law depends on the views: set it again

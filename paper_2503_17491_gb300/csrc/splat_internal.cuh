@@ -527,8 +527,7 @@ constexpr int64_t max_segments(int64_t max_pairs)
 struct BinArgs {
     const ViewDesc *views;
     int n_views;
-    const uint8_t *active;      // nullable: views drawn for this step, at most max_active
-    int max_active;
+    const uint8_t *active;      // nullable: views drawn for this step
     int64_t n;                  // primitives per view
     int tile_h, tile_w;
     int64_t n_tiles;
@@ -538,7 +537,8 @@ struct BinArgs {
     const float *kappa;
     const uint32_t *touch_count;
     int64_t max_pairs;
-    int max_view_tiles;         // most tiles of one view
+    int bands, max_active_bands;   // of all views; of the views drawn, at most
+    int max_band_tiles;         // most tiles of one band
     uint32_t *tile_count;       // zeroed before; counted, then counted down by the emission
     uint32_t *cta_count;        // cta_count_words(...): the counts of every counting CTA
     uint2 *ranges;
@@ -560,10 +560,18 @@ struct BinArgs {
 };
 constexpr int kBinCtas = 4;              // counting and emitting CTAs per SM
 constexpr int kMinChunk = kLargeBlock;   // primitives each takes at least
-constexpr int kMaxSharedTiles = 12288;   // views up to this are counted in shared memory (48 KB)
+// A view's tiles are counted and emitted band by band, each a run of whole tile rows of at most
+// kMaxSharedTiles tiles (the counters of one CTA, 48 KB).  Views have up to 4,096 tile columns, so
+// that every band but a view's last has more than 8,192 tiles.
+constexpr int kMaxSharedTiles = 12288;
+__host__ __device__ inline int band_rows(int tiles_c) { return kMaxSharedTiles / tiles_c; }
+__host__ __device__ inline int view_bands(int tiles_r, int tiles_c)
+{
+    return (tiles_r + band_rows(tiles_c) - 1) / band_rows(tiles_c);
+}
 inline int64_t cta_count_words(int sms, int max_views, int64_t max_tiles)
 {
-    return (int64_t{kBinCtas} * sms + max_views) *
+    return (int64_t{kBinCtas} * sms + max_views + max_tiles / 8192) *
            (max_tiles < kMaxSharedTiles ? max_tiles : kMaxSharedTiles);
 }
 // kBinHuge, kBinLong, kBinMid: tiles (in work order) with at least kHugeList, kListCap and 256

@@ -53,7 +53,7 @@ constexpr size_t kOffCtaCount = align256(kOffTileCount + 4 * size_t{kMaxTiles});
 // one view: a counting CTA takes at least kMinChunk primitives
 constexpr size_t kCountCtas = kMaxGaussians / splat::kMinChunk + 1;
 static_assert(kMaxGaussians < 1 << 18, "blocks of kSmallBlock primitives");
-static_assert(kMaxTiles <= splat::kMaxSharedTiles, "counted in shared memory");
+static_assert(kMaxTiles <= splat::kMaxSharedTiles, "one band");
 constexpr size_t kOffEntries = align256(kOffCtaCount + 4 * kCountCtas * kMaxTiles);
 constexpr size_t kOffEntries2 = align256(kOffEntries + 8 * (kMaxPairs + 128));
 constexpr size_t kOffBlocks = align256(kOffEntries2 + 8 * kMaxPairs);
@@ -289,7 +289,7 @@ extern "C" SPLAT_API int splat_render_noalloc(const splat_gaussians *g,
     NA_CK(splat::launch_project(pa, st));
     splat::BinArgs ba{};
     ba.views = view;
-    ba.n_views = ba.max_active = 1;
+    ba.n_views = 1;
     ba.n = n;
     ba.tile_h = th;
     ba.tile_w = tw;
@@ -300,7 +300,8 @@ extern "C" SPLAT_API int splat_render_noalloc(const splat_gaussians *g,
     ba.kappa = pa.kappa;
     ba.touch_count = pa.touch_count;
     ba.max_pairs = kMaxPairs;
-    ba.max_view_tiles = static_cast<int>(n_tiles);
+    ba.bands = ba.max_active_bands = 1;
+    ba.max_band_tiles = static_cast<int>(n_tiles);
     ba.tile_count = tile_count;
     ba.cta_count = reinterpret_cast<uint32_t *>(base + kOffCtaCount);
     ba.ranges = ranges;

@@ -1,8 +1,8 @@
 // K2-K4: tile binning, from the projection's pixel rectangles to the per-tile lists in
 // (range, primitive id) order (Sec. 3.2.1).
 //
-//   count    list lengths: a CTA counts the tiles of a chunk of one view's touching pairs in
-//            shared memory and adds its counts to the global ones;
+//   count    list lengths: a CTA counts the tiles of a band of one view over a chunk of its
+//            touching pairs in shared memory and adds its counts to the global ones;
 //   layout   one CTA: [start, end) of every tile's list by an exclusive scan of the counts, the
 //            work order (longest lists first) and the total;
 //   emission (range key << 32 | pair id) into each touched tile's slice: a CTA reserves as many
@@ -208,33 +208,52 @@ __global__ void __launch_bounds__(kLayoutThreads) k_layout(
 }
 
 // ---------------------------------------------------------------------------------------------
-// count and emission: a CTA takes a chunk of one view's touching pairs
+// count and emission: a CTA takes a chunk of one view's touching pairs and a band of its tiles
 // ---------------------------------------------------------------------------------------------
 constexpr int kChunkThreads = 512;
 
 struct Chunk {
+    int view;
     const uint2 *touch;
     const float *kappa;
     const uint32_t *touch_count;
     int begin, end;        // units of 32 places: unit u is places 32 u .. of the view
     int unit_shift;        // log2 of the units a block
-    int tiles_c, n_tiles;
+    int tiles_c;
+    int row0, rows;        // the band's tile rows
+    int n_tiles;           // and tiles, which the three arrays below begin with
     uint32_t *tile_count;
-    uint32_t *cta_count;   // this CTA's count of every tile of the view
+    uint32_t *cta_count;   // this CTA's count of every tile of the band
     const uint2 *ranges;
 };
 
-__device__ __forceinline__ Chunk chunk_of(const BinArgs &A, int v)
+// The chunk of this CTA; false when its view is not drawn.  kBanded: at least one view has more
+// than one band.
+template <bool kBanded>
+__device__ __forceinline__ bool chunk_of(const BinArgs &A, Chunk &c)
 {
+    int v = 0, band = 0, row = 0;   // row: rank of the band among those of the drawn views
+    if (kBanded) {
+        band = blockIdx.y;
+        for (;; ++v) {
+            const int nb = view_bands(A.views[v].tiles_r, A.views[v].tiles_c);
+            if (band < nb) break;
+            band -= nb;
+            if (!A.active || A.active[v]) row += nb;
+        }
+        row += band;
+    } else {
+        v = row = blockIdx.y;
+        if (A.active) {
+            row = 0;
+            for (int k = 0; k < v; ++k) row += A.active[k] ? 1 : 0;
+        }
+    }
+    if (A.active && !A.active[v]) return false;
     const ViewDesc &vd = A.views[v];
     const int64_t p0 = static_cast<int64_t>(v) * A.n;
-    int row = v;   // the view's rank among the drawn ones
-    if (A.active) {
-        row = 0;
-        for (int k = 0; k < v; ++k) row += A.active[k] ? 1 : 0;
-    }
     const int first = A.chunk * static_cast<int>(blockIdx.x);
-    Chunk c;
+    c.view = v;
     c.touch = A.touch + p0;
     c.kappa = A.kappa + p0;
     c.touch_count = A.touch_count + static_cast<int64_t>(v) * A.blocks;
@@ -242,23 +261,26 @@ __device__ __forceinline__ Chunk chunk_of(const BinArgs &A, int v)
     c.begin = first << c.unit_shift;
     c.end = min(first + A.chunk, A.blocks) << c.unit_shift;
     c.tiles_c = vd.tiles_c;
-    c.n_tiles = vd.tiles_r * vd.tiles_c;
-    c.tile_count = A.tile_count + vd.tile_offset;
+    c.row0 = kBanded ? band * band_rows(vd.tiles_c) : 0;
+    c.rows = kBanded ? min(vd.tiles_r - c.row0, band_rows(vd.tiles_c)) : vd.tiles_r;
+    c.n_tiles = c.rows * vd.tiles_c;
+    const int64_t t0 = vd.tile_offset + static_cast<int64_t>(c.row0) * vd.tiles_c;
+    c.tile_count = A.tile_count + t0;
     c.cta_count = A.cta_count +
-                  (static_cast<int64_t>(row) * gridDim.x + blockIdx.x) * A.max_view_tiles;
-    c.ranges = A.ranges + vd.tile_offset;
-    return c;
+                  (static_cast<int64_t>(row) * gridDim.x + blockIdx.x) * A.max_band_tiles;
+    c.ranges = A.ranges + t0;
+    return true;
 }
 
-// f(tile of the view, range key bits, primitive in the view) for every tile of every touching pair
-// of the chunk, 32 pairs a warp at a time, kUnitLoads of them read ahead (the range keys only with
+// f(tile of the band, range key bits, primitive in the view) for every tile of the band of every
+// touching pair of the chunk, 32 pairs a warp at a time, kUnitLoads of them read ahead (the range keys only with
 // kKeys).  While no
 // pair of a warp touches more than kLaneTiles tiles, every lane walks its own; otherwise the warp
 // numbers the tiles of its 32 pairs by a prefix sum and gives one to every lane, so that one wide
 // pair costs its warp no more than as many narrow ones.
 constexpr int kLaneTiles = 8, kUnitLoads = 4;
 
-template <bool kKeys, typename F>
+template <bool kBanded, bool kKeys, typename F>
 __device__ __forceinline__ void for_each_entry(const Chunk &c, F f)
 {
     const int lane = threadIdx.x & 31;
@@ -292,6 +314,11 @@ __device__ __forceinline__ void for_each_entry(const Chunk &c, F f)
             uint32_t local = 0, cnt = 0;
             if (static_cast<uint32_t>(lane) < live[i]) {
                 t = unpack_touch(word[i], local);
+                if (kBanded) {   // the part inside the band
+                    const int r0 = max(t.r0 - c.row0, 0);
+                    t.nr = max(min(t.r0 - c.row0 + t.nr, c.rows) - r0, 0);
+                    t.r0 = r0;
+                }
                 cnt = static_cast<uint32_t>(t.nr) * static_cast<uint32_t>(t.nc);
             }
             if (!__any_sync(kFull, cnt > kLaneTiles)) {
@@ -338,61 +365,55 @@ __device__ __forceinline__ void for_each_entry(const Chunk &c, F f)
     }
 }
 
-// With shared counters a tile's count sees one global atomic per CTA instead of one per entry:
+// Counted in shared memory, a tile sees one global atomic per CTA instead of one per entry:
 // neighbouring threads' pairs fall on a few hundred tiles of one view, and same-address atomics
-// in L2 serialise (emission of 5.3 M entries: 0.95 ms with an atomic per entry).
-template <bool kShared>
+// in L2 serialise (emission of 5.3 M entries: 0.95 ms with an atomic per entry).  A view of more
+// tiles than the counters hold is taken in bands, each by its own CTAs, which pass over the pairs
+// that miss their band: eleven 64 x 1024 views and one of 128 x 32,000 over 500 k primitives (11.6 M
+// entries), counted and emitted with global atomics 0.63 ms, in bands 0.29; the wide view alone
+// (16,000 tiles, 6.2 M entries) 0.13 either way.
+template <bool kBanded>
 __global__ void __launch_bounds__(kChunkThreads) k_count(const BinArgs A)
 {
     chain_wait();
     extern __shared__ uint32_t s_cnt[];
-    const int v = blockIdx.y;
-    if (A.active && !A.active[v]) return;
-    const Chunk c = chunk_of(A, v);
-    if (kShared) {
-        for (int t = threadIdx.x; t < c.n_tiles; t += kChunkThreads) s_cnt[t] = 0u;
-        __syncthreads();
-    }
-    uint32_t *cnt = kShared ? s_cnt : c.tile_count;
-    for_each_entry<false>(c, [&](uint32_t t, uint32_t, uint32_t) { atomicAdd(cnt + t, 1u); });
-    if (kShared) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < c.n_tiles; t += kChunkThreads) {
-            const uint32_t n = s_cnt[t];
-            if (n) atomicAdd(c.tile_count + t, n);
-            c.cta_count[t] = n;
-        }
+    Chunk c;
+    if (!chunk_of<kBanded>(A, c)) return;
+    for (int t = threadIdx.x; t < c.n_tiles; t += kChunkThreads) s_cnt[t] = 0u;
+    __syncthreads();
+    for_each_entry<kBanded, false>(
+        c, [&](uint32_t t, uint32_t, uint32_t) { atomicAdd(s_cnt + t, 1u); });
+    __syncthreads();
+    for (int t = threadIdx.x; t < c.n_tiles; t += kChunkThreads) {
+        const uint32_t n = s_cnt[t];
+        if (n) atomicAdd(c.tile_count + t, n);
+        c.cta_count[t] = n;
     }
 }
 
-template <bool kShared>
+template <bool kBanded>
 __global__ void __launch_bounds__(kChunkThreads) k_emit(const BinArgs A)
 {
     chain_wait();
     extern __shared__ uint32_t s_cnt[];
-    const int v = blockIdx.y;
-    if (A.active && !A.active[v]) return;
-    const Chunk c = chunk_of(A, v);
+    Chunk c;
+    if (!chunk_of<kBanded>(A, c)) return;
     // (a frame past its capacity checks every place against its list's end)
     const bool over = A.bin[kBinOver] != 0u;
-    if (kShared) {
-        for (int t = threadIdx.x; t < c.n_tiles; t += kChunkThreads) {
-            const uint32_t n = c.cta_count[t];   // the tile's count counts down: this CTA takes n
-            if (n)
-                s_cnt[t] = atomicSub(c.tile_count + t, n) - n + (over ? 0u : c.ranges[t].x);
-        }
-        __syncthreads();
+    for (int t = threadIdx.x; t < c.n_tiles; t += kChunkThreads) {
+        const uint32_t n = c.cta_count[t];   // the tile's count counts down: this CTA takes n
+        if (n) s_cnt[t] = atomicSub(c.tile_count + t, n) - n + (over ? 0u : c.ranges[t].x);
     }
-    const uint32_t p0 = static_cast<uint32_t>(static_cast<int64_t>(v) * A.n);
-    if (kShared && !over) {
-        for_each_entry<true>(c, [&](uint32_t t, uint32_t key, uint32_t i) {
+    __syncthreads();
+    const uint32_t p0 = static_cast<uint32_t>(static_cast<int64_t>(c.view) * A.n);
+    if (!over) {
+        for_each_entry<kBanded, true>(c, [&](uint32_t t, uint32_t key, uint32_t i) {
             A.entries[atomicAdd(s_cnt + t, 1u)] = static_cast<uint64_t>(key) << 32 | (p0 + i);
         });
         return;
     }
-    for_each_entry<true>(c, [&](uint32_t t, uint32_t key, uint32_t i) {
-        const uint32_t k =
-            kShared ? atomicAdd(s_cnt + t, 1u) : atomicSub(c.tile_count + t, 1u) - 1u;
+    for_each_entry<kBanded, true>(c, [&](uint32_t t, uint32_t key, uint32_t i) {
+        const uint32_t k = atomicAdd(s_cnt + t, 1u);
         const uint2 rg = c.ranges[t];
         if (k < rg.y - rg.x) A.entries[rg.x + k] = static_cast<uint64_t>(key) << 32 | (p0 + i);
     });
@@ -984,17 +1005,17 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) k_lists(const BinArgs
     }
 }
 
-// blocks a CTA counts or emits: at most kBinCtas CTAs per SM over the drawn views, at least
+// blocks a CTA counts or emits: at most kBinCtas CTAs per SM over the drawn views' bands, at least
 // kMinChunk primitives (below that the CTA's counters cost more than its pairs)
 dim3 chunk_grid(BinArgs &a)
 {
     a.block_prims = block_prims(a.n);
     a.blocks = static_cast<int>(project_blocks(a.n));
-    const int64_t c = int64_t{a.blocks} * a.max_active / (int64_t{kBinCtas} * a.sms) + 1;
+    const int64_t c = int64_t{a.blocks} * a.max_active_bands / (int64_t{kBinCtas} * a.sms) + 1;
     const int64_t least = kMinChunk / a.block_prims;
     a.chunk = static_cast<int>(c < least ? least : c);
     return dim3(static_cast<unsigned>((a.blocks + a.chunk - 1) / a.chunk),
-                static_cast<unsigned>(a.n_views));
+                static_cast<unsigned>(a.bands));
 }
 
 bool chained(const BinArgs &a) { return chained_size(a.n * a.n_views); }
@@ -1020,15 +1041,14 @@ cudaError_t launch_bin_counts(const BinArgs &args, cudaStream_t st)
     BinArgs a = args;
     if (a.n > 0) {
         const dim3 grid = chunk_grid(a);
-        const bool shared = a.max_view_tiles <= kMaxSharedTiles;
-        const cudaError_t e = launch_chained(chained(a), shared ? k_count<true> : k_count<false>, grid,
-                                             kChunkThreads, shared ? 4 * a.max_view_tiles : 0, st,
-                                             a);
+        const cudaError_t e =
+            launch_chained(chained(a), a.bands > a.n_views ? k_count<true> : k_count<false>, grid,
+                           kChunkThreads, 4 * a.max_band_tiles, st, a);
         if (e != cudaSuccess) return e;
     }
-    return launch_chained(chained(a), k_layout, dim3(1), kLayoutThreads, 0, st, a.tile_count, a.n_tiles,
-                          a.max_pairs, a.ranges, a.order, a.d_count, a.status, a.bin, a.warps,
-                          a.rec_cap, a.n_rows, a.refine);
+    return launch_chained(chained(a), k_layout, dim3(1), kLayoutThreads, 0, st, a.tile_count,
+                          a.n_tiles, a.max_pairs, a.ranges, a.order, a.d_count, a.status, a.bin,
+                          a.warps, a.rec_cap, a.n_rows, a.refine);
 }
 
 cudaError_t launch_emit(const BinArgs &args, cudaStream_t st)
@@ -1036,9 +1056,8 @@ cudaError_t launch_emit(const BinArgs &args, cudaStream_t st)
     BinArgs a = args;
     if (a.n <= 0) return cudaSuccess;
     const dim3 grid = chunk_grid(a);
-    const bool shared = a.max_view_tiles <= kMaxSharedTiles;
-    return launch_chained(chained(a), shared ? k_emit<true> : k_emit<false>, grid, kChunkThreads,
-                          shared ? 4 * a.max_view_tiles : 0, st, a);
+    return launch_chained(chained(a), a.bands > a.n_views ? k_emit<true> : k_emit<false>, grid,
+                          kChunkThreads, 4 * a.max_band_tiles, st, a);
 }
 
 cudaError_t launch_lists(const BinArgs &a, cudaStream_t st)

@@ -10,7 +10,7 @@ import torch
 
 import oracle
 from paper_2503_17491_gb300 import api, scenes
-from gpu_common import check_lists, make_ctx, to_dev
+from gpu_common import check_lists, make_ctx, oracle_lists, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -223,3 +223,75 @@ def test_one_long_list_takes_several_ctas():
     t = {n: _stage(_one_tile(n, rng.uniform(2.0, 60.0, n), 1), "tile sort")
          for n in (30_000, 600_000)}
     assert t[600_000] <= 7 * t[30_000], t
+
+
+def _wide_view(cols=32_000, rows=112):
+    return scenes.View(np.eye(4), rows, cols, scenes.deg(-20), scenes.deg(20))
+
+
+@pytest.mark.parametrize("tile", [(16, 16), (4, 64)])
+@pytest.mark.parametrize("draws", [0, 2])
+def test_bands(tile, draws):
+    """Views counted in one band, in two and in several (the last band a single tile row), drawn or
+    not: the lists of the drawn views against the oracle's."""
+    s = scenes.tiny_scene(2500, 6, rows=16, cols=64, dist=(0.6, 9.0), log_scale=(-5.0, -1.0))
+    views = [_wide_view(700, 45), _wide_view(), s.views[0], _wide_view(32_767, 225)]
+    ctx = make_ctx(s.n, views, tile, max_pairs=1 << 22)
+    if not draws:
+        ctx.render(*to_dev(s))
+        assert ctx.status() == 0
+        check_lists(ctx, s, views, tile)
+        return
+    ctx.set_view_sampling(draws, 0.3, 5)
+    seen = set()
+    for _ in range(6):
+        ctx.render(*to_dev(s))
+        assert ctx.status() == 0
+        on = ctx.active_views()
+        seen.add(tuple(on))
+        okeys, oids, _, _ = oracle_lists(s, views, tile)
+        starts = np.cumsum([0] + [-(-v.rows // tile[0]) * -(-v.cols // tile[1]) for v in views])
+        view = np.searchsorted(starts, (okeys >> np.uint64(32)).astype(np.int64), side="right") - 1
+        gk, gv, _ = ctx.sorted_lists()
+        np.testing.assert_array_equal(gk, (okeys >> np.uint64(32)).astype(np.uint32)[on[view]])
+        np.testing.assert_array_equal(gv % s.n, oids[on[view]])
+    assert len(seen) > 1
+
+
+@pytest.mark.parametrize("wide", [False, True])
+def test_lists_past_the_capacity(wide):
+    """Lists keep the places below the capacity, each filled by a pair that belongs there, in
+    order; the status says that pairs are missing."""
+    s = scenes.tiny_scene(3000, 5, rows=112, cols=700, dist=(0.6, 9.0), log_scale=(-5.0, -1.0))
+    views = [_wide_view() if wide else s.views[0]]
+    ctx = make_ctx(s.n, views, max_pairs=1 << 21)
+    ctx.render(*to_dev(s))
+    assert ctx.status() == 0
+    _, ids, ranges = ctx.sorted_lists()
+    kappa = ctx.pair_records(s.n)["kappa"]
+    cap = 2 * len(ids) // 3
+    low = make_ctx(s.n, views, max_pairs=cap)
+    low.render(*to_dev(s))
+    assert low.status() == 1   # SPLAT_STATUS_CAPACITY
+    _, got, cut = low.sorted_lists()
+    assert len(got) == cap
+    full = ranges[:, 1] > ranges[:, 0]
+    np.testing.assert_array_equal(cut, np.where(full[:, None], np.minimum(ranges, cap), 0))
+    for (a, b), (c, d) in zip(ranges[full].astype(np.int64), cut[full].astype(np.int64)):
+        assert set(got[c:d]) <= set(ids[a:b]) and len(set(got[c:d])) == d - c
+        key = list(zip(kappa[got[c:d]], got[c:d]))
+        assert key == sorted(key)
+
+
+def test_a_wide_view_costs_the_others_nothing():
+    """Eleven views and one of more tiles than a CTA's counters hold are counted and emitted in one
+    call in about the time of two calls (half as much again is allowed for the spread of times this
+    short).  With a global atomic for every entry of every view it was 2.4 times."""
+    s = scenes.workload(1, n=200_000)
+    narrow = [scenes.View(s.views[0].T_ws, 64, 1024, scenes.deg(-22.5), scenes.deg(22.5))] * 11
+    wide = [scenes.View(s.views[0].T_ws, 128, 32_000, scenes.deg(-22.5), scenes.deg(22.5))]
+    ms = []
+    for views in (narrow, wide, narrow + wide):
+        s.views = views
+        ms.append(_stage(s, "emission", max_pairs=1 << 24))
+    assert ms[2] <= 1.5 * (ms[0] + ms[1]), ms
