@@ -106,10 +106,18 @@ __device__ __forceinline__ T block_excl_scan(T v, T *s_warp, T *total)
 //   128x2048, 1 M, urban block, 2.1 shares              .249 .225 |           | .274 .250
 //   12 keyframes, 500 k, 1.8 shares                     .729 .816 |           | .768 .842
 // Where even the longest list is below kSplitFrom shares the queue evens the warps out by itself
-// and splitting only costs, so such a frame is left whole: the whole pass at 2.44 and 2.51 shares
-// (128x2048, 1 M, forward and backward) 0.66 whole, 0.69 split; at 2.76 and 2.78 (eight 128x1024,
-// forward) 0.76 whole, 0.69 split.  The longest list is taken exactly: rounded up to a bucket the
-// line lay anywhere up to 3.1 shares.
+// and splitting mostly costs, so such a frame is left whole.  The line is taken over random frames
+// (rooms, streets, blocks and a city, 1 to 12 views of 32 x 512 to 128 x 2048, 5,000 to 2 M
+// primitives, all tile shapes, longest lists of 1 to 12 shares), forward and backward.  Splitting
+// against whole blocks, geometric mean of 600 frames by the shares of their longest list: 0.93 at 1
+// to 1.5, 0.97 up to 2, 1.02 up to 2.5, 1.11 up to 3, 1.17 up to 4, 1.33 up to 6, 1.63 above.  Single
+// frames scatter widely about that, so the mean hardly depends on the line (660 frames, against
+// the better of both in each: 1.024 splitting all, 1.016 with the line at 2.0, 1.020 at 2.4, 1.024
+// at 2.65, 1.031 at 3.0, 1.228 splitting none), but the frames that splitting makes slower do: of
+// 600, 149 by more than 3 % without a line, 72 with the line at 2.0, 48 at 2.4, 28 at 2.65, the
+// worst by 30, 27, 25 and 16 %.  Each part also adds its own rounded gradient sums.  Hence the
+// highest line that costs less than 1 % of the mean.  The longest list is taken exactly: rounded
+// up to a bucket the line lay anywhere up to 3.1 shares.
 // A split block keeps one contributor record per part and primitive, so nothing is split when the
 // record pool might not hold one record for every row of 8 pixels that every pair meets (n_rows
 // counts those): the pool then overflows for no frame that it held unsplit.
