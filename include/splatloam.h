@@ -423,7 +423,8 @@ SPLAT_API int splat_stage_times(splat_ctx *ctx, float *ms);
  * list (uint32, n_pairs; pair id = view * n + primitive); 2: per-tile [start, end) (uint32 x 2 x
  * n_tiles); 3: per-(view, primitive) records (16 bytes each: int16 row0, row1, col0, ncols;
  * float32 kappa; uint32 bits 0-29 tile count, bit 30 normal flipped, bit 31 invalid input);
- * 4: per-pixel final transmittance (float32, P); 5: per-pixel contributor bound (int32, P).
+ * 4: per-pixel final transmittance (float32, P); 5: per-pixel contributor bound (int32, P);
+ * 6: how many tiles' 4 x 8 pixel blocks were composited by four and by two warps (uint32 x 2).
  * bytes is the size of dst; returns the number of bytes copied, or -1 on error. */
 SPLAT_API int64_t splat_debug_copy(splat_ctx *ctx, int32_t which, void *dst, int64_t bytes);
 

@@ -1121,7 +1121,7 @@ SPLAT_API int splat_stage_times(splat_ctx *ctx, float *ms)
 
 SPLAT_API int64_t splat_debug_copy(splat_ctx *ctx, int32_t which, void *dst, int64_t bytes)
 {
-    if (!ctx || !dst || bytes < 0 || which < 0 || which > 5) return -1;
+    if (!ctx || !dst || bytes < 0 || which < 0 || which > 6) return -1;
     if (cudaDeviceSynchronize() != cudaSuccess) return -1;
     if (!ctx->rendered) return -1;
     uint32_t m = 0;
@@ -1172,7 +1172,9 @@ SPLAT_API int64_t splat_debug_copy(splat_ctx *ctx, int32_t which, void *dst, int
             return e == cudaSuccess ? need : -1;
         }
         case 4: return get(ctx->d_tfinal, int64_t{4} * ctx->n_pixels);
-        default: return get(ctx->d_nlast, int64_t{4} * ctx->n_pixels);
+        case 5: return get(ctx->d_nlast, int64_t{4} * ctx->n_pixels);
+        default:   // kBinSplit4 and kBinSplit2 lie side by side
+            return get(ctx->d_counters + kCountersBin + splat::kBinSplit4, int64_t{4} * 2);
         }
     } catch (...) {
         return -1;

@@ -105,6 +105,55 @@ def test_split_blocks(tile):
         assert (x - y).abs().max() <= 1e-5 * y.abs().max()
 
 
+def _split_tiles(ctx):
+    """Tiles whose blocks went to four and to two warps in the last render."""
+    return ctx.debug_copy(6, 2, np.uint32).tolist()
+
+
+@pytest.mark.parametrize("tile", [(16, 16), (8, 32), (32, 8), (4, 64)])
+def test_split_levels(tile):
+    """What decides on splitting, on both sides of each line.  The longest lists of two scans of a
+    street are long against a warp's even share of the frame: their blocks go to four warps,
+    others' to two, the shortest stay whole; images as with whole blocks (a record pool too small
+    for the split), gradients equal up to the order of float additions (as in test_split_blocks).
+    Over twelve such scans the same lists are below 2.65 shares, and nothing is split."""
+    s = scenes.workload(1, n=60_000)
+    v = s.views[0]
+    dev = to_dev(s)
+    warps = 3 * 8 * torch.cuda.get_device_properties(0).multi_processor_count
+
+    def shares(ctx):   # entries of a block's list against an even share, longest first
+        r = ctx.sorted_lists()[2].astype(np.int64)
+        share = 8.0 * ctx.stats()["n_pairs"] / warps
+        assert 0.4 * share > 64   # (shorter lists are never split)
+        return np.sort(r[:, 1] - r[:, 0])[::-1] / share
+
+    ctx = make_ctx(s.n, [v, v], tile)
+    a = ctx.render(*dev)
+    st = ctx.stats()
+    sh = shares(ctx)
+    n4, n2 = _split_tiles(ctx)
+    assert sh[0] > 2.65 * 1.05 and n4 > 0 and n2 > 0 and n4 + n2 < len(sh)
+    # lists go to four warps from 0.8 shares and to two from 0.4, both rounded up to a bucket of
+    # list lengths, of which there are four an octave
+    assert np.all(sh[:n4] >= 0.8) and np.all(sh[n4:n4 + n2] >= 0.4)
+    assert np.all(sh[n4:] < 0.8 * 1.25) and np.all(sh[n4 + n2:] < 0.4 * 1.25)
+    whole = api.SplatContext(s.n, 2, 2 * v.n_pixels, st["n_pairs"] + 8,
+                             api.RenderConfig(tile_h=tile[0], tile_w=tile[1]),
+                             max_tiles=st["n_tiles"])
+    whole.set_views([v, v])
+    b = whole.render(*dev)
+    assert _split_tiles(whole) == [0, 0]
+    assert all(torch.equal(x, y) for x, y in zip(a, b))
+    up = [torch.ones_like(t) for t in a]
+    for x, y in zip(ctx.backward(*dev, *up), whole.backward(*dev, *up)):
+        assert (x - y).abs().max() <= 1e-5 * y.abs().max()
+    many = make_ctx(s.n, [v] * 12, tile, max_pairs=16 * st["n_pairs"])
+    many.render(*dev)
+    assert shares(many)[0] < 2.65 * 0.95 and _split_tiles(many) == [0, 0]
+    assert ctx.status() == 0 and whole.status() == 0 and many.status() == 0
+
+
 def test_many_tiles():
     """A view of more tiles than the shared-memory counters hold (14,000), beside one of few: both
     in one call."""
