@@ -100,7 +100,13 @@ typedef struct {
 } splat_render_config;
 
 /* Workspace limits fixed at creation.  max_pairs bounds the number of (tile, primitive) pairs
- * of one render call summed over views; max_tiles = 0 derives a bound from max_pixels. */
+ * of one render call summed over views; max_tiles = 0 derives a bound from max_pixels.
+ * max_pairs also sizes the contributor records that the forward leaves for the backward, 2
+ * max_pairs + 256 max_tiles of them.  Where a few lists are long against the frame, their pixel
+ * blocks are split over several warps, which takes up to one record for every row of 8 pixels that
+ * each pair's bounding box meets, and 768 more for every split tile; a render that might not find
+ * them leaves its blocks whole: same images, but up to twice the time on small frames.  A
+ * max_pairs of 32 times the list entries always suffices for the boxes. */
 typedef struct {
     int64_t max_gaussians;
     int32_t max_views;
@@ -199,8 +205,8 @@ SPLAT_API int64_t splat_view_pixel_offset(const splat_ctx *ctx, int32_t v);
  * buffers depth[P], normal[3][P], alpha[P] (device, caller-owned).  The per-tile lists,
  * transmittances and contributor counts are kept in the context for the next backward call.
  * Stages: per-primitive projection and spherical bounding box (one pass over all views), tile
- * binning, sort of every tile's list by range, per-tile front-to-back compositing (one persistent launch
- * over the tiles of all views).  Errors: INVALID_ARG, STATE (no views), CUDA. */
+ * binning, sort of every tile's list by range, per-tile front-to-back compositing (one persistent
+ * launch over the tiles of all views).  Errors: INVALID_ARG, STATE (no views), CUDA. */
 SPLAT_API int splat_render_views(splat_ctx *ctx, const splat_gaussians *g, float *depth,
                                  float *normal, float *alpha, void *stream);
 

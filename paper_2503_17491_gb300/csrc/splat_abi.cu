@@ -84,7 +84,6 @@ struct splat_ctx {
     int device = 0;
     int sms = 0;
     int grid_fwd = 0, grid_bwd = 0;
-    int64_t max_pairs_views = 0;   // max_gaussians * max_views
 
     // registered views
     int n_views = 0;
@@ -129,10 +128,10 @@ struct splat_ctx {
 
     // profiling events: [0,1] forward compositing, [2,3] backward compositing, then one event
     // after the stages of the last profiled render / refinement step: [0] before the
-    // projection, [1] after it, [3] after layout and emission, [4] after the list sort, [6] after
-    // the loss, [7] after the fused Adam
+    // projection, [1] after it, [2] after layout and emission, [3] after the list sort, [4] after
+    // the loss, [5] after the fused Adam
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
-    static constexpr int kStageEvents = 8;
+    static constexpr int kStageEvents = 6;
     cudaEvent_t stage_ev[kStageEvents] = {};
     bool stage_rec[kStageEvents] = {};
     bool profiling = false;
@@ -291,9 +290,9 @@ int render_core(splat_ctx *ctx, const splat_gaussians *g, float *depth, float *n
     if (refine) ba.refine = *refine;
     CK(splat::launch_bin_counts(ba, st));
     CK(splat::launch_emit(ba, st));
-    CK(stage_mark(3));
+    CK(stage_mark(2));
     CK(splat::launch_lists(ba, st));
-    CK(stage_mark(4));
+    CK(stage_mark(3));
     splat::RenderArgs a = render_args(ctx, g);
     a.depth = depth;
     a.normal = normal;
@@ -358,9 +357,8 @@ int backward_core(splat_ctx *ctx, const splat_gaussians *g, const float *gD, con
 
 void free_ctx(splat_ctx *c)
 {
-    void *ptrs[] = {c->d_views, c->d_prect, c->d_touch, c->d_kappa,
-                    c->d_touch_count,
-                    c->d_zero, c->d_cta_count, c->d_entries, c->d_entries2, c->d_blocks, c->d_segments,
+    void *ptrs[] = {c->d_views, c->d_prect, c->d_touch, c->d_kappa, c->d_touch_count, c->d_zero,
+                    c->d_cta_count, c->d_entries, c->d_entries2, c->d_blocks, c->d_segments,
                     c->d_ranges, c->d_tfinal, c->d_nlast, c->d_wgrad, c->d_prim,
                     c->d_pose, c->d_rec, c->d_rec_prev, c->d_rec_head, c->d_rec_fill,
                     c->d_samp_thr, c->d_active, c->d_grow_sums,
@@ -434,7 +432,6 @@ SPLAT_API int splat_ctx_create(const splat_render_config *cfg, const splat_capac
     if (c->cap.max_tiles == 0)
         c->cap.max_tiles = 2 * (cap->max_pixels / (cfg->tile_h * cfg->tile_w)) +
                            int64_t{256} * cap->max_views;
-    c->max_pairs_views = mpv;
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess)
         e = cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
@@ -447,7 +444,8 @@ SPLAT_API int splat_ctx_create(const splat_render_config *cfg, const splat_capac
     if (e == cudaSuccess) e = dalloc(&c->d_kappa, mpv);
     if (e == cudaSuccess)
         e = dalloc(&c->d_touch_count,
-                   static_cast<size_t>(splat::max_project_blocks(cap->max_gaussians)) * cap->max_views);
+                   static_cast<size_t>(splat::max_project_blocks(cap->max_gaussians)) *
+                       cap->max_views);
     if (e == cudaSuccess) e = dalloc(&c->d_zero, kZeroTiles + static_cast<size_t>(TT));
     if (e == cudaSuccess)
         e = dalloc(&c->d_cta_count, splat::cta_count_words(c->sms, cap->max_views, TT));
@@ -464,7 +462,8 @@ SPLAT_API int splat_ctx_create(const splat_render_config *cfg, const splat_capac
     if (e == cudaSuccess) e = dalloc(&c->d_tfinal, P);
     if (e == cudaSuccess) e = dalloc(&c->d_nlast, P);
     if (e == cudaSuccess) e = dalloc(&c->d_wgrad, static_cast<size_t>(cap->max_gaussians) * 4);
-    if (e == cudaSuccess) e = dalloc(&c->d_prim, static_cast<size_t>(cap->max_gaussians) * splat::kPrimRow);
+    if (e == cudaSuccess)
+        e = dalloc(&c->d_prim, static_cast<size_t>(cap->max_gaussians) * splat::kPrimRow);
     if (e == cudaSuccess) e = dalloc(&c->d_pose, static_cast<size_t>(cap->max_views) * 6);
     if (e == cudaSuccess) e = dalloc(&c->d_samp_thr, static_cast<size_t>(splat::kMaxViews));
     if (e == cudaSuccess) e = dalloc(&c->d_active, static_cast<size_t>(cap->max_views));
@@ -855,8 +854,8 @@ SPLAT_API int splat_view_loss(splat_ctx *ctx, const float *depth, const float *n
     if (ctx->n_views < 1) return SPLAT_ERR_STATE;
     CK(splat::launch_loss(depth, normal, alpha, target_depth, target_normal, ctx->n_pixels,
                           cfg->lambda_n, cfg->lambda_o, cfg->o_eps, cfg->rho_exp, dL_ddepth, dL_dnormal,
-                          dL_dalpha, loss_out, static_cast<cudaStream_t>(stream), false, ctx->d_views,
-                          ctx->n_views, nullptr, cfg->normal_mode));
+                          dL_dalpha, loss_out, static_cast<cudaStream_t>(stream), false,
+                          ctx->d_views, ctx->n_views, nullptr, cfg->normal_mode));
     return SPLAT_OK;
 }
 
@@ -933,8 +932,8 @@ SPLAT_API int splat_refine_step(splat_ctx *ctx, float *pos_logit, float *quat, f
                           loss_cfg->normal_mode));
     const bool prof = ctx->profiling && !capturing(st);
     if (prof) {
-        CK(cudaEventRecord(ctx->stage_ev[6], st));
-        ctx->stage_rec[6] = true;
+        CK(cudaEventRecord(ctx->stage_ev[4], st));
+        ctx->stage_rec[4] = true;
     }
     r = backward_core(ctx, &g, gd, gn, ga, st, true);
     if (r) return r;
@@ -963,8 +962,8 @@ SPLAT_API int splat_refine_step(splat_ctx *ctx, float *pos_logit, float *quat, f
     a.chain = splat::chained_size(n * ctx->n_views);
     CK(splat::launch_adam_fused(a, ctx->d_wgrad, st));
     if (prof) {
-        CK(cudaEventRecord(ctx->stage_ev[7], st));
-        ctx->stage_rec[7] = true;
+        CK(cudaEventRecord(ctx->stage_ev[5], st));
+        ctx->stage_rec[5] = true;
     }
     ctx->launches += 2;   // loss, fused Adam
     return SPLAT_OK;
@@ -1093,22 +1092,22 @@ SPLAT_API int splat_kernel_times(splat_ctx *ctx, float *fwd_ms, float *bwd_ms)
 SPLAT_API int splat_stage_times(splat_ctx *ctx, float *ms)
 {
     if (!ctx || !ms) return SPLAT_ERR_INVALID_ARG;
-    // the loss runs between the end of the forward compositing and event 6, the fused Adam
-    // between the end of the backward and event 7; the binning has no global range sort and no
+    // the loss runs between the end of the forward compositing and event 4, the fused Adam
+    // between the end of the backward and event 5; the binning has no global range sort and no
     // separate ranges pass, which take no time in a render that was profiled
     struct Span {
         cudaEvent_t a, b;
         bool ok;
     };
-    const Span binning{nullptr, nullptr, ctx->stage_rec[0] && ctx->stage_rec[4]};
+    const Span binning{nullptr, nullptr, ctx->stage_rec[0] && ctx->stage_rec[3]};
     const Span spans[7] = {
         {ctx->stage_ev[0], ctx->stage_ev[1], ctx->stage_rec[0] && ctx->stage_rec[1]},
         binning,
-        {ctx->stage_ev[1], ctx->stage_ev[3], ctx->stage_rec[1] && ctx->stage_rec[3]},
-        {ctx->stage_ev[3], ctx->stage_ev[4], ctx->stage_rec[3] && ctx->stage_rec[4]},
+        {ctx->stage_ev[1], ctx->stage_ev[2], ctx->stage_rec[1] && ctx->stage_rec[2]},
+        {ctx->stage_ev[2], ctx->stage_ev[3], ctx->stage_rec[2] && ctx->stage_rec[3]},
         binning,
-        {ctx->ev[1], ctx->stage_ev[6], ctx->rec_fwd && ctx->stage_rec[6]},
-        {ctx->ev[3], ctx->stage_ev[7], ctx->rec_bwd && ctx->stage_rec[7]},
+        {ctx->ev[1], ctx->stage_ev[4], ctx->rec_fwd && ctx->stage_rec[4]},
+        {ctx->ev[3], ctx->stage_ev[5], ctx->rec_bwd && ctx->stage_rec[5]},
     };
     for (int k = 0; k < 7; ++k) {
         ms[k] = spans[k].ok ? 0.0f : -1.0f;

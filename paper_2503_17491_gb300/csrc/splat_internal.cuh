@@ -249,7 +249,7 @@ struct PairRec {
 };
 static_assert(sizeof(PairRec) == 16, "PairRec is 16 bytes");
 
-enum : uint32_t { kCountMask = 0x3FFFFFFFu, kPairFlip = 1u << 30, kPairInvalid = 1u << 31 };
+enum : uint32_t { kPairFlip = 1u << 30, kPairInvalid = 1u << 31 };
 
 // ---------------------------------------------------------------------------------------------
 // tile geometry shared by the binning and the render kernels
@@ -378,8 +378,6 @@ __device__ __forceinline__ f2 f2_add(f2 a, f2 b)
     return r;
 }
 
-__device__ __forceinline__ f2 f2_neg(f2 a) { return f2{-a.h, -a.l}; }
-
 // Sum_j M_j x_j + u in float-pair arithmetic, rounded to one float (x exact floats).
 __device__ __forceinline__ float f2_dot3_add(f2 m0, f2 m1, f2 m2, float x0, float x1, float x2,
                                              f2 u)
@@ -454,8 +452,6 @@ __device__ __forceinline__ void chain_params(const float4 pl, const float4 q, co
 // ---------------------------------------------------------------------------------------------
 // kernel launchers (defined in the .cu files)
 // ---------------------------------------------------------------------------------------------
-struct Workspace;   // host-side bookkeeping, defined in splat_abi.cu
-
 // Record the text of a failed CUDA call for splat_last_cuda_error (thread-local) and return
 // SPLAT_ERR_CUDA.
 int cuda_fail(cudaError_t e, const char *what);
@@ -643,7 +639,7 @@ struct RenderArgs {
     const uint2 *entries;
     const uint8_t *entry_blocks;  // per list entry: the 4 x 8 blocks of its tile it meets
     int64_t n_tiles;
-    const uint32_t *split;        // leading tiles of the order whose blocks go to 4 warps, then to 2
+    const uint32_t *split;        // leading tiles of the order whose blocks go to 4 warps, to 2
     float alpha_min, alpha_max, t_min, sigma;
     // forward outputs (packed pixels)
     float *depth, *normal, *alpha;

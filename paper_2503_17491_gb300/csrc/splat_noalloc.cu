@@ -3,10 +3,10 @@
 // that runs after its process has handed all device memory to another allocator, or that must
 // not call cudaMalloc once it is running.
 //
-// Every buffer the render pipeline needs (projection records, sort buffers and histograms, tile
-// lists, tile tables, per-pixel auxiliaries, counters) lives in one file-scope __device__ array,
-// g_noalloc_scratch, sized for the limits below.  The host-side tables are built in file-scope
-// host arrays.  Nothing here calls cudaMalloc, cudaFree, malloc or new.
+// Every buffer the render pipeline needs (pixel rectangles and touching pairs, tile counts, tile
+// lists and their segments, tile tables, per-pixel auxiliaries, counters) lives in one file-scope
+// __device__ array, g_noalloc_scratch, sized for the limits below.  The host-side tables are built
+// in file-scope host arrays.  Nothing here calls cudaMalloc, cudaFree, malloc or new.
 //
 // Limits: at most kMaxGaussians primitives, kMaxRows image rows, kMaxPixels pixels, kMaxTiles
 // tiles and kMaxPairs (tile, primitive) pairs; larger requests return SPLAT_ERR_INVALID_ARG

@@ -319,9 +319,9 @@ cudaError_t launch_loss(const float *depth, const float *normal, const float *al
     int64_t blocks = (n_pixels + 255) / 256;
     if (blocks > 4096) blocks = 4096;
     auto kern = normal_mode == 1 ? k_loss<1> : k_loss<0>;
-    return launch_chained(chain, kern, dim3(static_cast<unsigned>(blocks)), 256, 0, st, depth, normal,
-                          alpha, t_depth, t_normal, n_pixels, lambda_n, lambda_o, o_eps, rho_exp,
-                          g_depth, g_normal, g_alpha, loss_out, views, n_views, active);
+    return launch_chained(chain, kern, dim3(static_cast<unsigned>(blocks)), 256, 0, st, depth,
+                          normal, alpha, t_depth, t_normal, n_pixels, lambda_n, lambda_o, o_eps,
+                          rho_exp, g_depth, g_normal, g_alpha, loss_out, views, n_views, active);
 }
 
 cudaError_t launch_adam(const AdamArgs &a, const float4 *g_pl, const float4 *g_q,
@@ -335,16 +335,16 @@ cudaError_t launch_adam(const AdamArgs &a, const float4 *g_pl, const float4 *g_q
 cudaError_t launch_adam_fused(const AdamArgs &a, const float4 *wgrad, cudaStream_t st)
 {
     if (a.n <= 0) return cudaSuccess;
-    return launch_chained(a.chain, k_adam_fused, dim3(static_cast<unsigned>((a.n + 255) / 256)), 256, 0, st,
-                          a, wgrad);
+    return launch_chained(a.chain, k_adam_fused, dim3(static_cast<unsigned>((a.n + 255) / 256)),
+                          256, 0, st, a, wgrad);
 }
 
 cudaError_t launch_backward_start(const RefineStart &s, float4 *wgrad, int64_t n, bool chain,
                                   cudaStream_t st)
 {
     const int64_t n4 = 4 * n;
-    return launch_chained(chain, k_backward_start, dim3(static_cast<unsigned>(n4 > 0 ? (n4 + 255) / 256 : 1)),
-                          256, 0, st, s, wgrad, n4);
+    const unsigned blocks = static_cast<unsigned>(n4 > 0 ? (n4 + 255) / 256 : 1);
+    return launch_chained(chain, k_backward_start, dim3(blocks), 256, 0, st, s, wgrad, n4);
 }
 
 cudaError_t launch_step_inc(int32_t *step, cudaStream_t st)

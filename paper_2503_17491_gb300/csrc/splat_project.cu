@@ -330,7 +330,8 @@ __device__ __forceinline__ float approx_rsqrt(float x)
     return y;
 }
 
-// atan z for |z| <= 0.42 (the next term of the series is below 1.3e-7) and for |z| <= 0.27 (2.5e-7)
+// atan z for |z| <= tan(pi/8) (the next term of the series is below 1.3e-7) and for |z| <= 0.27
+// (8.5e-7; 5.2e-7 at the 0.2555 that an azimuth reaches)
 __device__ __forceinline__ float approx_atan_mid(float z)
 {
     const float z2 = z * z;
@@ -367,13 +368,13 @@ __device__ __forceinline__ float approx_atan(float y, float x)
 // kQuickUnsure.
 //
 // The extreme elevations and azimuths are taken over the vertices.  Against the contract's values
-// these are off by the rounding of both computations, below 2.5e-6 rad (positions to a few units
-// in 2^24 of the range, angles to 2^-22, series and approximate quotients to 4e-7), for which
-// kQuickAngle = 5e-6 stands, plus the final product's rounding of up to a few 2^-24 of the image
-// size in pixels; and the contract also takes the interior extrema of the edges.  Where a
-// great-circle arc of length phi reaches its highest elevation theta_m inside, its nearer end is
-// at most tan(theta_m) phi^2 / 8 lower: `bulge` bounds that for the longest edge, and only widens
-// the box.  So the contract's row bounds lie in [vhi - eps - bulge, vhi + eps] and
+// these are off by the rounding of both computations, below 3e-6 rad (positions to a few units in
+// 2^24 of the range, angles to 2^-22, series to 1e-6, approximate reciprocals and roots to 2.4e-7),
+// for which kQuickAngle stands at twice that, plus the final product's rounding of up to a few
+// 2^-24 of the image size in pixels; and the contract also takes the interior extrema of the
+// edges.  Where a great-circle arc of length phi reaches its highest elevation theta_m inside, its
+// nearer end is at most tan(theta_m) phi^2 / 8 lower: `bulge` bounds that for the longest edge, and
+// only widens the box.  So the contract's row bounds lie in [vhi - eps - bulge, vhi + eps] and
 // [vlo - eps, vlo + eps + bulge], its column bounds within eps; an integer is taken only when both
 // ends of its interval round to it.
 enum { kQuickUnsure = 0, kQuickEmpty, kQuickBox };

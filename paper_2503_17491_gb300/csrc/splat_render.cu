@@ -1132,7 +1132,8 @@ cudaError_t launch_render_fwd(const RenderArgs &a, int tile_h, int tile_w, int g
         constexpr int h = decltype(TH)::value, w = decltype(TW)::value;
         const cudaError_t e = fwd_prepare<h, w>();
         if (e != cudaSuccess) return e;
-        return launch_chained(a.chain, k_render_fwd<h, w>, dim3(grid), kBlock, sizeof(FwdShared), st, a);
+        return launch_chained(a.chain, k_render_fwd<h, w>, dim3(grid), kBlock, sizeof(FwdShared),
+                              st, a);
     });
 }
 
@@ -1143,7 +1144,8 @@ cudaError_t launch_render_bwd(const RenderArgs &a, int tile_h, int tile_w, int g
         constexpr int h = decltype(TH)::value, w = decltype(TW)::value;
         const cudaError_t e = bwd_prepare<h, w>();
         if (e != cudaSuccess) return e;
-        return launch_chained(a.chain, k_render_bwd<h, w>, dim3(grid), kBlock, sizeof(BwdShared), st, a);
+        return launch_chained(a.chain, k_render_bwd<h, w>, dim3(grid), kBlock, sizeof(BwdShared),
+                              st, a);
     });
 }
 

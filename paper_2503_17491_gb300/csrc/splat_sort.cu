@@ -110,8 +110,8 @@ __device__ __forceinline__ T block_excl_scan(T v, T *s_warp, T *total)
 // (rooms, streets, blocks and a city, 1 to 12 views of 32 x 512 to 128 x 2048, 5,000 to 2 M
 // primitives, all tile shapes, longest lists of 1 to 12 shares), forward and backward.  Splitting
 // against whole blocks, geometric mean of 600 frames by the shares of their longest list: 0.93 at 1
-// to 1.5, 0.97 up to 2, 1.02 up to 2.5, 1.11 up to 3, 1.17 up to 4, 1.33 up to 6, 1.63 above.  Single
-// frames scatter widely about that, so the mean hardly depends on the line (660 frames, against
+// to 1.5, 0.97 up to 2, 1.02 up to 2.5, 1.11 up to 3, 1.17 up to 4, 1.33 up to 6, 1.63 above.
+// Single frames scatter widely about that, so the mean hardly depends on the line (660, against
 // the better of both in each: 1.024 splitting all, 1.016 with the line at 2.0, 1.020 at 2.4, 1.024
 // at 2.65, 1.031 at 3.0, 1.228 splitting none), but the frames that splitting makes slower do: of
 // 600, 149 by more than 3 % without a line, 72 with the line at 2.0, 48 at 2.4, 28 at 2.65, the
@@ -281,11 +281,10 @@ __device__ __forceinline__ bool chunk_of(const BinArgs &A, Chunk &c)
 }
 
 // f(tile of the band, range key bits, primitive in the view) for every tile of the band of every
-// touching pair of the chunk, 32 pairs a warp at a time, kUnitLoads of them read ahead (the range keys only with
-// kKeys).  While no
-// pair of a warp touches more than kLaneTiles tiles, every lane walks its own; otherwise the warp
-// numbers the tiles of its 32 pairs by a prefix sum and gives one to every lane, so that one wide
-// pair costs its warp no more than as many narrow ones.
+// touching pair of the chunk, 32 pairs a warp at a time, kUnitLoads of them read ahead (the range
+// keys only with kKeys).  While no pair of a warp touches more than kLaneTiles tiles, every lane
+// walks its own; otherwise the warp numbers the tiles of its 32 pairs by a prefix sum and gives one
+// to every lane, so that one wide pair costs its warp no more than as many narrow ones.
 constexpr int kLaneTiles = 8, kUnitLoads = 4;
 
 template <bool kBanded, bool kKeys, typename F>
@@ -377,8 +376,8 @@ __device__ __forceinline__ void for_each_entry(const Chunk &c, F f)
 // neighbouring threads' pairs fall on a few hundred tiles of one view, and same-address atomics
 // in L2 serialise (emission of 5.3 M entries: 0.95 ms with an atomic per entry).  A view of more
 // tiles than the counters hold is taken in bands, each by its own CTAs, which pass over the pairs
-// that miss their band: eleven 64 x 1024 views and one of 128 x 32,000 over 500 k primitives (11.6 M
-// entries), counted and emitted with global atomics 0.63 ms, in bands 0.29; the wide view alone
+// that miss their band: eleven 64 x 1024 views and one of 128 x 32,000 over 500 k primitives (11.6
+// M entries), counted and emitted with global atomics 0.63 ms, in bands 0.29; the wide view alone
 // (16,000 tiles, 6.2 M entries) 0.13 either way.
 template <bool kBanded>
 __global__ void __launch_bounds__(kChunkThreads) k_count(const BinArgs A)
@@ -638,10 +637,10 @@ __device__ void recut(const BinArgs &A, SegmentRun run, uint32_t tile, int level
     }
 }
 
-// Cuts one list until no segment is above kListCap.  The first cut of a list that one CTA cuts takes
-// the fixed bins, where few lists of that length have more than kListCap entries in a bin; what is
-// oversized after it (a wall at one distance, a dense map) is cut again, exactly.  An oversized
-// segment is one bin, and a bin of an exact cut spans at most 2^-11 of the keys' range: keys have
+// Cuts one list until no segment is above kListCap.  The first cut of a list that one CTA cuts
+// takes the fixed bins, where few lists of that length have more than kListCap entries in a bin;
+// what is oversized after it (a wall at one distance, a dense map) is cut again, exactly.  An
+// oversized segment is one bin, and a bin of an exact cut spans at most 2^-11 of the keys' range: keys have
 // 63 bits at most and are unique, so that the bins of the fifth exact cut span no more than 8 keys.
 // A cluster cuts exactly from the start, goes on as one while more than half of the list stays in
 // one segment, and shares the rest out to its CTAs.
@@ -718,8 +717,9 @@ __device__ __forceinline__ void order_pair(uint64_t &a, uint64_t &b)
     b = hi;
 }
 
-// Batcher's odd-even merge sort of E keys in registers: phase p merges sorted runs of p keys, in
-// steps of comparison distance q = p, p / 2, ..., 1
+// Batcher's odd-even merge sort (Sorting networks and their applications, 1968) of E keys in
+// registers: phase p merges sorted runs of p keys, in steps of comparison distance q = p, p / 2,
+// ..., 1
 template <int E, int P, int Q>
 __device__ __forceinline__ void network(uint64_t (&k)[E])
 {
@@ -736,7 +736,7 @@ __device__ __forceinline__ void network(uint64_t (&k)[E])
 // Sorts the n <= G * E keys src[0 .. n) into s (padded places), with G threads (a warp or the
 // CTA) of E keys each: every thread sorts its keys in registers (network), then
 // runs of E, 2E, ... keys are merged pairwise, each thread finding its E outputs by a binary
-// search along its diagonal (merge path).
+// search along its diagonal (merge path: Odeh, Green, Mwassi, Shmueli, Birk 2012).
 template <int E, int G>
 __device__ __forceinline__ void sort_keys(const uint64_t *src, int n, uint64_t *s, int g)
 {
@@ -1030,8 +1030,8 @@ bool chained(const BinArgs &a) { return chained_size(a.n * a.n_views); }
 
 }  // namespace
 
-// k_lists' shared memory is above the 48 KB static limit.  Its three CTAs need 159 KB of an SM's 228;
-// what is left is L1, which the list sort lives on.  Left to the driver, a build whose registers
+// k_lists' shared memory is above the 48 KB static limit.  Its three CTAs need 159 of an SM's 228
+// KB; what is left is L1, which the list sort lives on.  Left to the driver, a build whose registers
 // allow a fourth CTA gets the shared memory for one and 20 KB of L1: 12 x 500 k primitives 0.096 ->
 // 0.130 ms.
 cudaError_t prepare_lists()
@@ -1080,8 +1080,8 @@ cudaError_t launch_lists(const BinArgs &a, cudaStream_t st)
         e = launch_cluster(chained(a), ranks, k_split, dim3(grid), kSplitThreads, 0, st, a);
         if (e != cudaSuccess) return e;
     }
-    return launch_chained(chained(a), k_lists, dim3(kListCtas * a.sms), kListThreads, sizeof(ListShared), st,
-                          a);
+    return launch_chained(chained(a), k_lists, dim3(kListCtas * a.sms), kListThreads,
+                          sizeof(ListShared), st, a);
 }
 
 }  // namespace splat

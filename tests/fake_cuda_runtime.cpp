@@ -36,7 +36,8 @@ std::vector<Config> g_config;
 cudaError_t launch(const void *fn, dim3 grid, dim3 block, size_t shared, bool chained)
 {
     const auto it = g_limit.find({g_device, fn});
-    if (shared > (it == g_limit.end() ? size_t{48} << 10 : it->second)) return cudaErrorInvalidValue;
+    const size_t limit = it == g_limit.end() ? size_t{48} << 10 : it->second;
+    if (shared > limit) return cudaErrorInvalidValue;
     g_launches.push_back(Launch{names()[fn], grid, block, shared, chained});
     return cudaSuccess;
 }
@@ -64,8 +65,8 @@ extern "C" {
 void **__cudaRegisterFatBinary(void *) { return static_cast<void **>(std::calloc(1, 8)); }
 void __cudaRegisterFatBinaryEnd(void **) {}
 void __cudaUnregisterFatBinary(void **) {}
-void __cudaRegisterFunction(void **, const char *host, char *, const char *name, int, void *, void *,
-                            void *, void *, int *)
+void __cudaRegisterFunction(void **, const char *host, char *, const char *name, int, void *,
+                            void *, void *, void *, int *)
 {
     names()[host] = name;
 }
@@ -113,8 +114,8 @@ cudaError_t cudaFuncSetAttribute(const void *fn, cudaFuncAttribute attr, int val
         g_limit[{g_device, fn}] = static_cast<size_t>(value);
     return cudaSuccess;
 }
-cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *, int, size_t,
-                                                                   unsigned)
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *, int,
+                                                                   size_t, unsigned)
 {
     *n = 1;
     return cudaSuccess;
@@ -131,7 +132,7 @@ cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int)
 }
 cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
-const char *cudaGetErrorString(cudaError_t e) { return e == cudaSuccess ? "no error" : "fake error"; }
+const char *cudaGetErrorString(cudaError_t e) { return e == cudaSuccess ? "none" : "fake error"; }
 cudaError_t cudaGetSymbolAddress(void **p, const void *)
 {
     static void *mem = std::calloc(1, size_t{64} << 20);
