@@ -433,10 +433,12 @@ def run_ours(args):
 
     # per-stage times of the same eager steps against the HBM roofline, with each stage's
     # algorithmic bytes (what its definition reads and writes once): n primitives, V keyframes,
-    # nv (view, primitive) pairs that touch a tile, M list entries, T tiles, P pixels
+    # nv (view, primitive) pairs that touch a tile, M list entries, T tiles, P pixels.  A
+    # primitive's 168 bytes in the projection: 40 read, 64 staged for the compositing, and its 64
+    # of gradient accumulators, which the projection of a refinement step clears
     hbm = float(peaks.get("hbm_gbs", 6800.0))
     n, V, nv, M, T = scene.n, len(views), s2["n_touching"], s2["n_pairs"], s2["n_tiles"]
-    stage_bytes = {"projection": 104 * n + 8 * n * V + 12 * nv,
+    stage_bytes = {"projection": 168 * n + 8 * n * V + 12 * nv,
                    "emission": 20 * nv + 8 * M + 20 * T,
                    "tile sort": 25 * M,
                    "loss": 52 * pixels,
