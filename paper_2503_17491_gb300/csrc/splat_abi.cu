@@ -488,15 +488,18 @@ SPLAT_API int splat_ctx_create(const splat_render_config *cfg, const splat_capac
     if (e == cudaSuccess) e = cudaMemset(c->d_counters, 0, kCounters * sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMemset(c->d_bwd_evals, 0, sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(c->d_zero, 0, kZeroTiles * sizeof(uint32_t));
+    int fwd_ctas = 1, bwd_ctas = 1;
     if (e == cudaSuccess) e = splat::prepare_lists();
+    if (e == cudaSuccess) e = splat::prepare_render_fwd(cfg->tile_h, cfg->tile_w, &fwd_ctas);
+    if (e == cudaSuccess) e = splat::prepare_render_bwd(cfg->tile_h, cfg->tile_w, &bwd_ctas);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         int r = cuda_fail(e, "splat_ctx_create");
         free_ctx(c);
         return r;
     }
-    c->grid_fwd = c->sms * splat::render_occupancy(cfg->tile_h, cfg->tile_w, false);
-    c->grid_bwd = c->sms * splat::render_occupancy(cfg->tile_h, cfg->tile_w, true);
+    c->grid_fwd = c->sms * std::max(fwd_ctas, 1);
+    c->grid_bwd = c->sms * std::max(bwd_ctas, 1);
     *out = c;
     return SPLAT_OK;
 }

@@ -67,9 +67,10 @@ cudaError_t launch_chained(bool chain, void (*kernel)(P...), dim3 grid, unsigned
 }
 
 // Raises a kernel's dynamic shared memory limit above the default 48 KB, once on each device: the
-// attribute belongs to the current device's copy of the kernel.  carveout (percent, negative for
-// the driver's choice): how much of an SM's memory is shared, the rest is L1.  One static object
-// per kernel; a failed call is tried again by the next one.
+// attribute belongs to the current device's copy of the kernel.  Called where a context, or the
+// call without one, is set up, not at every launch.  carveout (percent, negative for the driver's
+// choice): how much of an SM's memory is shared, the rest is L1.  One static object per kernel; a
+// failed call is tried again by the next one.
 class SharedLimit {
 public:
     template <typename Kernel>
@@ -665,7 +666,9 @@ cudaError_t launch_render_fwd(const RenderArgs &a, int tile_h, int tile_w, int g
                               cudaStream_t st);
 cudaError_t launch_render_bwd(const RenderArgs &a, int tile_h, int tile_w, int grid,
                               cudaStream_t st);
-int render_occupancy(int tile_h, int tile_w, bool backward);
+// once per device, before the first launch on it; *ctas: how many an SM takes
+cudaError_t prepare_render_fwd(int tile_h, int tile_w, int *ctas);
+cudaError_t prepare_render_bwd(int tile_h, int tile_w, int *ctas);
 
 cudaError_t launch_param_grads(const float4 *pos_logit, const float4 *quat, const float2 *log_scale,
                                const float4 *wgrad, int64_t n, float4 *g_pos_logit, float4 *g_quat,

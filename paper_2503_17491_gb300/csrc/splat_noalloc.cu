@@ -264,8 +264,10 @@ extern "C" SPLAT_API int splat_render_noalloc(const splat_gaussians *g,
     NA_CK(cudaMemsetAsync(tile_count, 0, 4 * n_tiles, st));
     NA_CK(cudaMemsetAsync(evals, 0, 8 * 3, st));
 
-    int sms = 0;
+    int sms = 0, ctas = 1;
     NA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    NA_CK(splat::prepare_lists());
+    NA_CK(splat::prepare_render_fwd(th, tw, &ctas));
     splat::ProjectArgs pa{};
     pa.pos_logit = reinterpret_cast<const float4 *>(g->pos_logit);
     pa.quat = reinterpret_cast<const float4 *>(g->quat_wxyz);
@@ -314,7 +316,7 @@ extern "C" SPLAT_API int splat_render_noalloc(const splat_gaussians *g,
     ba.status = cnt + 1;
     ba.bin = cnt + kCountersBin;
     ba.sms = sms;
-    const int grid = sms * splat::render_occupancy(th, tw, false);
+    const int grid = sms * (ctas > 0 ? ctas : 1);
     ba.warps = static_cast<uint32_t>(grid) * (splat::kBlock / 32);
     ba.rec_cap = 0;   // no contributor records (forward only)
     ba.n_rows = evals + 2;

@@ -1110,28 +1110,11 @@ cudaError_t dispatch(int th, int tw, K k)
 
 }  // namespace
 
-// both kernels' shared memory is above the 48 KB static limit: allow it for every instantiation
-template <int TH, int TW>
-cudaError_t fwd_prepare()
-{
-    static SharedLimit limit;
-    return limit.raise(k_render_fwd<TH, TW>, sizeof(FwdShared));
-}
-
-template <int TH, int TW>
-cudaError_t bwd_prepare()
-{
-    static SharedLimit limit;
-    return limit.raise(k_render_bwd<TH, TW>, sizeof(BwdShared));
-}
-
 cudaError_t launch_render_fwd(const RenderArgs &a, int tile_h, int tile_w, int grid,
                               cudaStream_t st)
 {
     return dispatch(tile_h, tile_w, [&](auto TH, auto TW) {
         constexpr int h = decltype(TH)::value, w = decltype(TW)::value;
-        const cudaError_t e = fwd_prepare<h, w>();
-        if (e != cudaSuccess) return e;
         return launch_chained(a.chain, k_render_fwd<h, w>, dim3(grid), kBlock, sizeof(FwdShared),
                               st, a);
     });
@@ -1142,30 +1125,34 @@ cudaError_t launch_render_bwd(const RenderArgs &a, int tile_h, int tile_w, int g
 {
     return dispatch(tile_h, tile_w, [&](auto TH, auto TW) {
         constexpr int h = decltype(TH)::value, w = decltype(TW)::value;
-        const cudaError_t e = bwd_prepare<h, w>();
-        if (e != cudaSuccess) return e;
         return launch_chained(a.chain, k_render_bwd<h, w>, dim3(grid), kBlock, sizeof(BwdShared),
                               st, a);
     });
 }
 
-int render_occupancy(int tile_h, int tile_w, bool backward)
+// both kernels' shared memory is above the 48 KB static limit: allow it for every instantiation
+cudaError_t prepare_render_fwd(int tile_h, int tile_w, int *ctas)
 {
-    int blocks = 0;
-    dispatch(tile_h, tile_w, [&](auto TH, auto TW) {
+    return dispatch(tile_h, tile_w, [&](auto TH, auto TW) {
         constexpr int h = decltype(TH)::value, w = decltype(TW)::value;
-        if (backward) {
-            const cudaError_t e = bwd_prepare<h, w>();
-            if (e != cudaSuccess) return e;
-            return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_render_bwd<h, w>,
-                                                                 kBlock, sizeof(BwdShared));
-        }
-        const cudaError_t e = fwd_prepare<h, w>();
+        static SharedLimit limit;
+        const cudaError_t e = limit.raise(k_render_fwd<h, w>, sizeof(FwdShared));
         if (e != cudaSuccess) return e;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_render_fwd<h, w>, kBlock,
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, k_render_fwd<h, w>, kBlock,
                                                              sizeof(FwdShared));
     });
-    return blocks > 0 ? blocks : 1;
+}
+
+cudaError_t prepare_render_bwd(int tile_h, int tile_w, int *ctas)
+{
+    return dispatch(tile_h, tile_w, [&](auto TH, auto TW) {
+        constexpr int h = decltype(TH)::value, w = decltype(TW)::value;
+        static SharedLimit limit;
+        const cudaError_t e = limit.raise(k_render_bwd<h, w>, sizeof(BwdShared));
+        if (e != cudaSuccess) return e;
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, k_render_bwd<h, w>, kBlock,
+                                                             sizeof(BwdShared));
+    });
 }
 
 cudaError_t launch_param_grads(const float4 *pos_logit, const float4 *quat, const float2 *log_scale,

@@ -690,7 +690,10 @@ __global__ void __launch_bounds__(kSplitThreads) k_split(const BinArgs A)
     const uint32_t n_long = A.bin[kBinLong], n_huge = all.ranks > 1 ? A.bin[kBinHuge] : 0u;
     for (uint32_t l = blockIdx.x / all.ranks; l < n_huge; l += gridDim.x / all.ranks)
         split_list(A, A.order[l], sh, all);
-    for (uint32_t l = n_huge + blockIdx.x; l < n_long; l += gridDim.x) {
+    // the longest of the others first to the CTAs that had no part in a huge one
+    const uint32_t busy = min(n_huge * all.ranks, gridDim.x);
+    const uint32_t place = blockIdx.x < busy ? blockIdx.x + gridDim.x - busy : blockIdx.x - busy;
+    for (uint32_t l = n_huge + place; l < n_long; l += gridDim.x) {
         split_list(A, A.order[l], sh, one);
         __syncthreads();
     }
@@ -1071,13 +1074,12 @@ cudaError_t launch_emit(const BinArgs &args, cudaStream_t st)
 cudaError_t launch_lists(const BinArgs &a, cudaStream_t st)
 {
     if (a.n <= 0) return cudaSuccess;
-    cudaError_t e = prepare_lists();
-    if (e != cudaSuccess) return e;
     // a list holds each primitive once: below kListCap primitives none is long
     if (a.n >= kListCap) {
         const int ranks = a.n >= kHugeList ? kSplitCluster : 1;
         const int grid = a.sms >= ranks ? a.sms / ranks * ranks : ranks;
-        e = launch_cluster(chained(a), ranks, k_split, dim3(grid), kSplitThreads, 0, st, a);
+        const cudaError_t e =
+            launch_cluster(chained(a), ranks, k_split, dim3(grid), kSplitThreads, 0, st, a);
         if (e != cudaSuccess) return e;
     }
     return launch_chained(chained(a), k_lists, dim3(kListCtas * a.sms), kListThreads,

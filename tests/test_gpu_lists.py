@@ -344,3 +344,29 @@ def test_a_wide_view_costs_the_others_nothing():
         s.views = views
         ms.append(_stage(s, "emission", max_pairs=1 << 24))
     assert ms[2] <= 1.5 * (ms[0] + ms[1]), ms
+
+
+@pytest.mark.parametrize("n", [70_000, 600_000])
+def test_clusters_under_capture(n):
+    """A render whose list is cut by clusters, chained (up to 2^19 pairs) and not, replayed from a
+    graph: the same images and lists as from plain launches."""
+    rng = np.random.default_rng(n)
+    s = _one_tile(n, rng.uniform(2.0, 60.0, n), 4)
+    ctx = make_ctx(s.n, s.views)
+    dev = to_dev(s)
+    plain = [t.clone() for t in ctx.render(*dev)]
+    lists = ctx.sorted_lists()
+    out = ctx.alloc_images()
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        ctx.render(*dev, out=out, stream=torch.cuda.current_stream())
+    for _ in range(2):
+        for t in out:
+            t.zero_()
+        graph.replay()
+    torch.cuda.synchronize()
+    assert ctx.status() == 0
+    assert all(torch.equal(x, y) for x, y in zip(plain, out))
+    for x, y in zip(lists, ctx.sorted_lists()):
+        np.testing.assert_array_equal(x, y)
