@@ -724,8 +724,7 @@ SPLAT_API int splat_render_views_backward(splat_ctx *ctx, const splat_gaussians 
                                  reinterpret_cast<const float2 *>(g->log_scale), ctx->d_wgrad, g->n,
                                  reinterpret_cast<float4 *>(g_pos_logit),
                                  reinterpret_cast<float4 *>(g_quat),
-                                 reinterpret_cast<float2 *>(g_log_scale), accumulate, st,
-                                 splat::chained_size(g->n * ctx->n_views)));
+                                 reinterpret_cast<float2 *>(g_log_scale), accumulate, st));
     ctx->launches += 1;
     return SPLAT_OK;
 }

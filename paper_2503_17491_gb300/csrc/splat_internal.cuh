@@ -672,7 +672,7 @@ cudaError_t prepare_render_bwd(int tile_h, int tile_w, int *ctas);
 
 cudaError_t launch_param_grads(const float4 *pos_logit, const float4 *quat, const float2 *log_scale,
                                const float4 *wgrad, int64_t n, float4 *g_pos_logit, float4 *g_quat,
-                               float2 *g_log_scale, int accumulate, cudaStream_t st, bool chain);
+                               float2 *g_log_scale, int accumulate, cudaStream_t st);
 
 // active (nullable): pixels of views with active[v] == 0 count as invalid (views: the registered
 // views, for the pixel -> view lookup).  normal_mode 0: normal term against t_normal; 1:

@@ -1157,13 +1157,12 @@ cudaError_t prepare_render_bwd(int tile_h, int tile_w, int *ctas)
 
 cudaError_t launch_param_grads(const float4 *pos_logit, const float4 *quat, const float2 *log_scale,
                                const float4 *wgrad, int64_t n, float4 *g_pos_logit, float4 *g_quat,
-                               float2 *g_log_scale, int accumulate, cudaStream_t st, bool chain)
+                               float2 *g_log_scale, int accumulate, cudaStream_t st)
 {
     (void)log_scale;
     if (n <= 0) return cudaSuccess;
-    return launch_chained(chain, k_param_grads, dim3(static_cast<unsigned>((n + 255) / 256)), 256,
-                          0, st, pos_logit, quat, wgrad, n, g_pos_logit, g_quat, g_log_scale,
-                          accumulate);
+    return launch_chained(chained_size(n), k_param_grads, dim3(static_cast<unsigned>((n + 255) / 256)), 256, 0, st,
+                          pos_logit, quat, wgrad, n, g_pos_logit, g_quat, g_log_scale, accumulate);
 }
 
 }  // namespace splat

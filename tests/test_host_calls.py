@@ -96,17 +96,6 @@ def test_shared_memory_limits_on_a_second_device(host):
     assert len(names) == 6 and len(set(names)) == 3   # lists, forward, backward on either device
 
 
-@pytest.mark.parametrize("n,views,chained", [(1 << 18, 2, True), ((1 << 18) + 1, 2, False),
-                                             (200_000, 4, False), (1 << 19, 1, True)])
-def test_chained_launches_follow_the_pairs(host, n, views, chained):
-    """A call of up to 2^19 pairs chains every kernel, a larger one none: a kernel scheduled early
-    behind one that fills the SMs only costs."""
-    assert host.create(n, views) == 0
-    host.lib.fake_clear()
-    assert host.render() == 0 and host.backward() == 0
-    assert {x["chained"] for x in host.launches()} == {chained}
-
-
 def test_stage_times_of_a_profiled_render_add_up(host):
     """Every stage of a profiled render has a time (the two that the binning no longer has take
     none), so that the values can be summed; what was not recorded gives -1."""
