@@ -22,7 +22,11 @@ constexpr int kBlock = 256;          // threads per render CTA = pixels per tile
 // short as the gaps between them (render of 2,000 primitives 44 -> 36 us, 64x1024 over 100,000 with
 // autograd 329 -> 313 us, three scans over 83,000 336 -> 323 us) and costs where they fill the SMs,
 // since a kernel scheduled early crowds onto the SMs that come free first (1 M primitives 664 ->
-// 681 us, 12 x 500,000 2,209 -> 2,238 us): calls of up to kChainPairs pairs are chained.
+// 681 us, 12 x 500,000 2,209 -> 2,238 us): calls of up to kChainPairs pairs are chained.  The last
+// kernel of a backward, the parameter gradients, has no view loop and goes by the primitives
+// alone: the compositing kernel before it leaves no room on its SMs, so that being scheduled early
+// only hides the launch (render and backward of 4 x 200,000 primitives 394.1 -> 392.8 us, 8 x
+// 400,000 1,008.5 -> 1,005.5).
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void chain_wait()
 {

@@ -459,18 +459,20 @@ struct SplitShared {
     unsigned long long lo[32], hi[32];   // smallest and largest key by warp
 };
 
-// The CTAs that cut one list: one, or all of a cluster, each with a slice of the keys.
-struct SplitGroup {
+// The CTAs that cut one list, each with a slice of the keys: this one, or all of its cluster.
+struct OneCta {
+    static constexpr uint32_t ranks = 1, rank = 0;
+    __device__ void sync() const { __syncthreads(); }
+    template <typename T>
+    __device__ T *of(T *shared, uint32_t) const { return shared; }
+};
+struct WholeCluster {
     uint32_t ranks, rank;
-    __device__ void sync() const
-    {
-        if (ranks > 1) cooperative_groups::this_cluster().sync();
-        else __syncthreads();
-    }
+    __device__ void sync() const { cooperative_groups::this_cluster().sync(); }
     template <typename T>
     __device__ T *of(T *shared, uint32_t r) const
     {
-        return ranks > 1 ? cooperative_groups::this_cluster().map_shared_rank(shared, r) : shared;
+        return cooperative_groups::this_cluster().map_shared_rank(shared, r);
     }
 };
 
@@ -495,11 +497,12 @@ __device__ __forceinline__ void warp_range(unsigned long long &lo, unsigned long
 // gathered into segments of at most kListCap entries by the kSegTarget-entry stretch of the keys
 // their first entry falls into, and the keys scattered by bin into the other buffer.  A segment
 // above kListCap is a single bin.  The bins are
-// linear in the keys' bits, which for floats spaces them like the logarithm: with `exact` between
+// linear in the keys' bits, which for floats spaces them like the logarithm: with kExact between
 // the smallest and the largest key, which takes one more pass over them, else 128 an octave of
 // range from 2^-12 on (the ends take what lies beyond).
-__device__ SegmentRun cut(const BinArgs &A, uint32_t start, uint32_t len, uint32_t tile, int level,
-                          bool exact, SplitShared &sh, const SplitGroup &g)
+template <bool kExact, typename Group>
+__device__ __forceinline__ SegmentRun cut(const BinArgs &A, uint32_t start, uint32_t len,
+                                          uint32_t tile, int level, SplitShared &sh, const Group &g)
 {
     const int tid = threadIdx.x;
     const uint32_t s0 = static_cast<uint32_t>(uint64_t{len} * g.rank / g.ranks);
@@ -507,9 +510,9 @@ __device__ SegmentRun cut(const BinArgs &A, uint32_t start, uint32_t len, uint32
     const uint64_t *src = (level & 1 ? A.entries2 : A.entries) + start + s0;
     uint64_t *dst = (level & 1 ? A.entries : A.entries2) + start;
     for (int k = tid; k < kSplitBins; k += kSplitThreads) sh.bin[k] = 0u;
-    unsigned long long lo = uint64_t{(127 - 12) << 7} << 48;
-    int down = 48;
-    if (exact) {
+    unsigned long long lo = 0ull;
+    int down = 0;
+    if constexpr (kExact) {
         unsigned long long hi = 0ull;
         lo = ~0ull;
         for_each_key(src, n, [&](uint64_t e) {
@@ -532,8 +535,10 @@ __device__ SegmentRun cut(const BinArgs &A, uint32_t start, uint32_t len, uint32
     } else {
         __syncthreads();
     }
-    auto bin = [=](uint64_t e) {
-        return static_cast<uint32_t>(min(e < lo ? 0ull : (e - lo) >> down, kSplitBins - 1ull));
+    auto bin = [=](uint64_t e) -> uint32_t {
+        if constexpr (kExact) return static_cast<uint32_t>((e - lo) >> down);
+        const int b = static_cast<int>(e >> 48) - ((127 - 12) << 7);
+        return static_cast<uint32_t>(min(max(b, 0), kSplitBins - 1));
     };
     for_each_key(src, n, [&](uint64_t e) { atomicAdd(&sh.bin[bin(e)], 1u); });
     g.sync();
@@ -601,10 +606,10 @@ __device__ SegmentRun cut(const BinArgs &A, uint32_t start, uint32_t len, uint32
 
 // Cuts the segments of `run`, left by a cut at `level`, again until none holds more than kListCap
 // entries, depth first, by this CTA alone; it takes every ranks-th of the run.
-__device__ void recut(const BinArgs &A, SegmentRun run, uint32_t tile, int level, SplitShared &sh,
-                      const SplitGroup &g)
+template <typename Group>
+__device__ __noinline__ void recut(const BinArgs &A, SegmentRun run, uint32_t tile, int level,
+                                   SplitShared &sh, const Group &g)
 {
-    const SplitGroup one{1u, 0u};
     uint32_t next[kSplitLevels], end[kSplitLevels];   // by level: segments not yet looked at
     const int first = level;
     next[level] = run.begin;
@@ -630,7 +635,7 @@ __device__ void recut(const BinArgs &A, SegmentRun run, uint32_t tile, int level
         next[level] = at + 1;
         const uint32_t start = __ldcg(&A.segments[at].start), len = __ldcg(&A.segments[at].len);
         ++level;
-        run = cut(A, start, len, tile, level, true, sh, one);
+        run = cut<true>(A, start, len, tile, level, sh, OneCta{});
         if (threadIdx.x == 0) A.segments[at].len = 0u;   // read by all before the cut
         next[level] = run.begin;
         end[level] = run.oversized ? run.end : run.begin;
@@ -647,16 +652,23 @@ __device__ void recut(const BinArgs &A, SegmentRun run, uint32_t tile, int level
 // What the exact pass costs a list of 5,000 or 20,000 entries on one CTA: 4 us on 4.5 and 18.  What
 // it saves: 150,000 primitives of one tile within 0.1 mm of range, cut and sorted, 0.105 ms; left
 // in one segment and merged by one CTA 2.99.
-__device__ void split_list(const BinArgs &A, uint32_t tile, SplitShared &sh, const SplitGroup &g)
+__device__ void split_list(const BinArgs &A, uint32_t tile, SplitShared &sh)
+{
+    const uint2 rg = A.ranges[tile];
+    const SegmentRun run = cut<false>(A, rg.x, rg.y - rg.x, tile, 0, sh, OneCta{});
+    if (run.oversized) recut(A, run, tile, 0, sh, OneCta{});
+}
+
+__device__ void split_list(const BinArgs &A, uint32_t tile, SplitShared &sh, const WholeCluster &g)
 {
     const uint2 rg = A.ranges[tile];
     uint32_t start = rg.x, len = rg.y - rg.x;
     for (int level = 0;; ++level) {
-        SegmentRun run = cut(A, start, len, tile, level, level > 0 || g.ranks > 1, sh, g);
+        const SegmentRun run = cut<true>(A, start, len, tile, level, sh, g);
         if (!run.oversized) return;
         // a huge segment that the cluster goes on with
         uint32_t at = kFull;
-        if (g.ranks > 1 && level + 1 < kSplitLevels) {
+        if (level + 1 < kSplitLevels) {
             if (threadIdx.x == 0) sh.next = kFull;
             __syncthreads();
             for (uint32_t k = run.begin + threadIdx.x; k < run.end; k += kSplitThreads) {
@@ -686,7 +698,7 @@ __global__ void __launch_bounds__(kSplitThreads) k_split(const BinArgs A)
     chain_wait();
     __shared__ SplitShared sh;
     const auto cluster = cooperative_groups::this_cluster();
-    const SplitGroup all{cluster.num_blocks(), cluster.block_rank()}, one{1u, 0u};
+    const WholeCluster all{cluster.num_blocks(), cluster.block_rank()};
     const uint32_t n_long = A.bin[kBinLong], n_huge = all.ranks > 1 ? A.bin[kBinHuge] : 0u;
     for (uint32_t l = blockIdx.x / all.ranks; l < n_huge; l += gridDim.x / all.ranks)
         split_list(A, A.order[l], sh, all);
@@ -694,7 +706,7 @@ __global__ void __launch_bounds__(kSplitThreads) k_split(const BinArgs A)
     const uint32_t busy = min(n_huge * all.ranks, gridDim.x);
     const uint32_t place = blockIdx.x < busy ? blockIdx.x + gridDim.x - busy : blockIdx.x - busy;
     for (uint32_t l = n_huge + place; l < n_long; l += gridDim.x) {
-        split_list(A, A.order[l], sh, one);
+        split_list(A, A.order[l], sh);
         __syncthreads();
     }
 }

@@ -96,6 +96,19 @@ def test_shared_memory_limits_on_a_second_device(host):
     assert len(names) == 6 and len(set(names)) == 3   # lists, forward, backward on either device
 
 
+@pytest.mark.parametrize("n,views", [(1 << 18, 2), ((1 << 18) + 1, 2), (1 << 19, 1),
+                                     ((1 << 19) + 1, 1)])
+def test_chained_launches_follow_the_size(host, n, views):
+    """A call of up to 2^19 pairs chains every kernel, a larger one none but the parameter
+    gradients, which go by the primitives."""
+    assert host.create(n, views) == 0
+    host.lib.fake_clear()
+    assert host.render() == 0 and host.backward() == 0
+    last = [x["chained"] for x in host.launches() if "k_param_grads" in x["name"]]
+    rest = {x["chained"] for x in host.launches() if "k_param_grads" not in x["name"]}
+    assert last == [n <= 1 << 19] and rest == {n * views <= 1 << 19}
+
+
 def test_stage_times_of_a_profiled_render_add_up(host):
     """Every stage of a profiled render has a time (the two that the binning no longer has take
     none), so that the values can be summed; what was not recorded gives -1."""
