@@ -20,7 +20,7 @@
 // two passes of three launches each, whose per-tile ranking is one serial chain of shared memory
 // per warp; here an entry is written once and read by the list sort, in five launches.  From
 // pairs to lists, 12 views x 500 k primitives (5.3 M entries): 0.51 ms in 24 launches -> 0.23 ms
-// (count 0.032, layout 0.010, emission 0.062, split 0.024, lists 0.097); 64 tiles of 1,500
+// (count 0.032, layout 0.010, emission 0.067, split 0.030, lists 0.095); 64 tiles of 1,500
 // entries: 0.13 -> 0.022 ms.  The lists stage is bound by the shared-memory latency of its four
 // passes over the keys, the counting stages by instruction issue.
 // Everything runs on counts that stay on the device, with fixed launch shapes, so the pipeline
@@ -496,10 +496,10 @@ __device__ __forceinline__ void warp_range(unsigned long long &lo, unsigned long
 // Cuts the keys [start, start + len) of the buffer that `level` reads: a histogram over bins, bins
 // gathered into segments of at most kListCap entries by the kSegTarget-entry stretch of the keys
 // their first entry falls into, and the keys scattered by bin into the other buffer.  A segment
-// above kListCap is a single bin.  The bins are
-// linear in the keys' bits, which for floats spaces them like the logarithm: with kExact between
-// the smallest and the largest key, which takes one more pass over them, else 128 an octave of
-// range from 2^-12 on (the ends take what lies beyond).
+// above kListCap is a single bin.  The bins are linear in the keys' bits, which for floats spaces
+// them like the logarithm: with kExact between the smallest and the largest key, which takes one
+// more pass over them, else 128 an octave of range from 2^-12 on (the ends take what lies beyond).
+// Bound by the latency of those passes and of the barriers between them, one CTA an SM.
 template <bool kExact, typename Group>
 __device__ __forceinline__ SegmentRun cut(const BinArgs &A, uint32_t start, uint32_t len,
                                           uint32_t tile, int level, SplitShared &sh, const Group &g)
@@ -645,8 +645,9 @@ __device__ __noinline__ void recut(const BinArgs &A, SegmentRun run, uint32_t ti
 // Cuts one list until no segment is above kListCap.  The first cut of a list that one CTA cuts
 // takes the fixed bins, where few lists of that length have more than kListCap entries in a bin;
 // what is oversized after it (a wall at one distance, a dense map) is cut again, exactly.  An
-// oversized segment is one bin, and a bin of an exact cut spans at most 2^-11 of the keys' range: keys have
-// 63 bits at most and are unique, so that the bins of the fifth exact cut span no more than 8 keys.
+// oversized segment is one bin, and a bin of an exact cut spans at most 2^-11 of the keys' range:
+// keys have 63 bits at most and are unique, so that the bins of the fifth exact cut span no more
+// than 8 keys.
 // A cluster cuts exactly from the start, goes on as one while more than half of the list stays in
 // one segment, and shares the rest out to its CTAs.
 // What the exact pass costs a list of 5,000 or 20,000 entries on one CTA: 4 us on 4.5 and 18.  What
@@ -1046,9 +1047,9 @@ bool chained(const BinArgs &a) { return chained_size(a.n * a.n_views); }
 }  // namespace
 
 // k_lists' shared memory is above the 48 KB static limit.  Its three CTAs need 159 of an SM's 228
-// KB; what is left is L1, which the list sort lives on.  Left to the driver, a build whose registers
-// allow a fourth CTA gets the shared memory for one and 20 KB of L1: 12 x 500 k primitives 0.096 ->
-// 0.130 ms.
+// KB; what is left is L1, which the list sort lives on.  Left to the driver, a build whose
+// registers allow a fourth CTA gets the shared memory for one and 20 KB of L1: 12 x 500 k
+// primitives 0.096 -> 0.130 ms.
 cudaError_t prepare_lists()
 {
     constexpr int kShared = kListCtas * (sizeof(ListShared) + 1024);   // 1 KB a CTA is the system's
