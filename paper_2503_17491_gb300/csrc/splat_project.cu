@@ -20,7 +20,8 @@
 // pairs along a long street, 3-4 % in a street or block) are queued per warp and boxed by the
 // contract 32 at a time.  Projection of 12 x 500 k pairs: 0.214 -> 0.19 ms, in a refinement with
 // the gradient accumulators zeroed on the way; of 8 x 1 M pairs along a 600 m street: 0.278
-// -> 0.188 ms.  Issue bound (74 % of the slots, 640 instructions per warp and view).
+// -> 0.188 ms.  Bound by instruction issue: in that refinement 67 % of the slots, 700 instructions
+// per warp and view.
 //
 // A pair leaves its pixel rectangle with the normal-flip bit (8 bytes, zero when it touches no
 // tile).  A pair that touches a tile also appends its tile rectangle and range key (12 bytes) to
