@@ -906,9 +906,9 @@ __device__ __forceinline__ uint32_t get_bin(const uint32_t *bins, uint32_t b)
 // then ranked against the other keys of its bin -- one or two on lists whose ranges spread.  A
 // list with a bin above kMaxInBin (a wall behind a near object) is merge sorted.  The keys are
 // read three times rather than held: they stay in L1, and short loops keep the code in the
-// instruction cache.  24 warps with 52 KB a CTA leave 72 KB of L1, which bounds the misses in
-// flight: with the rectangles gathered into shared memory as well (68 KB a CTA) the stage took
-// 0.178 ms instead of 0.121 on 5.3 M entries, with four CTAs per SM 0.157.
+// instruction cache.  24 warps with 52 KB a CTA leave a third of an SM's memory to L1, which bounds
+// the misses in flight: with the rectangles gathered into shared memory as well (68 KB a CTA) the
+// stage took 0.178 ms instead of 0.121 on 5.3 M entries, with four CTAs per SM 0.157.
 template <int G>
 __device__ __forceinline__ void sort_list(const BinArgs &A, const uint64_t *src, uint32_t start,
                                           int n, uint32_t tile, uint64_t *key,
@@ -1049,7 +1049,7 @@ bool chained(const BinArgs &a) { return chained_size(a.n * a.n_views); }
 
 // k_lists' shared memory is above the 48 KB static limit.  Its three CTAs need 159 of an SM's 228
 // KB; what is left is L1, which the list sort lives on.  Left to the driver, a build whose
-// registers allow a fourth CTA gets the shared memory for one and 20 KB of L1: 12 x 500 k
+// registers allow a fourth CTA gets the shared memory for one at the cost of the L1: 12 x 500 k
 // primitives 0.096 -> 0.130 ms.
 cudaError_t prepare_lists()
 {
